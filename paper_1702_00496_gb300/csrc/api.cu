@@ -192,6 +192,17 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
   for (int k = 0; k < cfg->L; ++k)
     for (int m = 0; m < T; ++m)
       p.w[k][m] = cfg->scheme == AT_AT ? c2.w[k][m] : (m == 0 ? 1.0 : 0.0);
+  if (p.dim == 1) {
+    double t[2 * AT_MAX_H + 1];
+    const int hi = atfd::fx_reach(h, p.ts > 1);
+    for (int j = -hi; j <= hi; ++j) t[j + hi] = j == 0 ? p.s0 : p.s[0][j + h];
+    atfd::fx_prepare(t, 2 * hi + 1, &p.fs);
+    atfd::fx_prepare(p.b1, 2 * h + 1, &p.fb1);
+    atfd::fx_prepare(p.b2, 2 * h + 1, &p.fb2);
+    const uint32_t gS = (uint32_t)((p.use_pe[0] ? p.S[0] : p.n[0]) >> 2);
+    p.div_g = atfd::fast_div(gS);
+    p.div_in = atfd::fast_div(gS > 2 ? gS - 2 : 1);
+  }
   return AT_OK;
 }
 

@@ -33,8 +33,11 @@ using namespace atfd;
 // Grouped kernel: a thread updates four consecutive x points per iteration (grid-stride); every thread
 // also draws the delays of one slice of the PE sides for step n+1 into the other half of the double-buffered
 // delay array, so the next launch finds them ready.
+//
+// 1D groups are summed in fixed point (stencil.cuh); two blocks of 512 per SM (64 registers) hide the latency of their
+// integer chains: at N = 2^24 the AB2 step of order 4 takes 105 us against 133 us with the 88 registers it would use.
 template <int DIM, int H, int AB, int KIND>
-__global__ void __launch_bounds__(512) forward_group_kernel(const StepParams p, const int64_t n_off,
+__global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   const int64_t n = n_off + (n_base ? *n_base : 0);
   const double *__restrict__ un = p.ring + (n % p.R) * p.ntot;
@@ -150,13 +153,80 @@ __global__ void __launch_bounds__(128) forward_zones_kernel(const StepParams p, 
   }
 }
 
-// The last step m = n + K - 1 of a block: inner groups U^{n+K} = ck * U^n, edge groups the step from U^m.
-template <int H, int K>
-__global__ void __launch_bounds__(512) forward_block_kernel(const StepParams p, const int64_t n_off,
+// One inner cell of a block as an FP64 chain: U^{n+K}_x = sum ck_j U^n_{x+j}, the centre first, then j ascending.
+template <int TK>
+__device__ __noinline__ double block_cell(const StepParams &p, const double *__restrict__ u0, int x) {
+  const int nx = p.n[0];
+  double acc = fma(p.ck[TK], LdgNC::ld(u0 + x), p.zero);
+  for (int j = -TK; j <= TK; ++j)
+    if (j != 0) acc = fma(p.ck[j + TK], LdgNC::ld(u0 + wrap_coord(x + j, nx)), acc);
+  return acc;
+}
+
+// Cells per lane and warp tile of the inner cells: a tile is 32 C consecutive cells of one PE.
+template <int TK, int C>
+struct BlockTile {
+  static constexpr int CELLS = 32 * C, WIN = CELLS + 2 * TK;
+  static constexpr int SLOTS = WIN + WIN / C + 1;  // one pad slot per C cells: lanes C cells apart take all banks
+  static constexpr int BYTES = SLOTS * 8;
+};
+
+// The C outputs of a lane from its window in shared memory, four at a time (independent chains for the pipe's latency).
+// F32: the low parts are there as FP32 and the cross terms are summed in FP32.
+template <int TK, int C, bool F32, int NT>
+__device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, int lane, int ex, double r[C]) {
+  int2 w[C + 2 * TK];
+  float h[C + 2 * TK];
+#pragma unroll
+  for (int i = 0; i < C + 2 * TK; ++i) {
+    w[i] = sm[lane * (C + 1) + i + i / C];
+    if (F32) h[i] = __int2float_rn(w[i].x);
+  }
+#pragma unroll
+  for (int q0 = 0; q0 < C; q0 += 4) {
+    int64_t A[4], B[4], D[4];
+    float c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      A[q] = 0; B[q] = kFxB0; D[q] = kFxC0;
+      c[q] = 0.0f;
+    }
+#pragma unroll
+    for (int j = 0; j <= 2 * TK; ++j) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = q0 + q + j;
+        A[q] = fx_mad(t.w1[j], w[i].x, A[q]);
+        if (F32) {
+          c[q] = fmaf(t.f1[j], __int_as_float(w[i].y), c[q]);
+          c[q] = fmaf(t.f0[j], h[i], c[q]);
+        } else {
+          B[q] = fx_mad(t.w1[j], w[i].y, B[q]);
+          D[q] = fx_mad(t.w0[j], w[i].x, D[q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) A[q] = F32 ? A[q] + (int64_t)__float2int_rn(c[q]) * 8 : fx_join(A[q], B[q], D[q]);
+    fx_results<4>(A, ex, r + q0);
+  }
+}
+
+// The last step m = n + K - 1 of a block: inner cells U^{n+K} = ck * U^n, edge groups the step from U^m.
+//
+// The inner cells are a contraction of 2 h K + 1 constant taps, which the FP64 pipe bounded (17 DFMA per cell at order
+// 4 and K = 4).  They are summed in block fixed point (fixed.cuh): three integer multiply-adds per tap.  A warp takes a
+// tile of 32 C cells: it reads the tile and its halo once (coalesced, all loads in flight together), finds their
+// largest exponent, converts every value once and lays the two 32-bit parts in shared memory; each lane then reads the
+// window of its C cells once, sums its C outputs from registers, and the results go back through shared memory to
+// coalesced stores.  What bounds it is the issue of the 32-bit integer pipe: 3 (2 h K + 1) multiply-adds per cell
+// beside about 30 logic and shift instructions (11 per converted value, 19 per rounded result).
+template <int H, int K, int C>
+__global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   constexpr int TK = H * K;                  // half-width of the composed stencil
-  constexpr int WK = (TK + 1) / 2 * 2;       // its x window, rounded to even cells (16-byte loads)
-  constexpr int NW = 4 + 2 * WK;
+  using Tile = BlockTile<TK, C>;
+  extern __shared__ int2 block_smem[];
   const int64_t m = n_off + (n_base ? *n_base : 0), n0 = m - (K - 1);
   const double *__restrict__ u0 = p.ring + (n0 % p.R) * p.ntot;
   const double *__restrict__ um = p.ring + (m % p.R) * p.ntot;
@@ -164,39 +234,90 @@ __global__ void __launch_bounds__(512) forward_block_kernel(const StepParams p, 
   const uint8_t *keff = p.keff + (m & 1) * p.nb;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
   const int nx = p.n[0];
-  const int64_t groups = nx >> 2;
-  const int64_t gS = p.use_pe[0] ? p.S[0] >> 2 : groups;
-  const int64_t n_inner = (groups / gS) * (gS - 2 * p.fe);
-  // Inner groups first: they read U^n only, so they may run while the zone launch (this block's steps n .. m-1 near
+  const int lane = threadIdx.x & 31;
+  int2 *sm = block_smem + (threadIdx.x >> 5) * Tile::SLOTS;
+  const int S = p.use_pe[0] ? p.S[0] : nx, inner = S - 8 * p.fe;
+  const int per_pe = (inner + Tile::CELLS - 1) / Tile::CELLS;
+  const int tiles = (nx / S) * per_pe;
+  // Inner cells first: they read U^n only, so they may run while the zone launch (this block's steps n .. m-1 near
   // the PE boundaries, launched with a programmatic dependency) still does.  Then wait for it: the edge groups read
   // its U^m, and the delays of step m+1 go into the buffer slot its first step reads.
-  for (int64_t k = tid; k < n_inner; k += nthreads) {
-    const int x0 = (int)(group_1d_order_e(p, k, p.fe) << 2);
-    double v[NW];
-    if (x0 >= WK && x0 + 4 + WK <= nx) {
+  for (int t = (int)(tid >> 5); t < tiles; t += (int)(nthreads >> 5)) {
+    const int pe = t / per_pe, off = (t - pe * per_pe) * Tile::CELLS;
+    const int x0 = pe * S + 4 * p.fe + off, len = min(Tile::CELLS, inner - off);
+    // A PE's last tile reads on past its inner cells: U^n is written nowhere meanwhile, and only the scale sees them.
+    double v[C + 1];  // 2 TK <= 24 < 32: the halo takes at most one more value per lane
+    const double *src = u0 + (x0 - TK + lane);
+    if (x0 >= TK && x0 - TK + Tile::WIN <= nx) {
 #pragma unroll
-      for (int t = 0; t < NW; t += 2) {
-        const double2 a = LdgNC::ld2(u0 + x0 - WK + t);
-        v[t] = a.x; v[t + 1] = a.y;
+      for (int q = 0; q < C; ++q) v[q] = LdgNC::ld(src + 32 * q);
+      v[C] = lane < 2 * TK ? LdgNC::ld(src + 32 * C) : v[0];
+    } else {  // the window wraps around the domain, or around a small one more than once
+#pragma unroll
+      for (int q = 0; q <= C; ++q) {
+        int i = x0 - TK + min(lane + 32 * q, Tile::WIN - 1);
+        i = i < 0 ? i + nx : i;
+        v[q] = LdgNC::ld(u0 + i % nx);
       }
+    }
+    int hi = 0, lo = 0x7fffffff;
+#pragma unroll
+    for (int q = 0; q <= C; ++q) {
+      hi = max(hi, fx_mag(v[q]));
+      lo = min(lo, fx_mag(v[q]));
+    }
+    const int E = __reduce_max_sync(0xffffffffu, hi) >> 20;
+    const bool near = (__reduce_min_sync(0xffffffffu, lo) >> 20) >= E - kFxNear;
+    bool fixed = p.fck.ok && fx_usable(E);  // the same for the whole warp
+    double r[C];
+    __syncwarp();
+    if (fixed) {
+#pragma unroll
+      for (int q = 0; q <= C; ++q) {
+        const int i = lane + 32 * q;
+        const Fx f = fx_split(fx_from(v[q], E));
+        const int low = near ? __float_as_int(__int2float_rn(f.lo)) : f.lo;
+        if (q < C || lane < 2 * TK) sm[i + i / C] = make_int2(f.hi, low);
+      }
+      __syncwarp();
+      if (near) {
+        block_sums<TK, C, true>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
+      } else {
+        // every run of 8 cells must hold a value within kFxGuard bits of the tile's largest one
+        constexpr int G = C < 8 ? C : 8;
+#pragma unroll
+        for (int g = 0; g < C; g += G) {
+          const int a = C * lane + TK + g + G / 8, b = C * lane + TK + g + G - 1 - G / 8;
+          const int ha = sm[a + a / C].x, hb = sm[b + b / C].x;
+          if ((((ha ^ (ha >> 31)) | (hb ^ (hb >> 31))) >> (29 - kFxGuard)) == 0) fixed = false;
+        }
+        if (fixed) block_sums<TK, C, false>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
+      }
+    }
+    if (!fixed) {
+#pragma unroll
+      for (int q = 0; q < C; ++q)
+        if (C * lane + q < len) r[q] = block_cell<TK>(p, u0, x0 + C * lane + q);
+    }
+    __syncwarp();
+    double *ro = reinterpret_cast<double *>(sm) + lane * (C + 1);
+#pragma unroll
+    for (int q = 0; q < C; ++q) ro[q] = r[q];
+    __syncwarp();
+    ro = reinterpret_cast<double *>(sm);
+    double *dst = out + x0 + lane;
+    if (len == Tile::CELLS) {
+#pragma unroll
+      for (int q = 0; q < C; ++q) dst[32 * q] = ro[lane + 32 * q + (lane + 32 * q) / C];
     } else {
 #pragma unroll
-      for (int t = 0; t < NW; ++t) v[t] = LdgNC::ld(u0 + wrap_coord(x0 - WK + t, nx));
+      for (int q = 0; q < C; ++q)
+        if (lane + 32 * q < len) dst[32 * q] = ro[lane + 32 * q + (lane + 32 * q) / C];
     }
-    double r[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      double acc = fma(p.ck[TK], v[q + WK], p.zero);
-#pragma unroll
-      for (int j = -TK; j <= TK; ++j)
-        if (j != 0) acc = fma(p.ck[j + TK], v[q + WK + j], acc);
-      r[q] = acc;
-    }
-    reinterpret_cast<double2 *>(out + x0)[0] = make_double2(r[0], r[1]);
-    reinterpret_cast<double2 *>(out + x0)[1] = make_double2(r[2], r[3]);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   draw_sides(p, m + 1, tid, nthreads, p.keff + ((m + 1) & 1) * p.nb);
+  const int64_t groups = nx >> 2, n_inner = (int64_t)(nx / S) * (inner >> 2);
   for (int64_t k = n_inner + tid; k < groups; k += nthreads)
     group_step<1, H, LdgNC, false, 0>(p, keff, um, out, m, (int)(group_1d_order_e(p, k, p.fe) << 2), 0, 0);
 }
@@ -225,10 +346,12 @@ __global__ void __launch_bounds__(512) forward_point_kernel(const StepParams p, 
   for (int64_t i = tid; i < p.ntot; i += nthreads) {
     int c[3];
     point_coords(p, DIM, i, c);
+    AbLevels<1> old;
+    if (AB) ab_fetch<1>(p, n, i, old);
     if (DIM == 1 && KIND == 1) {
       double r[1] = {point_update_burgers<H, LdgNC>(p, keff, un, n, i)};
       const double u[1] = {un[i]};
-      if (AB) ab_combine<1>(p, n, i, u, r);
+      if (AB) ab_combine<1>(p, n, i, u, r, old);
       else r[0] = u[0] + r[0];
       out[i] = r[0];
       continue;
@@ -237,7 +360,7 @@ __global__ void __launch_bounds__(512) forward_point_kernel(const StepParams p, 
                                          : point_update<DIM, H, LdgNC>(p, keff, un, n, i, c)};
     if (AB) {
       const double u[1] = {un[i]};
-      ab_combine<1>(p, n, i, u, r);
+      ab_combine<1>(p, n, i, u, r, old);
     }
     out[i] = r[0];
   }
@@ -359,21 +482,45 @@ cudaError_t launch_forward_step(const StepParams &p, int64_t n, const int64_t *n
 
 namespace {
 
-template <int H, int K>
-void launch_block_typed(const StepParams &p, int blocks, int zblocks, int threads, int64_t n_off,
+template <int H, int K, int C>
+void launch_block_tiles(const StepParams &p, int max_blocks, int64_t tiles, int threads, int64_t n_off,
                         const int64_t *n_base, cudaStream_t st) {
-  forward_zones_kernel<H, K><<<zblocks, 128, 0, st>>>(p, n_off, n_base);
+  const int warps = threads / 32, bytes = warps * BlockTile<H * K, C>::BYTES;
+  auto kernel = forward_block_kernel<H, K, C>;
+  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const int64_t b = (tiles + warps - 1) / warps;
   // the block launch depends programmatically on the zone launch (it waits for it inside, before its edge groups)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.gridDim = dim3((unsigned)(b < max_blocks ? b : max_blocks));
   cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)bytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, forward_block_kernel<H, K>, p, n_off + K - 1, n_base);
+  cudaLaunchKernelEx(&cfg, kernel, p, n_off + K - 1, n_base);
+}
+
+// Tiles of 32 C cells over the inner cells of every PE.
+int64_t block_tiles(const StepParams &p, int C) {
+  const int64_t S = p.use_pe[0] ? p.S[0] : p.n[0], inner = S - 8 * p.fe;
+  return p.n[0] / S * ((inner + 32 * C - 1) / (32 * C));
+}
+
+template <int H, int K>
+void launch_block_typed(const StepParams &p, int max_blocks, int zblocks, int threads, int64_t n_off,
+                        const int64_t *n_base, cudaStream_t st) {
+  forward_zones_kernel<H, K><<<zblocks, 128, 0, st>>>(p, n_off, n_base);
+  // Cells per lane: 8 convert 9/8 of the values and give a PE's last tile of 256 cells to fill, 4 convert 5/4 of them
+  // and fill tiles of 128; instructions per tile: C + 1 conversions and C outputs.
+  const int64_t t8 = block_tiles(p, 8), t4 = block_tiles(p, 4);
+  const int taps = 3 * (2 * H * K + 1) + 22;
+  if (t8 >= 152 * 16 && t8 * (9 * 11 + 8 * taps) <= t4 * (5 * 11 + 4 * (taps + 8)))
+    launch_block_tiles<H, K, 8>(p, max_blocks, t8, threads, n_off, n_base, st);
+  else
+    launch_block_tiles<H, K, 4>(p, max_blocks, t4, threads, n_off, n_base, st);
 }
 
 template <int H>
@@ -387,16 +534,14 @@ void launch_block_h(const StepParams &p, int blocks, int zblocks, int threads, i
 }  // namespace
 
 cudaError_t launch_forward_block(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st) {
-  const int threads = p.threads > 0 ? p.threads : 256;
+  const int threads = p.threads == 128 ? 128 : 256;  // the block kernel's 80 registers give three blocks of 256 per SM
   const int max_blocks = sm_count() * (p.blocks_per_sm > 0 ? p.blocks_per_sm : 32);
-  const int64_t b = (p.ntot / 4 + threads - 1) / threads;
-  const int blocks = (int)(b < max_blocks ? b : max_blocks);
   const int64_t nwarps = p.use_pe[0] ? p.pe[0] : 1;  // zone launch: one warp per PE boundary, four per block
   const int64_t zb = (nwarps + 3) / 4;
   const int zblocks = (int)(zb < max_blocks ? zb : max_blocks);
-  if (p.h == 1) launch_block_h<1>(p, blocks, zblocks, threads, n_off, n_base, st);
-  else if (p.h == 2) launch_block_h<2>(p, blocks, zblocks, threads, n_off, n_base, st);
-  else launch_block_h<3>(p, blocks, zblocks, threads, n_off, n_base, st);
+  if (p.h == 1) launch_block_h<1>(p, max_blocks, zblocks, threads, n_off, n_base, st);
+  else if (p.h == 2) launch_block_h<2>(p, max_blocks, zblocks, threads, n_off, n_base, st);
+  else launch_block_h<3>(p, max_blocks, zblocks, threads, n_off, n_base, st);
   return cudaGetLastError();
 }
 
@@ -439,6 +584,7 @@ void fuse_setup(StepParams *p, int k) {
   p->fe = 0;
   std::memset(p->zr, 0, sizeof(p->zr));
   std::memset(p->ck, 0, sizeof(p->ck));
+  std::memset(&p->fck, 0, sizeof(p->fck));
   if (k <= 1) return;
   const int h = p->h;
   fuse_radii(h, k, &p->fe, p->zr);
@@ -456,6 +602,7 @@ void fuse_setup(StepParams *p, int k) {
     for (int i = 0; i <= 2 * w; ++i) c[i] = t[i];
   }
   for (int i = 0; i <= 2 * w; ++i) p->ck[i] = c[i];
+  fx_prepare(p->ck, 2 * w + 1, &p->fck);
 }
 
 cudaError_t launch_sync_rhs(const StepParams &p, const double *u, double *out, cudaStream_t st) {

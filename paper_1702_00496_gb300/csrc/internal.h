@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/at.h"
+#include "fixed.cuh"
 
 #define AT_MAX_L 8
 #define AT_MAX_T 4
@@ -18,6 +19,35 @@
 #define AT_MAX_FUSE 4
 
 void at_internal_set_error(const char *msg);
+
+namespace atfd {
+
+// q = n / d for 0 <= n < 2^30 and 1 <= d < 2^30 without a division: n m >> (32 + s) with m = ceil(2^(32 + s) / d), s =
+// ceil(log2 d) - 2 at least 0, is exact as m's rounding error times n stays under 2^(32 + s) / d.
+struct FastDiv {
+  uint32_t m, s;
+};
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f = {0u, 0u};
+  if (d < 1) d = 1;
+  while (((uint64_t)4 << f.s) < d) ++f.s;
+  const uint64_t m = (((uint64_t)1 << (32 + f.s)) + d - 1) / d;
+  f.m = m > 0xffffffffull ? 0u : (uint32_t)m;  // d = 1: 2^32 does not fit; m = 0 stands for it
+  return f;
+}
+#if defined(__CUDACC__)
+__host__ __device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv &f) {
+  return f.m == 0 ? n : (uint32_t)(((uint64_t)n * f.m) >> 32) >> f.s;
+}
+#endif
+
+// Half-width of the 1D Euler step's taps that are summed in fixed point.  The outermost pair of a stencil of five or
+// more taps stays with the FP64 pipe, which is idle otherwise: two DFMA per point take 32 SM clocks beside about 40 of
+// the integer pipes, and the window to convert gets two values shorter.  Adams-Bashforth steps sum every tap in fixed
+// point: their combination keeps the FP64 pipe as busy.
+constexpr int fx_reach(int h, bool ab) { return h >= 2 && !ab ? h - 1 : h; }
+
+}  // namespace atfd
 
 // Everything one forward step needs, passed to the kernel by value.
 struct StepParams {
@@ -82,6 +112,13 @@ struct StepParams {
   // pre-history, ts-1 from a caller's field); from it on the weights are beta[ts-1] at every step, and AB2 steps
   // take the combination's steady form.
   int64_t ab_steady;
+  // The block's composed taps ck in fixed point (fixed.cuh), index j + h K; ok = 0: the FP64 chain everywhere.
+  atfd::FxTaps<2 * AT_MAX_H * AT_MAX_FUSE + 1> fck;
+  // 1D step in fixed point: the merged taps of half-width fx_h (index j + fx_h; fx_reach says why not all of them) and
+  // Burgers' first and second derivative.
+  atfd::FxTaps<2 * AT_MAX_H + 1> fs, fb1, fb2;
+  // Division by the groups of a PE (S/4) and by its groups without the first and the last (1D).
+  atfd::FastDiv div_g, div_in;
 };
 
 // The modes of one axis at one time t, prepared on the host for the recurrences over k: sorted by wavenumber,

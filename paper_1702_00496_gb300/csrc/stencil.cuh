@@ -73,10 +73,10 @@ __device__ __forceinline__ double halo_value(const StepParams &p, int64_t cell, 
 __device__ __forceinline__ int64_t group_1d_order(const StepParams &p, int64_t k) {
   const uint32_t gS = (uint32_t)(p.use_pe[0] ? p.S[0] >> 2 : p.n[0] >> 2);
   if (gS < 3) return k;
-  const uint32_t inner = gS - 2, npe = (uint32_t)(p.n[0] >> 2) / gS, uk = (uint32_t)k;
+  const uint32_t inner = gS - 2, npe = p.use_pe[0] ? (uint32_t)p.pe[0] : 1u, uk = (uint32_t)k;
   const uint32_t n_int = npe * inner;
   if (uk < n_int) {
-    const uint32_t pe = uk / inner;
+    const uint32_t pe = fdiv(uk, p.div_in);
     return (int64_t)pe * gS + 1 + (uk - pe * inner);
   }
   const uint32_t kk = uk - n_int;
@@ -226,46 +226,177 @@ __device__ __forceinline__ void ab_store(double *dst, const double a[NP]) {
 // Adams-Bashforth combination of NP consecutive points starting at i (16-byte aligned for NP = 4): r holds
 // dt f^n and becomes U^{n+1} = U^n + sum_{m<l} beta_m dt f^{n-m} (l = levels stored so far, at most ts), formed
 // as a chain of l FMAs onto U^n; dt f^n takes the slot of the oldest right-hand side, which only this thread
-// reads, after the read.
+// reads.  ab_fetch loads the stored levels before the stencil's sum, ab_combine uses them and stores dt f^n after it:
+// a store to an address whose load is still in flight holds the warp (Case 4 at N = 2^24 took 674 us per step with
+// the load between the sum and the store, 67 cycles of load wait per instruction).
 //
 // STEADY = true: the host launches this form only for steps whose ts levels are all stored (l = ts); with ts = 2
-// the weights beta[1] are then fixed and come straight from the kernel parameters.  The operations are the same;
-// this takes Case 4 (AB2, N = 2^24) on GB300 from 248 to 214 us per step.  (AB3 in this form ran at 492 against
-// 307 us, so other ts take the general code.)
+// the weights beta[1] are then fixed and come straight from the kernel parameters.  The operations are the same.
+template <int NP>
+struct AbLevels {
+  double a1[NP], a2[NP];
+  int l;
+};
+
 template <int NP, bool STEADY = false>
-__device__ __forceinline__ void ab_combine(const StepParams &p, int64_t n, int64_t i, const double u[NP],
-                                           double r[NP]) {
+__device__ __forceinline__ void ab_fetch(const StepParams &p, int64_t n, int64_t i, AbLevels<NP> &o) {
   if (STEADY && p.ts == 2) {
-    double *f = p.frhs + i;  // dt f^{n-1}, then dt f^n
-    double a1[NP];
-    ab_load<NP>(f, a1);
-    ab_store<NP>(f, r);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = fma(p.beta[1][0], r[q], u[q]);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = fma(p.beta[1][1], a1[q], r[q]);
+    o.l = 2;
+    ab_load<NP>(p.frhs + i, o.a1);
     return;
   }
   const int64_t stored = n - *p.ab_first + 1;
-  const int l = stored < p.ts ? (int)stored : p.ts;
-  const double *beta = p.beta[l - 1];
+  o.l = stored < p.ts ? (int)stored : p.ts;
   const bool two = p.ts == 3;  // two stored slots, else one
-  double *f_now = p.frhs + (two ? (n & 1) : 0) * p.ntot + i;          // dt f^{n-2} (AB3) or dt f^{n-1} (AB2)
-  const double *f_1 = p.frhs + (two ? ((n - 1) & 1) : 0) * p.ntot + i;  // dt f^{n-1}
-  double a1[NP], a2[NP];
-  if (l > 1) ab_load<NP>(f_1, a1);
-  if (l > 2) ab_load<NP>(f_now, a2);
-  ab_store<NP>(f_now, r);
+  if (o.l > 1) ab_load<NP>(p.frhs + (two ? ((n - 1) & 1) : 0) * p.ntot + i, o.a1);  // dt f^{n-1}
+  if (o.l > 2) ab_load<NP>(p.frhs + (n & 1) * p.ntot + i, o.a2);                    // dt f^{n-2}
+}
+
+template <int NP, bool STEADY = false>
+__device__ __forceinline__ void ab_combine(const StepParams &p, int64_t n, int64_t i, const double u[NP],
+                                           double r[NP], const AbLevels<NP> &o) {
+  double f[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) f[q] = r[q];
+  if (STEADY && p.ts == 2) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) r[q] = fma(p.beta[1][0], r[q], u[q]);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) r[q] = fma(p.beta[1][1], o.a1[q], r[q]);
+    ab_store<NP>(p.frhs + i, f);
+    return;
+  }
+  const double *beta = p.beta[o.l - 1];
 #pragma unroll
   for (int q = 0; q < NP; ++q) r[q] = fma(beta[0], r[q], u[q]);
-  if (l > 1) {
+  if (o.l > 1) {
 #pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = fma(beta[1], a1[q], r[q]);
+    for (int q = 0; q < NP; ++q) r[q] = fma(beta[1], o.a1[q], r[q]);
   }
-  if (l > 2) {
+  if (o.l > 2) {
 #pragma unroll
-    for (int q = 0; q < NP; ++q) r[q] = fma(beta[2], a2[q], r[q]);
+    for (int q = 0; q < NP; ++q) r[q] = fma(beta[2], o.a2[q], r[q]);
   }
+  ab_store<NP>(p.frhs + (p.ts == 3 ? (n & 1) : 0) * p.ntot + i, f);
+}
+
+// ---------------------------------------------------------------- 1D groups in fixed point
+//
+// The four points of a 1D group from its window of 4 + 2 W values, summed in block fixed point (fixed.cuh) with the
+// window's own scale, so the bits depend on the group alone.  Three integer multiply-adds per tap and point, beside the
+// window's conversions and four roundings per group, where a DFMA holds the FP64 pipe for 16 SM clocks per warp; what
+// the FP64 pipe can do meanwhile stays with it: the outermost pair of taps of an Euler step (fx_reach), the
+// combination of an Adams-Bashforth step.
+//
+// A group is taken only when both halves of it hold a value within kFxGuard bits of the window's largest; the others
+// (and windows that hold infinities or NaN, or lie at the ends of the exponent range) go through the chain.
+
+// x window of a 1D group: cells x0-W .. x0+3+W, buffer points replaced by the halo values of step n.
+template <int H, class LD, bool OWN_SIDES = false>
+__device__ __forceinline__ void window_1d(const StepParams &p, const uint8_t *__restrict__ keff,
+                                          const double *__restrict__ un, int64_t n, int x0, double v[XWin<H>::N]) {
+  constexpr int W = XWin<H>::W, NW = XWin<H>::N;
+  const int nx = p.n[0];
+  const int pidx[3] = {p.use_pe[0] ? (int)fdiv((uint32_t)x0 >> 2, p.div_g) : 0, 0, 0};  // groups lie inside a PE
+  const int pos0 = x0 - pidx[0] * p.S[0];
+  if (x0 >= W && x0 + 4 + W <= nx) {
+#pragma unroll
+    for (int t = 0; t < NW; t += 2) {
+      const double2 a = LD::ld2(un + x0 - W + t);
+      v[t] = a.x; v[t + 1] = a.y;
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < NW; ++t) v[t] = LD::ld(un + wrap_coord(x0 - W + t, nx));
+  }
+  if (p.use_pe[0] && (pos0 < H || pos0 + 3 >= p.S[0] - H)) {
+    const int sn = (int)(n % p.R);
+    const bool lo = !OWN_SIDES || pos0 < H, hi = !OWN_SIDES || pos0 + 3 >= p.S[0] - H;
+    const int kl = lo ? keff[side_of<1>(p, pidx, 0, 0)] : 0, kr = hi ? keff[side_of<1>(p, pidx, 0, 1)] : 0;
+#pragma unroll
+    for (int t = W - H; t <= W + 3 + H; ++t) {
+      const int rel = pos0 - W + t;
+      const int k = rel < 0 ? kl : (rel >= p.S[0] ? kr : 0);
+      if (k > 0) v[t] = halo_value<LD>(p, wrap_coord(x0 - W + t, nx), sn, k);
+    }
+  }
+}
+
+// Scale of a 1D window (the cells within HI of the group), or -1 when the group goes through the chain.
+template <int W, int HI>
+__device__ __forceinline__ int window_scale(const double v[4 + 2 * W]) {
+  int mag = 0;
+#pragma unroll
+  for (int t = W - HI; t <= W + 3 + HI; ++t) mag = max(mag, fx_mag(v[t]));
+  const int E = mag >> 20;
+  const int near = min(max(fx_mag(v[W]), fx_mag(v[W + 1])), max(fx_mag(v[W + 2]), fx_mag(v[W + 3]))) >> 20;
+  return fx_usable(E) && near >= E - kFxGuard ? E : -1;
+}
+
+// R of the four points for the 2 HI + 1 taps t; x[i] is cell i - HI of the group.
+template <int HI, int NT>
+__device__ __forceinline__ void window_sums(const FxTaps<NT> &t, const Fx x[4 + 2 * HI], int64_t R[4]) {
+  int64_t A[4], B[4], C[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { A[q] = 0; B[q] = kFxB0; C[q] = kFxC0; }
+#pragma unroll
+  for (int j = 0; j <= 2 * HI; ++j) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      A[q] = fx_mad(t.w1[j], x[q + j].hi, A[q]);
+      B[q] = fx_mad(t.w1[j], x[q + j].lo, B[q]);
+      C[q] = fx_mad(t.w0[j], x[q + j].hi, C[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) R[q] = fx_join(A[q], B[q], C[q]);
+}
+
+// -u (dt D1 u) + dt alpha D2 u of Burgers' equation: R1 in units 2^-fb1.sw, R2 in units 2^-fb2.sw (of 2^(E - 1023)).
+// The product X R1 2^-62 has units 2^(2 (E - 1023) + 1 - fb1.sw) and goes down sh places to R2's.
+__device__ __forceinline__ int64_t burgers_sum(const Fx &x, int64_t R1, int64_t R2, int sh) {
+  const Fx r = fx_split(R1);
+  const int64_t A = (int64_t)x.hi * r.hi, B = fx_mad(x.hi, r.lo, (int64_t)x.lo * r.hi);
+  return R2 - fx_shr((A << 2) + (B >> 30), sh);
+}
+
+// The step's sum for the four points of a window, r: U^{n+1} (Euler), dt f^n (Adams-Bashforth, Burgers).  KIND 0:
+// linear, 1: Burgers.  false: the group goes through the chain.
+template <int H, bool AB, int KIND>
+__device__ __forceinline__ bool group_fixed(const StepParams &p, const double v[XWin<H>::N], double r[4]) {
+  constexpr int W = XWin<H>::W, HI = KIND ? H : fx_reach(H, AB);
+  if (KIND ? !(p.fb1.ok && p.fb2.ok) : !p.fs.ok) return false;
+  const int E = window_scale<W, HI>(v);
+  if (E < 0) return false;
+  const int sh = KIND ? p.fb1.sw - p.fb2.sw - (E - 1023) - 1 : 0;
+  if (KIND && (sh < 1 || sh > 200)) return false;
+  Fx x[4 + 2 * HI];
+#pragma unroll
+  for (int t = 0; t < 4 + 2 * HI; ++t) x[t] = fx_split(fx_from(v[W - HI + t], E));
+  int64_t R[4];
+  if (KIND) {
+    int64_t R1[4];
+    window_sums<HI>(p.fb1, x, R1);
+    window_sums<HI>(p.fb2, x, R);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) R[q] = burgers_sum(x[HI + q], R1[q], R[q], sh);
+  } else {
+    window_sums<HI>(p.fs, x, R);
+  }
+  const int ex = E - 1023 - (KIND ? p.fb2.sw : p.fs.sw);
+  if (AB || KIND) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) r[q] = fx_to_any(R[q], ex);
+  } else {
+    fx_results<4>(R, ex, r);
+    if (HI < H) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = fma(p.s[0][0], v[q + W - H], r[q]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = fma(p.s[0][2 * H], v[q + W + H], r[q]);
+    }
+  }
+  return true;
 }
 
 // Update the four points x0..x0+3 of row (y, z) (the forward step; AB: 0 forward Euler, 1 Adams-Bashforth, 2
@@ -275,9 +406,29 @@ __device__ __forceinline__ void group_update(const StepParams &p, const uint8_t 
                                              const double *__restrict__ un, double *__restrict__ out, int64_t n,
                                              int x0, int y, int z) {
   double r[4], uc[4];
-  group_eval<DIM, H, LD, false, OWN_SIDES>(p, keff, un, n, x0, y, z, r, uc);
   const int64_t i0 = (DIM == 3 ? ((int64_t)z * p.n[1] + y) * p.n[0] : 0) + x0;
-  if (AB) ab_combine<4, AB == 2>(p, n, i0, uc, r);
+  AbLevels<4> old;
+  if (AB) ab_fetch<4, AB == 2>(p, n, i0, old);
+  if constexpr (DIM == 1) {
+    constexpr int W = XWin<H>::W;
+    double v[XWin<H>::N];
+    window_1d<H, LD, OWN_SIDES>(p, keff, un, n, x0, v);
+    if (!group_fixed<H, AB != 0, 0>(p, v, r)) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        double acc = fma(p.s0, v[q + W], p.zero);
+#pragma unroll
+        for (int j = -H; j <= H; ++j)
+          if (j != 0) acc = fma(p.s[0][j + H], v[q + W + j], acc);
+        r[q] = acc;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) uc[q] = v[q + W];
+  } else {
+    group_eval<DIM, H, LD, false, OWN_SIDES>(p, keff, un, n, x0, y, z, r, uc);
+  }
+  if (AB) ab_combine<4, AB == 2>(p, n, i0, uc, r, old);
   reinterpret_cast<double2 *>(out + i0)[0] = make_double2(r[0], r[1]);
   reinterpret_cast<double2 *>(out + i0)[1] = make_double2(r[2], r[3]);
 }
@@ -313,39 +464,10 @@ __device__ double point_update(const StepParams &p, const uint8_t *__restrict__ 
 }
 
 // Viscous Burgers' equation (1D, Case 6): dt f = -u_i (dt D1 u) + dt alpha D2 u with the same x window and the
-// same extrapolated halo values as the linear step; r receives dt f^n of the four points x0..x0+3, uc their
-// level-n values.  Each derivative is its own FMA chain; u_i enters through the final FMA.
-template <int H, class LD>
-__device__ __forceinline__ void group_eval_burgers(const StepParams &p, const uint8_t *__restrict__ keff,
-                                                   const double *__restrict__ un, int64_t n, int x0, double r[4],
-                                                   double uc[4]) {
-  constexpr int W = XWin<H>::W, NW = XWin<H>::N;
-  const int nx = p.n[0];
-  const int sn = (int)(n % p.R);
-  const int pidx[3] = {x0 / p.S[0], 0, 0};
-  const int pos0 = x0 - pidx[0] * p.S[0];
-  double v[NW];
-  if (x0 >= W && x0 + 4 + W <= nx) {
-#pragma unroll
-    for (int t = 0; t < NW; t += 2) {
-      const double2 a = LD::ld2(un + x0 - W + t);
-      v[t] = a.x; v[t + 1] = a.y;
-    }
-  } else {
-#pragma unroll
-    for (int t = 0; t < NW; ++t) v[t] = LD::ld(un + wrap_coord(x0 - W + t, nx));
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) uc[q] = v[W + q];
-  if (p.use_pe[0] && (pos0 < H || pos0 + 3 >= p.S[0] - H)) {
-    const int kl = keff[side_of<1>(p, pidx, 0, 0)], kr = keff[side_of<1>(p, pidx, 0, 1)];
-#pragma unroll
-    for (int t = W - H; t <= W + 3 + H; ++t) {
-      const int rel = pos0 - W + t;
-      const int k = rel < 0 ? kl : (rel >= p.S[0] ? kr : 0);
-      if (k > 0) v[t] = halo_value<LD>(p, wrap_coord(x0 - W + t, nx), sn, k);
-    }
-  }
+// same extrapolated halo values as the linear step; r receives dt f^n of the four points of the window.  Each derivative is its own FMA chain; u_i enters through the final FMA.
+template <int H>
+__device__ __forceinline__ void burgers_chain(const StepParams &p, const double v[XWin<H>::N], double r[4]) {
+  constexpr int W = XWin<H>::W;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     double a1 = fma(p.b1[0], v[q + W - H], p.zero);
@@ -458,10 +580,15 @@ __device__ __forceinline__ void group_step(const StepParams &p, const uint8_t *_
                                            const double *__restrict__ un, double *__restrict__ out, int64_t n,
                                            int x0, int y, int z) {
   if (DIM == 1 && KIND == 1) {
-    double r[4], uc[4];
-    group_eval_burgers<H, LD>(p, keff, un, n, x0, r, uc);
+    double v[XWin<H>::N], r[4], uc[4];
+    AbLevels<4> old;
+    if (AB) ab_fetch<4, AB == 2>(p, n, x0, old);
+    window_1d<H, LD>(p, keff, un, n, x0, v);
+    if (!group_fixed<H, AB != 0, 1>(p, v, r)) burgers_chain<H>(p, v, r);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) uc[q] = v[XWin<H>::W + q];
     if (AB) {
-      ab_combine<4, AB == 2>(p, n, x0, uc, r);
+      ab_combine<4, AB == 2>(p, n, x0, uc, r, old);
     } else {
 #pragma unroll
       for (int q = 0; q < 4; ++q) r[q] = uc[q] + r[q];

@@ -1,0 +1,117 @@
+"""The step kernels' fixed-point sums on fields that take each of their routes, against the FP64 oracle.
+
+Smooth fields keep every value of a window near its largest (cross terms in FP32 in the blocks), noise does not (integer
+cross terms), fields that fall by many binades within a few cells, exact zeros, infinities, NaN and values at the ends of
+the exponent range go through the FP64 chain.  Bars: delays bit-exact, elementwise within 1e-12 of the max norm as in
+the other parity tests; where the field falls steeply, elementwise within 256 ulp (5.7e-14) of the largest value in the
+cell's domain of dependence (2 h + 1 roundings per step on each side, under 12 steps); non-finite cells in the same places."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+THREADS = os.cpu_count() or 1
+STEPS = 11
+
+PROBLEMS = [
+    ("block_o2", lambda: W.wl_1d(72 * 24, 24, 2, 3, 0, 601, (1, 2))[0]),
+    ("block_o4_tile_edge", lambda: W.wl_1d(3 * 2072, 3, 4, 4, 0, 602, (1, 2))[0]),
+    ("block_o4_unsplit_small", lambda: W.wl_1d(64, 1, 4, 4, 0, 603, (1, 2))[0]),
+    ("block_o6", lambda: W.wl_1d(2 * 2500, 2, 6, 3, 0, 604, (1, 2), r_alpha=0.02)[0]),
+    ("single_o2", lambda: W.wl_1d(16 * 20, 20, 2, 3, 0, 605, (1, 2))[0]),
+    ("single_o4", lambda: W.wl_1d(64 * 8, 8, 4, 3, 0, 606, (1, 2))[0]),
+    ("single_o6", lambda: W.wl_1d(8 * 32, 32, 6, 3, 0, 607, (1, 2), r_alpha=0.01)[0]),
+    ("ab2_o4", lambda: W.wl_1d(64 * 20, 20, 4, 3, 0, 608, (1, 2), r_alpha=0.02, tsteps=2)[0]),
+    ("ab3_o6", lambda: W.wl_1d(64 * 20, 20, 6, 3, 0, 609, (1, 2), r_alpha=0.01, tsteps=3)[0]),
+    ("burgers_ab2_o4", lambda: dict(W.wl_1d(64 * 20, 20, 4, 3, 0, 610, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
+    ("burgers_euler_o2", lambda: dict(W.wl_1d(64 * 20, 20, 2, 3, 0, 611, (1, 2), c=0.0, r_alpha=0.02)[0], burgers=1)),
+    ("3d_o2", lambda: W.wl_3d([24, 20, 18], [2, 2, 3], 2, 3, 0, 612, c=(0.3, 0.2, 0.1))[0]),
+    ("3d_o4", lambda: W.wl_3d([72, 18, 20], [2, 1, 2], 4, 3, 0, 613, c=(0.3, 0.2, 0.1))[0]),
+    ("3d_o4_ragged", lambda: W.wl_3d([39, 22, 14], [3, 2, 1], 4, 3, 0, 614, c=(0.3, 0.2, 0.1))[0]),
+    ("3d_o6", lambda: W.wl_3d([40, 16, 24], [1, 2, 2], 6, 3, 0, 615, c=(0.3, 0.2, 0.1), dt=0.01 * W.dx_of(40) ** 2 / 0.05)[0]),
+    ("3d_o4_ab2", lambda: W.wl_3d([24, 20, 16], [2, 2, 2], 4, 3, 0, 616, c=(0.3, 0.2, 0.1), tsteps=2)[0]),
+]
+
+
+def _field(spec, kind):
+    rng = np.random.default_rng([spec["seed"], len(kind)])
+    u = oracle.initial(oracle.Config(spec)) + 3.0
+    if kind == "smooth":
+        return u
+    noise = rng.standard_normal(u.shape)
+    if kind == "noise":
+        return noise
+    if kind == "steep":  # falls by more than a binade from cell to cell along x, and is zero in places
+        x = np.arange(u.shape[-1])
+        v = u * np.exp(-((x % 64) - 20.0) ** 2 / 30.0)
+        return np.where(x % 64 > 50, 0.0, v)
+    if kind == "spikes":
+        return np.where(rng.random(u.shape) < 0.02, 1e6 * noise, 1e-6 * noise)
+    if kind == "small":
+        return noise * 1e-250
+    return {"tiny": noise * 1e-290, "large": noise * 1e280}[kind]
+
+
+def _gpu(spec, u0, steps, single=False):
+    from paper_1702_00496_gb300 import Solver, at_set_fusion
+    s = Solver(spec, log_steps=steps)
+    if single:
+        at_set_fusion(s.h, 1)
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.step(steps)
+    s.sync()
+    u, d = s.field().cpu().numpy().copy(), s.delays().cpu().numpy().copy()
+    s.close()
+    return u, d
+
+
+def _local_max(a, reach):
+    """Largest |a| within `reach` cells along every axis (periodic)."""
+    m = np.abs(a)
+    for ax in range(a.ndim):
+        if a.shape[ax] == 1:
+            continue
+        m = np.max([np.roll(m, s, ax) for s in range(-reach, reach + 1)], axis=0)
+    return m
+
+
+@pytest.mark.parametrize("kind", ["smooth", "noise", "steep", "spikes", "small", "tiny", "large"])
+@pytest.mark.parametrize("name,make", PROBLEMS, ids=[p[0] for p in PROBLEMS])
+def test_every_route_matches_the_oracle(name, make, kind):
+    spec = make()
+    u0 = _field(spec, kind)
+    if spec.get("burgers") and kind in ("large", "spikes"):
+        u0 = u0 * 1e-279 if kind == "large" else u0 * 1e-6  # u u_x stays finite and the step stable
+    u, d = _gpu(spec, u0, STEPS)
+    ref, dref, _ = oracle.run(oracle.Config(spec), STEPS, threads=THREADS, u0=u0)
+    assert np.array_equal(d, dref)
+    assert np.abs(u - ref).max() <= 1e-12 * np.abs(ref).max()
+    if kind in ("steep", "spikes") and not spec.get("burgers"):
+        # each cell against the values it can depend on (levels 0 .. STEPS of its neighbourhood: the initial field's)
+        h = spec["order"] // 2
+        local = np.maximum(_local_max(u0, h * STEPS), np.abs(ref))
+        assert (np.abs(u - ref) <= 256 * 2.0 ** -52 * local).all()
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("name,make", [p for p in PROBLEMS if not p[0].startswith(("block", "burgers"))],
+                         ids=[p[0] for p in PROBLEMS if not p[0].startswith(("block", "burgers"))])
+def test_non_finite_values_spread_as_in_the_oracle(name, make, value):
+    spec = make()
+    u0 = _field(spec, "smooth").copy()
+    flat = u0.reshape(-1)
+    flat[[5, flat.size // 2 + 3]] = value
+    u, _ = _gpu(spec, u0, 3)
+    ref, _, _ = oracle.run(oracle.Config(spec), 3, threads=THREADS, u0=u0)
+    # the oracle multiplies each derivative's zero weights too (inf becomes NaN a cell or a step earlier there), so the
+    # cells are compared by being finite or not
+    fine = np.isfinite(ref)
+    assert np.array_equal(fine, np.isfinite(u))
+    assert np.abs(u[fine] - ref[fine]).max() <= 1e-12 * np.abs(ref[fine]).max()
