@@ -461,6 +461,8 @@ int sm_count() {
 }  // namespace
 
 cudaError_t launch_forward_step(const StepParams &p, int64_t n, const int64_t *n_base, cudaStream_t st) {
+  cudaError_t be = cudaSuccess;
+  if (p.dim == 3 && launch_forward_brick(p, n, n_base, st, &be)) return be;
   const int threads = p.threads > 0 ? p.threads : 256;
   const int max_blocks = sm_count() * (p.blocks_per_sm > 0 ? p.blocks_per_sm : 32);
   const bool grouped = grouped_shape(p, p.ring);

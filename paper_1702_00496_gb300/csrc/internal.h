@@ -117,6 +117,8 @@ struct StepParams {
   // 1D step in fixed point: the merged taps of half-width fx_h (index j + fx_h; fx_reach says why not all of them) and
   // Burgers' first and second derivative.
   atfd::FxTaps<2 * AT_MAX_H + 1> fs, fb1, fb2;
+  // 3D step in fixed point: s0, then the merged taps of x, y and z, each in offset order.
+  atfd::FxTaps<6 * AT_MAX_H + 1> f3;
   // Division by the groups of a PE (S/4) and by its groups without the first and the last (1D).
   atfd::FastDiv div_g, div_in;
 };
@@ -156,6 +158,9 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
 cudaError_t launch_forward_step(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
 // The fuse_k steps n .. n+fuse_k-1 of a block (n = n_off + *n_base): zone launches, then the block launch.
 cudaError_t launch_forward_block(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
+// 3D: the step in fixed point over tiles of the PEs (brick.cu); false: the shape or scheme is not one for it, nothing
+// launched.
+bool launch_forward_brick(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st, cudaError_t *e);
 // Largest block length K <= kmax (1: none) that the problem admits, and the block parameters for K (host).
 int fuse_max_k(const StepParams &p, const void *ring, int kmax);
 void fuse_setup(StepParams *p, int k);

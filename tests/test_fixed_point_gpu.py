@@ -37,6 +37,14 @@ PROBLEMS = [
     ("3d_o4_ragged", lambda: W.wl_3d([39, 22, 14], [3, 2, 1], 4, 3, 0, 614, c=(0.3, 0.2, 0.1))[0]),
     ("3d_o6", lambda: W.wl_3d([40, 16, 24], [1, 2, 2], 6, 3, 0, 615, c=(0.3, 0.2, 0.1), dt=0.01 * W.dx_of(40) ** 2 / 0.05)[0]),
     ("3d_o4_ab2", lambda: W.wl_3d([24, 20, 16], [2, 2, 2], 4, 3, 0, 616, c=(0.3, 0.2, 0.1), tsteps=2)[0]),
+    # large enough for the marched tiles: PEs of odd widths (partial tiles and groups, 8-byte stores), an unsplit axis
+    # (the tile wraps around the domain), aligned ones (16-byte stores), chunks of a PE along z
+    ("tiles_o2_ragged", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 2, 3, 0, 617, c=(0.3, 0.2, 0.1))[0]),
+    ("tiles_o4_ragged", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 4, 3, 0, 618, c=(0.3, 0.2, 0.1))[0]),
+    ("tiles_o6_ragged", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 6, 3, 0, 619, c=(0.3, 0.2, 0.1), dt=0.01 * W.dx_of(150) ** 2 / 0.05)[0]),
+    ("tiles_o4_wrap", lambda: W.wl_3d([132, 128, 130], [1, 2, 1], 4, 4, 0, 620, c=(0.3, 0.2, 0.1), scheme=W.ASYNC_STD)[0]),
+    ("tiles_o4_ab2", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 4, 3, 0, 621, c=(0.3, 0.2, 0.1), dt=0.02 * W.dx_of(150) ** 2 / 0.05, tsteps=2)[0]),
+    ("tiles_o4_ab3_aligned", lambda: W.wl_3d([128, 128, 128], [2, 2, 2], 4, 3, 0, 622, c=(0.3, 0.2, 0.1), dt=0.01 * W.dx_of(128) ** 2 / 0.05, tsteps=3)[0]),
 ]
 
 
