@@ -57,13 +57,13 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
   extern __shared__ int2 ring[];
   __shared__ int mx[3], pm[8], later[kBrickLater], n_later;
   const int64_t n = n_off + (n_base ? *n_base : 0);
-  const double *__restrict__ un = p.ring + (n % p.R) * p.ntot;
-  double *__restrict__ out = p.ring + ((n + 1) % p.R) * p.ntot;
+  const double *__restrict__ un = p.ring + slot_of(n, p.R) * p.ntot;
+  double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int tid = threadIdx.x;
   draw_sides(p, n + 1, (int64_t)blockIdx.x * kBrickThreads + tid, (int64_t)gridDim.x * kBrickThreads,
              p.keff + ((n + 1) & 1) * p.nb);
-  const int nx = p.n[0], ny = p.n[1], nz = p.n[2], sn = (int)(n % p.R);
+  const int nx = p.n[0], ny = p.n[1], nz = p.n[2], sn = (int)slot_of(n, p.R);
   const int64_t nxy = (int64_t)nx * ny;
   // tile: x fastest, then y, then chunk, then PE
   int pidx[3], x0, y0, zs, ze;

@@ -88,8 +88,8 @@ __device__ void run_member(const StepParams &p, uint8_t *keff_sh, int64_t nsteps
   atfd::draw_sides(p, 0, threadIdx.x, blockDim.x, keff_sh);
   __syncthreads();
   for (int64_t n = 0; n < nsteps; ++n) {
-    const double *un = p.ring + (n % p.R) * p.ntot;
-    double *out = p.ring + ((n + 1) % p.R) * p.ntot;
+    const double *un = p.ring + atfd::slot_of(n, p.R) * p.ntot;
+    double *out = p.ring + atfd::slot_of(n + 1, p.R) * p.ntot;
     if (n + 1 < nsteps) atfd::draw_sides(p, n + 1, threadIdx.x, blockDim.x, keff_sh + ((n + 1) & 1) * p.nb);
     const uint8_t *keff = keff_sh + (n & 1) * p.nb;
     for (int k = threadIdx.x; k < groups; k += blockDim.x)

@@ -40,8 +40,8 @@ template <int DIM, int H, int AB, int KIND>
 __global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   const int64_t n = n_off + (n_base ? *n_base : 0);
-  const double *__restrict__ un = p.ring + (n % p.R) * p.ntot;
-  double *__restrict__ out = p.ring + ((n + 1) % p.R) * p.ntot;
+  const double *__restrict__ un = p.ring + slot_of(n, p.R) * p.ntot;
+  double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
   draw_sides(p, n + 1, tid, nthreads, p.keff + ((n + 1) & 1) * p.nb);
@@ -61,95 +61,97 @@ __global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(co
   }
 }
 
-// Blocks of K steps (1D forward Euler, central and time-expanded rows).  Away from PE boundaries the step is the
-// same linear stencil at every point and step, so K steps of it are one stencil of half-width h K: its taps ck are
-// the K-fold composition of the merged taps, and a group whose K-step stencil stays inside its PE gets U^{n+K}
-// from U^n with 2 h K + 1 FMAs per point instead of K (2 h + 1).  The cells near a PE boundary, whose buffer points
-// take the delayed halo values of every step, are advanced step by step: the zone launch runs steps n .. n+K-2 of
-// the step kernel's arithmetic on the cells within zr[j] of each boundary (zones that shrink by at least h per
-// step), and the block launch gives the edge groups their last step from U^{n+K-1}.  The zones hold the face
-// strips, so the intermediate levels are in the ring wherever a later step reads a delayed level.  The delays of
-// steps n+1 .. n+K-1 are drawn by the zone launch and the delays of step n+K by the block launch, so the delay log
-// and the effective delays are those of single steps.
+// Blocks of K steps (1D forward Euler, central and time-expanded rows), one launch each.  Away from PE boundaries the
+// step is the same linear stencil at every point and step, so K steps of it are one stencil of half-width h K: its taps
+// ck are the K-fold composition of the merged taps, and a cell whose K-step stencil stays inside its PE gets U^{n+K}
+// from U^n with 2 h K + 1 taps instead of K (2 h + 1).  The cells near a PE boundary, whose buffer points take the
+// delayed halo values of every step, are advanced step by step by one warp per boundary (zone_steps): steps n .. n+K-2
+// on the cells within zr[j] of it (zones that shrink by at least h per step), the last step on the 4 fe cells that no
+// composed stencil reaches.  The zones hold the face strips, so the intermediate levels are in the ring wherever a later
+// step reads a delayed level.  A boundary's warp draws the delays of the two sides that face it for steps n+1 .. n+K,
+// so the delay log and the effective delays are those of single steps.
+//
+// Zones and inner cells of a block do not depend on one another: both read U^n (and a zone the delayed levels of its own
+// boundary's cells, before it overwrites them); a zone writes cells that only it reads; the slots of n+1 .. n+K differ
+// from U^n's (K < R).  As two launches, the second waiting for the first before its edge groups, a block of a 12000-point
+// problem took 17.6 us; as one it takes 6.9.
 
-// Zone launch of the block starting at step n: a warp per PE boundary runs steps n .. n+K-2 on its zone.  A zone
-// lies within S/2 of its boundary, so its cells read across that boundary only: the warp draws the delays of the two
-// sides facing it (the right side of the PE before, the left side of the PE after) for steps n+1 .. n+K-1 itself,
-// into the effective-delay buffer (whose slot for each step and side only this warp uses) and the log, and the
-// steps are separated by __syncwarp, so the loads are coherent ones.  A zone group reads only the delay of the side
-// it reaches across (its own), never one that another warp may be writing.  Without PE boundaries warp 0 only draws.
+// Shared memory of a zone: levels n .. n+K-1 of the region (cells b - RR .. b + RR - 1, RR = zr[0] + h <= 27), the 2 h
+// face cells at the R - 2 levels before n, and their halo values of the current step.
 template <int H, int K>
-__global__ void __launch_bounds__(128) forward_zones_kernel(const StepParams p, const int64_t n_off,
-                                                            const int64_t *n_base) {
-  // the block launch that follows may start now: its inner groups read only U^n, and it waits for this grid before
-  // its edge groups and its delay draws
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Each warp holds its boundary's region -- cells b - RR .. b + RR - 1, RR = zr[0] + h -- at levels n .. n+K-1 in
-  // shared memory: U^n is read once, each step's zone is computed from the level before it there, and only levels
-  // before n (the delayed halo levels at the face strips) are read from the ring.  The arithmetic is the step
-  // kernel's: the centre tap, then the taps in offset order, a buffer point's value extrapolated over the delayed
-  // levels w_m(k) in the order m = 0 .. T-1.
-  constexpr int CELLS = 64;  // 2 RR <= 2 (zr[0] + h) <= 54 for h <= 3, K <= 4
-  __shared__ double lev[4][K][CELLS];
-  const int64_t n = n_off + (n_base ? *n_base : 0);
-  const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t P = p.pe[0], nbound = p.use_pe[0] ? P : 0;
-  const int nx = p.n[0], RR = p.zr[0] + H;
-  for (int64_t b = warp; b < (nbound > 0 ? nbound : 1); b += nwarps) {
-    const int64_t sides[2] = {nbound ? 2 * ((b + P - 1) % P) + 1 : 0, nbound ? 2 * b : 1};
-    const int base = (int)(b * p.S[0]) - RR;  // cell of local index 0 (before wrapping)
-    if (nbound)
-      for (int i = lane; i < 2 * RR; i += 32) lev[wb][0][i] = p.ring[(n % p.R) * p.ntot + wrap_coord(base + i, nx)];
-    __syncwarp();
-    for (int j = 0; j + 1 < K; ++j) {
-      const int64_t st = n + j;  // the step this pass computes; it draws the delays of step st + 1
-      const uint8_t *keff = p.keff + (st & 1) * p.nb;
-      // delays of step st seen across this boundary: by the cells left of it (the right side of the PE before) and
-      // by the cells right of it (the left side of the PE after); read before this pass's draw of step st + 1
-      const int k_lo = nbound ? keff[sides[0]] : 0, k_hi = nbound ? keff[sides[1]] : 0;
-      __syncwarp();
-      if (lane < 2) {
-        const int64_t side = sides[lane];
-        int raw = 0;
-        if (p.scheme != 0)
-          raw = delay_draw(p.seed, (uint32_t)(st + 1), (uint32_t)side, p.L, p.use_thr ? p.thr : nullptr);
-        p.keff[((st + 1) & 1) * p.nb + side] = (uint8_t)delay_clamp(raw, st + 1, p.T);
-        if (p.log != nullptr && st + 1 < p.log_steps) p.log[(st + 1) * p.nb + side] = (uint8_t)raw;
-      }
-      if (nbound) {
-        double *out = p.ring + ((st + 1) % p.R) * p.ntot;
-        const int r = p.zr[j];
-        for (int i = RR - r + lane; i < RR + r; i += 32) {
-          const bool left = i < RR;
-          double acc = fma(p.s0, lev[wb][j][i], p.zero);
+struct Zone {
+  static constexpr int CELLS = 2 * 27 + 2, HIST = (AT_MAX_L + AT_MAX_T) * 2 * H;
+  static constexpr int BYTES = (K * CELLS + HIST + 2 * H) * 8;
+};
+
+// Steps n .. n+K-1 near the PE boundary b (a warp).  The arithmetic is the FP64 chain's: the centre tap, then the taps in
+// offset order, a buffer point's value extrapolated over the delayed levels w_m(k) in the order m = 0 .. T-1.  Every
+// global load is in flight before the first step.
+template <int H, int K>
+__device__ __forceinline__ void zone_steps(const StepParams &p, int64_t n, int sn, int b, int lane, double *sh) {
+  constexpr int CELLS = Zone<H, K>::CELLS;
+  double *lev = sh, *hist = sh + K * CELLS, *hv = hist + Zone<H, K>::HIST;
+  const bool split = p.use_pe[0] != 0;
+  const int P = p.pe[0], nx = p.n[0], RR = p.zr[0] + H, R = p.R;
+  // the sides facing the boundary: the right one of the PE before it, the left one of the PE after it
+  const int side = lane & 1 ? (split ? 2 * b : 1) : (split ? 2 * (b == 0 ? P - 1 : b - 1) + 1 : 0);
+  const int base = b * p.S[0] - RR;  // cell of local index 0 (before wrapping)
+  int k = lane < 2 ? p.keff[(n & 1) * p.nb + side] : 0;  // lanes 0, 1: delays of step n; lanes 2j, 2j+1: of step n + j
+  if (split) {
+    const double *un = p.ring + (int64_t)sn * p.ntot;
+    for (int i = lane; i < 2 * RR; i += 32) lev[i] = un[wrap_coord(base + i, nx)];
+    for (int e = lane; e < (R - 2) * 2 * H; e += 32) {
+      const int d = e / (2 * H), c = e - d * (2 * H);
+      hist[e] = p.ring[slot_back(sn, d + 1, R) * p.ntot + wrap_coord(base + RR - H + c, nx)];
+    }
+  }
+  int last = 0;
+  if (lane < 2 * K) {  // delays of steps n+1 .. n+K
+    const int64_t st = n + 1 + (lane >> 1);
+    int raw = 0;
+    if (p.scheme != 0) raw = delay_draw(p.seed, (uint32_t)st, (uint32_t)side, p.L, p.use_thr ? p.thr : nullptr);
+    last = delay_clamp(raw, st, p.T);
+    if (p.log != nullptr && st < p.log_steps) p.log[st * p.nb + side] = (uint8_t)raw;
+  }
+  const int up = __shfl_up_sync(0xffffffffu, last, 2);
+  if (lane >= 2) k = up;
+  if (lane >= 2 * K - 2 && lane < 2 * K) p.keff[((n + K) & 1) * p.nb + side] = (uint8_t)last;
+  if (!split) return;
+  __syncwarp();
 #pragma unroll
-          for (int t = -H; t <= H; ++t) {
-            if (t == 0) continue;
-            const int ii = i + t;
-            double v = lev[wb][j][ii];
-            const int k = left == (ii < RR) ? 0 : (left ? k_lo : k_hi);  // a tap across the boundary: buffer point
-            if (k > 0) {
-              const int cell = wrap_coord(base + ii, nx);
-              double h = 0.0;
+  for (int j = 0; j < K; ++j) {
+    const int k_lo = __shfl_sync(0xffffffffu, k, 2 * j), k_hi = __shfl_sync(0xffffffffu, k, 2 * j + 1);
+    if (lane < 2 * H) {  // halo value of face cell lane: the left ones are buffer points of the PE after the boundary
+      const int ii = RR - H + lane, kk = lane < H ? k_hi : k_lo;
+      double v = lev[j * CELLS + ii];
+      if (kk > 0) {
 #pragma unroll
-              for (int m = 0; m < AT_MAX_T; ++m) {
-                if (m >= p.T) break;
-                const int64_t q = st - k - m;  // level read: in shared memory from n on, else in the ring
-                const double u = q >= n ? lev[wb][q - n][ii] : p.ring[(q % p.R) * p.ntot + cell];
-                h = m == 0 ? fma(p.w[k][0], u, p.zero) : fma(p.w[k][m], u, h);
-              }
-              v = h;
-            }
-            acc = fma(p.s[0][t + H], v, acc);
-          }
-          lev[wb][j + 1][i] = acc;
-          out[wrap_coord(base + i, nx)] = acc;
+        for (int m = 0; m <= H; ++m) {
+          if (m >= p.T) break;
+          const int q = j - kk - m;  // level relative to n
+          const double u = q >= 0 ? lev[q * CELLS + ii] : hist[(-q - 1) * 2 * H + lane];
+          v = m == 0 ? fma(p.w[kk][0], u, p.zero) : fma(p.w[kk][m], u, v);
         }
       }
-      __syncwarp();
+      hv[lane] = v;
     }
+    __syncwarp();
+    double *out = p.ring + (int64_t)slot_back(sn, R - 1 - j, R) * p.ntot;  // slot of level n + j + 1
+    const int r = j + 1 < K ? p.zr[j] : 4 * p.fe;
+    for (int i = RR - r + lane; i < RR + r; i += 32) {
+      const bool left = i < RR;
+      double acc = fma(p.s0, lev[j * CELLS + i], p.zero);
+#pragma unroll
+      for (int t = -H; t <= H; ++t) {
+        if (t == 0) continue;
+        const int ii = i + t;
+        const double v = left == (ii < RR) ? lev[j * CELLS + ii] : hv[ii - (RR - H)];
+        acc = fma(p.s[0][t + H], v, acc);
+      }
+      if (j + 1 < K) lev[(j + 1) * CELLS + i] = acc;
+      out[wrap_coord(base + i, nx)] = acc;
+    }
+    __syncwarp();
   }
 }
 
@@ -168,8 +170,12 @@ template <int TK, int C>
 struct BlockTile {
   static constexpr int CELLS = 32 * C, WIN = CELLS + 2 * TK;
   static constexpr int SLOTS = WIN + WIN / C + 1;  // one pad slot per C cells: lanes C cells apart take all banks
-  static constexpr int BYTES = SLOTS * 8;
 };
+template <int H, int K, int C>
+constexpr int block_warp_bytes() {  // of a warp, for a zone or a tile
+  const int t = BlockTile<H * K, C>::SLOTS * 8, z = Zone<H, K>::BYTES;
+  return (t > z ? t : z) + 15 & ~15;
+}
 
 // The C outputs of a lane from its window in shared memory, four at a time (independent chains for the pipe's latency).
 // F32: the low parts are there as FP32 and the cross terms are summed in FP32.
@@ -212,37 +218,40 @@ __device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, 
   }
 }
 
-// The last step m = n + K - 1 of a block: inner cells U^{n+K} = ck * U^n, edge groups the step from U^m.
+// A block: zones near the PE boundaries, inner cells U^{n+K} = ck * U^n.
 //
 // The inner cells are a contraction of 2 h K + 1 constant taps, which the FP64 pipe bounded (17 DFMA per cell at order
-// 4 and K = 4).  They are summed in block fixed point (fixed.cuh): three integer multiply-adds per tap.  A warp takes a
-// tile of 32 C cells: it reads the tile and its halo once (coalesced, all loads in flight together), finds their
-// largest exponent, converts every value once and lays the two 32-bit parts in shared memory; each lane then reads the
-// window of its C cells once, sums its C outputs from registers, and the results go back through shared memory to
-// coalesced stores.  What bounds it is the issue of the 32-bit integer pipe: 3 (2 h K + 1) multiply-adds per cell
-// beside about 30 logic and shift instructions (11 per converted value, 19 per rounded result).
+// 4 and K = 4).  They are summed in block fixed point (fixed.cuh).  A warp takes a tile of 32 C cells: it reads the tile
+// and its halo once (coalesced, all loads in flight together), finds their largest exponent, converts every value once
+// and lays the two 32-bit parts in shared memory; each lane then reads the window of its C cells once, sums its C
+// outputs from registers, and the results go back through shared memory to coalesced stores.  What bounds it is the
+// issue of the integer and FP32 pipes: per cell 17 multiply-adds of 64 bits (four cycles of a quarter each), 34 FFMA and
+// about 70 other instructions at order 4 and K = 4.  The zones, bound by the FP64 pipe's latency, run beside.
 template <int H, int K, int C>
 __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams p, const int64_t n_off,
-                                                            const int64_t *n_base) {
+                                                               const int64_t *n_base) {
   constexpr int TK = H * K;                  // half-width of the composed stencil
   using Tile = BlockTile<TK, C>;
-  extern __shared__ int2 block_smem[];
-  const int64_t m = n_off + (n_base ? *n_base : 0), n0 = m - (K - 1);
-  const double *__restrict__ u0 = p.ring + (n0 % p.R) * p.ntot;
-  const double *__restrict__ um = p.ring + (m % p.R) * p.ntot;
-  double *__restrict__ out = p.ring + ((m + 1) % p.R) * p.ntot;
-  const uint8_t *keff = p.keff + (m & 1) * p.nb;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
+  extern __shared__ __align__(16) char block_smem[];
+  const int64_t n = n_off + (n_base ? *n_base : 0);
+  const int sn = (int)slot_of(n, p.R);
+  const double *__restrict__ u0 = p.ring + (int64_t)sn * p.ntot;
+  double *__restrict__ out = p.ring + slot_back(sn, p.R - K, p.R) * p.ntot;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, warps = (gridDim.x * blockDim.x) >> 5;
   const int nx = p.n[0];
   const int lane = threadIdx.x & 31;
-  int2 *sm = block_smem + (threadIdx.x >> 5) * Tile::SLOTS;
+  int2 *sm = reinterpret_cast<int2 *>(block_smem + (threadIdx.x >> 5) * block_warp_bytes<H, K, C>());
   const int S = p.use_pe[0] ? p.S[0] : nx, inner = S - 8 * p.fe;
   const int per_pe = (inner + Tile::CELLS - 1) / Tile::CELLS;
-  const int tiles = (nx / S) * per_pe;
-  // Inner cells first: they read U^n only, so they may run while the zone launch (this block's steps n .. m-1 near
-  // the PE boundaries, launched with a programmatic dependency) still does.  Then wait for it: the edge groups read
-  // its U^m, and the delays of step m+1 go into the buffer slot its first step reads.
-  for (int t = (int)(tid >> 5); t < tiles; t += (int)(nthreads >> 5)) {
+  const int tiles = (nx / S) * per_pe, zones = p.use_pe[0] ? p.pe[0] : 1;
+  // Work items, one per warp at a time: the zones (long chains) first, then the tiles.
+  for (int w = tid >> 5; w < zones + tiles; w += warps) {
+    if (w < zones) {
+      zone_steps<H, K>(p, n, sn, w, lane, reinterpret_cast<double *>(sm));
+      __syncwarp();
+      continue;
+    }
+    const int t = w - zones;
     const int pe = t / per_pe, off = (t - pe * per_pe) * Tile::CELLS;
     const int x0 = pe * S + 4 * p.fe + off, len = min(Tile::CELLS, inner - off);
     // A PE's last tile reads on past its inner cells: U^n is written nowhere meanwhile, and only the scale sees them.
@@ -315,11 +324,6 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
         if (lane + 32 * q < len) dst[32 * q] = ro[lane + 32 * q + (lane + 32 * q) / C];
     }
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  draw_sides(p, m + 1, tid, nthreads, p.keff + ((m + 1) & 1) * p.nb);
-  const int64_t groups = nx >> 2, n_inner = (int64_t)(nx / S) * (inner >> 2);
-  for (int64_t k = n_inner + tid; k < groups; k += nthreads)
-    group_step<1, H, LdgNC, false, 0>(p, keff, um, out, m, (int)(group_1d_order_e(p, k, p.fe) << 2), 0, 0);
 }
 
 __device__ __forceinline__ void point_coords(const StepParams &p, int dim, int64_t i, int c[3]) {
@@ -338,8 +342,8 @@ template <int DIM, int H, bool AB, int KIND>
 __global__ void __launch_bounds__(512) forward_point_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   const int64_t n = n_off + (n_base ? *n_base : 0);
-  const double *__restrict__ un = p.ring + (n % p.R) * p.ntot;
-  double *__restrict__ out = p.ring + ((n + 1) % p.R) * p.ntot;
+  const double *__restrict__ un = p.ring + slot_of(n, p.R) * p.ntot;
+  double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
   draw_sides(p, n + 1, tid, nthreads, p.keff + ((n + 1) & 1) * p.nb);
@@ -487,22 +491,11 @@ namespace {
 template <int H, int K, int C>
 void launch_block_tiles(const StepParams &p, int max_blocks, int64_t tiles, int threads, int64_t n_off,
                         const int64_t *n_base, cudaStream_t st) {
-  const int warps = threads / 32, bytes = warps * BlockTile<H * K, C>::BYTES;
+  const int warps = threads / 32, bytes = warps * block_warp_bytes<H, K, C>();
   auto kernel = forward_block_kernel<H, K, C>;
   if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  const int64_t b = (tiles + warps - 1) / warps;
-  // the block launch depends programmatically on the zone launch (it waits for it inside, before its edge groups)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(b < max_blocks ? b : max_blocks));
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)bytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, p, n_off + K - 1, n_base);
+  const int64_t items = tiles + (p.use_pe[0] ? p.pe[0] : 1), b = (items + warps - 1) / warps;
+  kernel<<<(unsigned)(b < max_blocks ? b : max_blocks), threads, bytes, st>>>(p, n_off, n_base);
 }
 
 // Tiles of 32 C cells over the inner cells of every PE.
@@ -512,9 +505,8 @@ int64_t block_tiles(const StepParams &p, int C) {
 }
 
 template <int H, int K>
-void launch_block_typed(const StepParams &p, int max_blocks, int zblocks, int threads, int64_t n_off,
-                        const int64_t *n_base, cudaStream_t st) {
-  forward_zones_kernel<H, K><<<zblocks, 128, 0, st>>>(p, n_off, n_base);
+void launch_block_typed(const StepParams &p, int max_blocks, int threads, int64_t n_off, const int64_t *n_base,
+                        cudaStream_t st) {
   // Cells per lane: 8 convert 9/8 of the values and give a PE's last tile of 256 cells to fill, 4 convert 5/4 of them
   // and fill tiles of 128; instructions per tile: C + 1 conversions and C outputs.
   const int64_t t8 = block_tiles(p, 8), t4 = block_tiles(p, 4);
@@ -526,11 +518,11 @@ void launch_block_typed(const StepParams &p, int max_blocks, int zblocks, int th
 }
 
 template <int H>
-void launch_block_h(const StepParams &p, int blocks, int zblocks, int threads, int64_t n_off, const int64_t *n_base,
+void launch_block_h(const StepParams &p, int blocks, int threads, int64_t n_off, const int64_t *n_base,
                     cudaStream_t st) {
-  if (p.fuse_k == 2) launch_block_typed<H, 2>(p, blocks, zblocks, threads, n_off, n_base, st);
-  else if (p.fuse_k == 3) launch_block_typed<H, 3>(p, blocks, zblocks, threads, n_off, n_base, st);
-  else launch_block_typed<H, 4>(p, blocks, zblocks, threads, n_off, n_base, st);
+  if (p.fuse_k == 2) launch_block_typed<H, 2>(p, blocks, threads, n_off, n_base, st);
+  else if (p.fuse_k == 3) launch_block_typed<H, 3>(p, blocks, threads, n_off, n_base, st);
+  else launch_block_typed<H, 4>(p, blocks, threads, n_off, n_base, st);
 }
 
 }  // namespace
@@ -538,12 +530,9 @@ void launch_block_h(const StepParams &p, int blocks, int zblocks, int threads, i
 cudaError_t launch_forward_block(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st) {
   const int threads = p.threads == 128 ? 128 : 256;  // the block kernel's 80 registers give three blocks of 256 per SM
   const int max_blocks = sm_count() * (p.blocks_per_sm > 0 ? p.blocks_per_sm : 32);
-  const int64_t nwarps = p.use_pe[0] ? p.pe[0] : 1;  // zone launch: one warp per PE boundary, four per block
-  const int64_t zb = (nwarps + 3) / 4;
-  const int zblocks = (int)(zb < max_blocks ? zb : max_blocks);
-  if (p.h == 1) launch_block_h<1>(p, max_blocks, zblocks, threads, n_off, n_base, st);
-  else if (p.h == 2) launch_block_h<2>(p, max_blocks, zblocks, threads, n_off, n_base, st);
-  else launch_block_h<3>(p, max_blocks, zblocks, threads, n_off, n_base, st);
+  if (p.h == 1) launch_block_h<1>(p, max_blocks, threads, n_off, n_base, st);
+  else if (p.h == 2) launch_block_h<2>(p, max_blocks, threads, n_off, n_base, st);
+  else launch_block_h<3>(p, max_blocks, threads, n_off, n_base, st);
   return cudaGetLastError();
 }
 

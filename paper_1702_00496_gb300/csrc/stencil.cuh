@@ -48,6 +48,9 @@ __device__ __forceinline__ void draw_sides(const StepParams &p, int64_t n, int64
   }
 }
 
+// Ring slot of level n: steps fit 32 bits (at_step refuses more), so no 64-bit division.
+__device__ __forceinline__ int64_t slot_of(int64_t n, int R) { return (int64_t)((uint32_t)n % (uint32_t)R); }
+
 // Slot of the level `back` levels below the level in slot sn (0 <= back < R): no 64-bit modulo per load.
 __device__ __forceinline__ int64_t slot_back(int sn, int back, int R) {
   const int s = sn - back;
@@ -124,7 +127,7 @@ __device__ __forceinline__ void group_eval(const StepParams &p, const uint8_t *_
                                            double r[4], double uc[4]) {
   constexpr int W = XWin<H>::W, NW = XWin<H>::N;
   const int nx = p.n[0];
-  const int sn = (int)(n % p.R);
+  const int sn = (int)slot_of(n, p.R);
   const int64_t row = DIM == 3 ? ((int64_t)z * p.n[1] + y) * nx : 0;
   const int64_t i0 = row + x0;
   int pidx[3] = {x0 / p.S[0], 0, 0}, pos[3] = {0, 0, 0};
@@ -310,7 +313,7 @@ __device__ __forceinline__ void window_1d(const StepParams &p, const uint8_t *__
     for (int t = 0; t < NW; ++t) v[t] = LD::ld(un + wrap_coord(x0 - W + t, nx));
   }
   if (p.use_pe[0] && (pos0 < H || pos0 + 3 >= p.S[0] - H)) {
-    const int sn = (int)(n % p.R);
+    const int sn = (int)slot_of(n, p.R);
     const bool lo = !OWN_SIDES || pos0 < H, hi = !OWN_SIDES || pos0 + 3 >= p.S[0] - H;
     const int kl = lo ? keff[side_of<1>(p, pidx, 0, 0)] : 0, kr = hi ? keff[side_of<1>(p, pidx, 0, 1)] : 0;
 #pragma unroll
@@ -456,7 +459,7 @@ __device__ double point_update(const StepParams &p, const uint8_t *__restrict__ 
       int k = 0;
       if (edge && pos[a] + j < 0) k = keff[side_of<DIM>(p, pidx, a, 0)];
       if (edge && pos[a] + j >= p.S[a]) k = keff[side_of<DIM>(p, pidx, a, 1)];
-      const double v = k > 0 ? halo_value<LD>(p, cell, (int)(n % p.R), k) : LD::ld(un + cell);
+      const double v = k > 0 ? halo_value<LD>(p, cell, (int)slot_of(n, p.R), k) : LD::ld(un + cell);
       acc = fma(p.s[a][j + H], v, acc);
     }
   }
@@ -500,7 +503,7 @@ __device__ double point_update_burgers(const StepParams &p, const uint8_t *__res
     int k = 0;
     if (edge && pos + j < 0) k = keff[side_of<1>(p, pidx, 0, 0)];
     if (edge && pos + j >= p.S[0]) k = keff[side_of<1>(p, pidx, 0, 1)];
-    const double v = k > 0 ? halo_value<LD>(p, cj, (int)(n % p.R), k) : LD::ld(un + cj);
+    const double v = k > 0 ? halo_value<LD>(p, cj, (int)slot_of(n, p.R), k) : LD::ld(un + cj);
     a1 = j == -H ? fma(p.b1[0], v, p.zero) : fma(p.b1[j + H], v, a1);
     a2 = fma(p.b2[j + H], v, a2);
   }
@@ -515,7 +518,7 @@ template <int DIM, class LD>
 __device__ double point_update_space(const StepParams &p, const uint8_t *__restrict__ keff,
                                      const double *__restrict__ un, int64_t n, int64_t i, const int c[3]) {
   const int64_t stride[3] = {1, (int64_t)p.n[0], (int64_t)p.n[0] * p.n[1]};
-  const int sn = (int)(n % p.R);
+  const int sn = (int)slot_of(n, p.R);
   int pidx[3] = {0, 0, 0}, krow[3] = {0, 0, 0}, srow[3] = {0, 0, 0};
 #pragma unroll
   for (int a = 0; a < DIM; ++a) pidx[a] = c[a] / p.S[a];  // the whole PE index before any side lookup
