@@ -398,6 +398,12 @@ extern "C" int at_step(at_handle_t *hd, int64_t nsteps) {
   if (hd->sp.log && hd->step + nsteps > hd->log_steps) return fail(AT_ERR_STATE, "at_step: delay log is full");
   if (hd->step + nsteps > 0xFFFFFFFFll) return fail(AT_ERR_STATE, "at_step: step counter exceeds 32 bits");
   cudaError_t e;
+  if (nsteps > 1 && hd->sp.fuse_k < 3 && small_steps_fit(hd->sp)) {
+    if ((e = launch_small_steps(hd->sp, hd->step, nsteps, hd->stream)) != cudaSuccess)
+      return cuda_fail(e, "at_step: launch");
+    hd->step += nsteps;
+    return AT_OK;
+  }
   int64_t s = 0;
   // the start of a multistep run from a caller's field, where the weights change from step to step, runs in single
   // launches; the captured graphs hold steps of the steady form

@@ -158,6 +158,9 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
 cudaError_t launch_forward_step(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
 // The fuse_k steps n .. n+fuse_k-1 of a block (n = n_off + *n_base): zone launches, then the block launch.
 cudaError_t launch_forward_block(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
+// nsteps steps n .. of a small 1D problem in one launch (small.cu), and whether the problem is one.
+bool small_steps_fit(const StepParams &p);
+cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t st);
 // 3D: the step in fixed point over tiles of the PEs (brick.cu); false: the shape or scheme is not one for it, nothing
 // launched.
 bool launch_forward_brick(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st, cudaError_t *e);

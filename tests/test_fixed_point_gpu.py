@@ -123,3 +123,36 @@ def test_non_finite_values_spread_as_in_the_oracle(name, make, value):
     fine = np.isfinite(ref)
     assert np.array_equal(fine, np.isfinite(u))
     assert np.abs(u[fine] - ref[fine]).max() <= 1e-12 * np.abs(ref[fine]).max()
+
+
+SMALL = [
+    ("n16_o2", lambda: W.wl_1d(16, 2, 2, 3, 0, 641, (1, 2))[0]),
+    ("n256_o2_log", lambda: W.wl_1d(256, 8, 2, 3, 0, 642, (1, 2))[0]),
+    ("n2048_o4_most_sides", lambda: W.wl_1d(2048, 512, 4, 4, 0, 643, (1, 2))[0]),
+    ("n2048_o6_ab3", lambda: W.wl_1d(2048, 64, 6, 3, 0, 644, (1, 2), r_alpha=0.01, tsteps=3)[0]),
+    ("n1288_o4_ab2_unsplit", lambda: W.wl_1d(1288, 1, 4, 3, 0, 645, (1, 2), r_alpha=0.02, tsteps=2)[0]),
+    ("n640_o4_burgers", lambda: dict(W.wl_1d(640, 10, 4, 3, 0, 646, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
+    ("n640_space", lambda: W.wl_1d(640, 10, 2, 3, 0, 647, (1, 2), scheme=W.AT_SPACE2)[0]),
+]
+
+
+@pytest.mark.parametrize("callers_field", [False, True])
+@pytest.mark.parametrize("name,make", SMALL, ids=[s[0] for s in SMALL])
+def test_small_problems_in_one_launch_are_bitwise_single_steps(name, make, callers_field):
+    """A call of several steps of a small problem runs in one launch, a call of one step is a launch of its own: the same
+    bits and delays for any split of the steps, also where the multistep start-up falls into the launch."""
+    from paper_1702_00496_gb300 import Solver, at_set_fusion
+    spec = make()
+    runs = []
+    for split in ([1] * 37, [37], [2, 1, 34]):
+        s = Solver(spec, log_steps=37)
+        at_set_fusion(s.h, 1)
+        if callers_field:
+            s.reset(torch.as_tensor(_field(spec, "smooth"), device="cuda"))
+        for m in split:
+            s.step(m)
+        s.sync()
+        runs.append((s.field().clone(), s.delays().clone()))
+        s.close()
+    for u, d in runs[1:]:
+        assert torch.equal(u, runs[0][0]) and torch.equal(d, runs[0][1])
