@@ -202,6 +202,8 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
     const uint32_t gS = (uint32_t)((p.use_pe[0] ? p.S[0] : p.n[0]) >> 2);
     p.div_g = atfd::fast_div(gS);
     p.div_in = atfd::fast_div(gS > 2 ? gS - 2 : 1);
+    const uint32_t up = ((uint32_t)(p.use_pe[0] ? p.S[0] : p.n[0]) + 3) >> 2;
+    p.div_up = atfd::fast_div(up > 3 ? up - 3 : 1);
   } else {
     double t[6 * AT_MAX_H + 1] = {p.s0};
     int c = 1;

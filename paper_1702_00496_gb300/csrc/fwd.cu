@@ -40,7 +40,8 @@ template <int DIM, int H, int AB, int KIND>
 __global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   const int64_t n = n_off + (n_base ? *n_base : 0);
-  const double *__restrict__ un = p.ring + slot_of(n, p.R) * p.ntot;
+  const int sn = (int)slot_of(n, p.R);
+  const double *__restrict__ un = p.ring + sn * p.ntot;
   double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
@@ -50,13 +51,13 @@ __global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(co
   for (int64_t k = tid; k < groups; k += nthreads) {
     if (DIM == 1) {
       const int64_t g = group_1d_order(p, k);
-      group_step<1, H, LdgNC, AB, KIND>(p, keff, un, out, n, (int)(g << 2), 0, 0);
+      group_step<1, H, LdgNC, AB, KIND>(p, keff, un, out, n, sn, (int)(g << 2), 0, 0);
     } else {
       const int64_t g = p.order ? (int64_t)p.order[k] : k;
       const int64_t r = g / gx;
       const int x0 = (int)(g - r * gx) << 2;
       const int z = (int)(r / p.n[1]), y = (int)(r - (int64_t)z * p.n[1]);
-      group_step<3, H, LdgNC, AB, KIND>(p, keff, un, out, n, x0, y, z);
+      group_step<3, H, LdgNC, AB, KIND>(p, keff, un, out, n, sn, x0, y, z);
     }
   }
 }
@@ -326,17 +327,6 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
   }
 }
 
-__device__ __forceinline__ void point_coords(const StepParams &p, int dim, int64_t i, int c[3]) {
-  c[0] = (int)i; c[1] = 0; c[2] = 0;
-  if (dim == 3) {
-    const int nx = p.n[0], ny = p.n[1];
-    const int64_t yz = i / nx;
-    c[0] = (int)(i - yz * nx);
-    c[2] = (int)(yz / ny);
-    c[1] = (int)(yz - (int64_t)c[2] * ny);
-  }
-}
-
 // Fallback for shapes the grouped kernel does not take (n[0] not a multiple of 4, odd slots).
 template <int DIM, int H, bool AB, int KIND>
 __global__ void __launch_bounds__(512) forward_point_kernel(const StepParams p, const int64_t n_off,
@@ -347,27 +337,24 @@ __global__ void __launch_bounds__(512) forward_point_kernel(const StepParams p, 
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nthreads = (int64_t)gridDim.x * blockDim.x;
   draw_sides(p, n + 1, tid, nthreads, p.keff + ((n + 1) & 1) * p.nb);
-  for (int64_t i = tid; i < p.ntot; i += nthreads) {
-    int c[3];
-    point_coords(p, DIM, i, c);
-    AbLevels<1> old;
-    if (AB) ab_fetch<1>(p, n, i, old);
-    if (DIM == 1 && KIND == 1) {
-      double r[1] = {point_update_burgers<H, LdgNC>(p, keff, un, n, i)};
-      const double u[1] = {un[i]};
-      if (AB) ab_combine<1>(p, n, i, u, r, old);
-      else r[0] = u[0] + r[0];
-      out[i] = r[0];
-      continue;
-    }
-    double r[1] = {(KIND == 2 && H == 1) ? point_update_space<DIM, LdgNC>(p, keff, un, n, i, c)
-                                         : point_update<DIM, H, LdgNC>(p, keff, un, n, i, c)};
-    if (AB) {
-      const double u[1] = {un[i]};
-      ab_combine<1>(p, n, i, u, r, old);
-    }
-    out[i] = r[0];
-  }
+  for (int64_t i = tid; i < p.ntot; i += nthreads) point_step<DIM, H, LdgNC, AB, KIND>(p, keff, un, out, n, i);
+}
+
+// Large 1D shapes without aligned groups of four: groups cut from each PE's first cell (750000 points in PEs of 250, order
+// 4: the per-point kernel took 15.7 us per step, bound by its FP64 chains and index divisions, this one 9.8; 10 million
+// points unsplit with AB2 851 against 90).
+template <int H, int AB, int KIND>
+__global__ void __launch_bounds__(256, 4) forward_ragged_kernel(const StepParams p, const int64_t n_off,
+                                                                const int64_t *n_base) {
+  const int64_t n = n_off + (n_base ? *n_base : 0);
+  const int sn = (int)slot_of(n, p.R);
+  const double *__restrict__ un = p.ring + sn * p.ntot;
+  double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
+  const uint8_t *keff = p.keff + (n & 1) * p.nb;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = gridDim.x * blockDim.x;
+  draw_sides(p, n + 1, tid, nthreads, p.keff + ((n + 1) & 1) * p.nb);
+  const int groups = p.use_pe[0] ? p.pe[0] * ((p.S[0] + 3) >> 2) : (p.n[0] + 3) >> 2;
+  for (int k = tid; k < groups; k += nthreads) group_ragged<H, LdgNC, AB, KIND>(p, keff, un, out, n, sn, k);
 }
 
 // dt f(u) with central differences everywhere (p carries no PE split and s0 without the 1): the right-hand
@@ -426,14 +413,25 @@ bool grouped_shape(const StepParams &p, const void *base) {
          (p.frhs == nullptr || (reinterpret_cast<uintptr_t>(p.frhs) % 16) == 0);
 }
 
+int sm_count() {
+  int sms = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 // AB: 0 forward Euler, 1 Adams-Bashforth, 2 AB2 with both levels stored (the 1D linear grouped step only; Burgers'
 // step, 3D and the per-point fallback take the general form: Burgers' AB2 step measured 462 against 406 us in it).
 template <int DIM, int H, int AB>
 void launch_typed(const StepParams &p, bool grouped, int blocks, int threads, int64_t n, const int64_t *n_base,
                   cudaStream_t st) {
   constexpr int ABG = AB ? 1 : 0;
+  // per step, tiny / per million points more, us: the per-point kernel 2.9 / 7.5 (order 2), 3.9 / 9.3 (order 4), 5.6 / 11.7
+  // (order 6), 4.3 / 22 (AB2); groups in fixed point 3.1 / 4.6, 4.6 / 5.8, 6.4 / 6.6, 5.4 / 9.5
+  const bool ragged = p.ntot >= 196608;
+  const int rblocks = (int)std::min<int64_t>((p.ntot / 2 + 255) / 256, (int64_t)sm_count() * 32);
   if (DIM == 1 && p.burgers) {
     if (grouped) forward_group_kernel<1, H, ABG, 1><<<blocks, threads, 0, st>>>(p, n, n_base);
+    else if (ragged) forward_ragged_kernel<H, ABG, 1><<<rblocks, 256, 0, st>>>(p, n, n_base);
     else forward_point_kernel<1, H, ABG != 0, 1><<<blocks, threads, 0, st>>>(p, n, n_base);
     return;
   }
@@ -445,6 +443,7 @@ void launch_typed(const StepParams &p, bool grouped, int blocks, int threads, in
     }
   }
   if (grouped) forward_group_kernel<DIM, H, DIM == 1 ? AB : ABG, 0><<<blocks, threads, 0, st>>>(p, n, n_base);
+  else if (DIM == 1 && ragged) forward_ragged_kernel<H, ABG, 0><<<rblocks, 256, 0, st>>>(p, n, n_base);
   else forward_point_kernel<DIM, H, AB != 0, 0><<<blocks, threads, 0, st>>>(p, n, n_base);
 }
 
@@ -454,12 +453,6 @@ void launch_h(const StepParams &p, bool grouped, int blocks, int threads, int64_
   if (p.h == 1) launch_typed<DIM, 1, AB>(p, grouped, blocks, threads, n, n_base, st);
   else if (p.h == 2) launch_typed<DIM, 2, AB>(p, grouped, blocks, threads, n, n_base, st);
   else launch_typed<DIM, 3, AB>(p, grouped, blocks, threads, n, n_base, st);
-}
-
-int sm_count() {
-  int sms = 152, dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
 }
 
 }  // namespace

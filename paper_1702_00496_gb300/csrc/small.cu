@@ -18,56 +18,74 @@ using namespace atfd;
 
 constexpr int kSmallThreads = 576;  // 512 groups of four points, and two warps that only draw delays
 
-template <int H, bool AB, int KIND>
+// GROUPED = false: shapes without aligned groups of four, point by point as the per-point kernel steps them.
+template <int H, bool AB, int KIND, bool GROUPED>
 __global__ void __launch_bounds__(kSmallThreads) small_steps_kernel(const StepParams p, const int64_t n0,
                                                                     const int64_t nsteps) {
   const int tid = threadIdx.x, nthreads = blockDim.x, groups = p.n[0] >> 2;
   const int g = tid < groups ? (int)group_1d_order(p, tid) : 0;
+  int sn = (int)slot_of(n0, p.R);
   for (int64_t n = n0; n < n0 + nsteps; ++n) {
-    const double *un = p.ring + slot_of(n, p.R) * p.ntot;
-    double *out = p.ring + slot_of(n + 1, p.R) * p.ntot;
+    const double *un = p.ring + sn * p.ntot;
+    const int sout = sn + 1 == p.R ? 0 : sn + 1;
+    double *out = p.ring + sout * p.ntot;
     const uint8_t *keff = p.keff + (n & 1) * p.nb;
     draw_sides(p, n + 1, nthreads - 1 - tid, nthreads, p.keff + ((n + 1) & 1) * p.nb);  // from the last thread down
-    if (tid < groups) group_step<1, H, LdCoherent, AB ? 1 : 0, KIND>(p, keff, un, out, n, g << 2, 0, 0);
+    if (GROUPED) {
+      if (tid < groups) group_step<1, H, LdCoherent, AB ? 1 : 0, KIND>(p, keff, un, out, n, sn, g << 2, 0, 0);
+    } else {
+      for (int i = tid; i < p.n[0]; i += nthreads) point_step<1, H, LdCoherent, AB, KIND>(p, keff, un, out, n, i);
+    }
     __syncthreads();
+    sn = sout;
   }
 }
 
+template <int H, bool AB, int KIND>
+void launch_small_typed(const StepParams &p, bool grouped, int64_t n, int64_t nsteps, cudaStream_t st) {
+  if (grouped) {
+    const int threads = (p.n[0] / 4 + 31) / 32 * 32 + (p.nb < 64 ? (int)(p.nb + 31) / 32 * 32 : 64);
+    small_steps_kernel<H, AB, KIND, true><<<1, threads, 0, st>>>(p, n, nsteps);
+  } else {
+    const int threads = p.n[0] < 512 ? (p.n[0] + 31) / 32 * 32 + 32 : kSmallThreads;
+    small_steps_kernel<H, AB, KIND, false><<<1, threads, 0, st>>>(p, n, nsteps);
+  }
+}
+
+bool small_grouped(const StepParams &p) {
+  return p.n[0] % 4 == 0 && (!p.use_pe[0] || p.S[0] % 4 == 0) && reinterpret_cast<uintptr_t>(p.ring) % 16 == 0 &&
+         (p.frhs == nullptr || reinterpret_cast<uintptr_t>(p.frhs) % 16 == 0);
+}
+
 template <int H>
-void launch_small_h(const StepParams &p, int threads, int64_t n, int64_t nsteps, cudaStream_t st) {
-  const bool ab = p.ts > 1;
+void launch_small_h(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t st) {
+  const bool ab = p.ts > 1, grouped = small_grouped(p);
   if (p.burgers) {
-    if (ab) small_steps_kernel<H, true, 1><<<1, threads, 0, st>>>(p, n, nsteps);
-    else small_steps_kernel<H, false, 1><<<1, threads, 0, st>>>(p, n, nsteps);
+    if (ab) launch_small_typed<H, true, 1>(p, grouped, n, nsteps, st);
+    else launch_small_typed<H, false, 1>(p, grouped, n, nsteps, st);
     return;
   }
   if constexpr (H == 1) {
     if (p.scheme >= AT_AT_SPACE2) {
-      small_steps_kernel<1, false, 2><<<1, threads, 0, st>>>(p, n, nsteps);
+      launch_small_typed<1, false, 2>(p, grouped, n, nsteps, st);
       return;
     }
   }
-  if (ab) small_steps_kernel<H, true, 0><<<1, threads, 0, st>>>(p, n, nsteps);
-  else small_steps_kernel<H, false, 0><<<1, threads, 0, st>>>(p, n, nsteps);
+  if (ab) launch_small_typed<H, true, 0>(p, grouped, n, nsteps, st);
+  else launch_small_typed<H, false, 0>(p, grouped, n, nsteps, st);
 }
 
 }  // namespace
 
-bool small_steps_fit(const StepParams &p) {
-  return p.dim == 1 && p.n[0] % 4 == 0 && p.n[0] <= 2048 && (!p.use_pe[0] || p.S[0] % 4 == 0) &&
-         reinterpret_cast<uintptr_t>(p.ring) % 16 == 0 &&
-         (p.frhs == nullptr || reinterpret_cast<uintptr_t>(p.frhs) % 16 == 0);
-}
+bool small_steps_fit(const StepParams &p) { return p.dim == 1 && p.n[0] <= (small_grouped(p) ? 2048 : 1024); }
 
 cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t st) {
-  const int groups = p.n[0] / 4;
-  int threads = (groups + 31) / 32 * 32 + (int)(p.nb < 64 ? (p.nb + 31) / 32 * 32 : 64);
   const int64_t most = 4096;  // steps of one launch
   for (int64_t s = 0; s < nsteps; s += most) {
     const int64_t m = nsteps - s < most ? nsteps - s : most;
-    if (p.h == 1) launch_small_h<1>(p, threads, n + s, m, st);
-    else if (p.h == 2) launch_small_h<2>(p, threads, n + s, m, st);
-    else launch_small_h<3>(p, threads, n + s, m, st);
+    if (p.h == 1) launch_small_h<1>(p, n + s, m, st);
+    else if (p.h == 2) launch_small_h<2>(p, n + s, m, st);
+    else launch_small_h<3>(p, n + s, m, st);
   }
   return cudaGetLastError();
 }

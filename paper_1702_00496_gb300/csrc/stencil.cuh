@@ -86,21 +86,6 @@ __device__ __forceinline__ int64_t group_1d_order(const StepParams &p, int64_t k
   return (int64_t)(kk >> 1) * gS + ((kk & 1) ? gS - 1 : 0);
 }
 
-// The same order with e edge groups at each PE end (e = 1 is group_1d_order): the gS - 2e inner groups of every PE
-// first, then the 2e edge groups of every PE.  k < number of groups; requires gS > 2e.
-__device__ __forceinline__ int64_t group_1d_order_e(const StepParams &p, int64_t k, int e) {
-  const uint32_t gS = (uint32_t)(p.use_pe[0] ? p.S[0] >> 2 : p.n[0] >> 2);
-  if (e == 0) return k;
-  const uint32_t inner = gS - 2 * e, npe = (uint32_t)(p.n[0] >> 2) / gS, uk = (uint32_t)k;
-  const uint32_t n_int = npe * inner;
-  if (uk < n_int) {
-    const uint32_t pe = uk / inner;
-    return (int64_t)pe * gS + e + (uk - pe * inner);
-  }
-  const uint32_t kk = uk - n_int, pe = kk / (2 * e), r = kk - pe * (2 * e);
-  return (int64_t)pe * gS + (r < (uint32_t)e ? r : gS - 2 * e + r);
-}
-
 // Side index of face (axis a, lo/hi) of the PE with index (px, py, pz).
 template <int DIM>
 __device__ __forceinline__ int64_t side_of(const StepParams &p, const int pidx[3], int a, int hi) {
@@ -118,10 +103,8 @@ struct XWin {
 
 // The merged stencil of the four points x0..x0+3 of row (y, z) into r[4] (and their level-n values into uc[4]);
 // requires n[0] % 4 == 0 and a 16-byte aligned slot.  keff: effective delays of step n.  ALPHA = true evaluates
-// the alpha derivative of the step instead (coefficients q0, q: dt times the AT second derivative).  OWN_SIDES = true
-// reads the delay of an x side only when the group reaches that side's buffer points (for callers whose other
-// sides' delays may be in flight).
-template <int DIM, int H, class LD, bool ALPHA, bool OWN_SIDES = false>
+// the alpha derivative of the step instead (coefficients q0, q: dt times the AT second derivative).
+template <int DIM, int H, class LD, bool ALPHA>
 __device__ __forceinline__ void group_eval(const StepParams &p, const uint8_t *__restrict__ keff,
                                            const double *__restrict__ un, int64_t n, int x0, int y, int z,
                                            double r[4], double uc[4]) {
@@ -151,8 +134,7 @@ __device__ __forceinline__ void group_eval(const StepParams &p, const uint8_t *_
 #pragma unroll
   for (int q = 0; q < 4; ++q) uc[q] = v[W + q];
   if (p.use_pe[0] && (pos[0] < H || pos[0] + 3 >= p.S[0] - H)) {
-    const bool lo = !OWN_SIDES || pos[0] < H, hi = !OWN_SIDES || pos[0] + 3 >= p.S[0] - H;
-    const int kl = lo ? keff[side_of<DIM>(p, pidx, 0, 0)] : 0, kr = hi ? keff[side_of<DIM>(p, pidx, 0, 1)] : 0;
+    const int kl = keff[side_of<DIM>(p, pidx, 0, 0)], kr = keff[side_of<DIM>(p, pidx, 0, 1)];
 #pragma unroll
     for (int t = W - H; t <= W + 3 + H; ++t) {
       const int rel = pos[0] - W + t;
@@ -294,10 +276,11 @@ __device__ __forceinline__ void ab_combine(const StepParams &p, int64_t n, int64
 // A group is taken only when both halves of it hold a value within kFxGuard bits of the window's largest; the others
 // (and windows that hold infinities or NaN, or lie at the ends of the exponent range) go through the chain.
 
-// x window of a 1D group: cells x0-W .. x0+3+W, buffer points replaced by the halo values of step n.
-template <int H, class LD, bool OWN_SIDES = false>
+// x window of a 1D group: cells x0-W .. x0+3+W, buffer points replaced by the halo values of step n (its level is in
+// slot sn).
+template <int H, class LD>
 __device__ __forceinline__ void window_1d(const StepParams &p, const uint8_t *__restrict__ keff,
-                                          const double *__restrict__ un, int64_t n, int x0, double v[XWin<H>::N]) {
+                                          const double *__restrict__ un, int sn, int x0, double v[XWin<H>::N]) {
   constexpr int W = XWin<H>::W, NW = XWin<H>::N;
   const int nx = p.n[0];
   const int pidx[3] = {p.use_pe[0] ? (int)fdiv((uint32_t)x0 >> 2, p.div_g) : 0, 0, 0};  // groups lie inside a PE
@@ -313,9 +296,7 @@ __device__ __forceinline__ void window_1d(const StepParams &p, const uint8_t *__
     for (int t = 0; t < NW; ++t) v[t] = LD::ld(un + wrap_coord(x0 - W + t, nx));
   }
   if (p.use_pe[0] && (pos0 < H || pos0 + 3 >= p.S[0] - H)) {
-    const int sn = (int)slot_of(n, p.R);
-    const bool lo = !OWN_SIDES || pos0 < H, hi = !OWN_SIDES || pos0 + 3 >= p.S[0] - H;
-    const int kl = lo ? keff[side_of<1>(p, pidx, 0, 0)] : 0, kr = hi ? keff[side_of<1>(p, pidx, 0, 1)] : 0;
+    const int kl = keff[side_of<1>(p, pidx, 0, 0)], kr = keff[side_of<1>(p, pidx, 0, 1)];
 #pragma unroll
     for (int t = W - H; t <= W + 3 + H; ++t) {
       const int rel = pos0 - W + t;
@@ -402,11 +383,25 @@ __device__ __forceinline__ bool group_fixed(const StepParams &p, const double v[
   return true;
 }
 
+// The sum as an FMA chain: the centre tap first, then the taps in offset order.
+template <int H>
+__device__ __forceinline__ void linear_chain(const StepParams &p, const double v[XWin<H>::N], double r[4]) {
+  constexpr int W = XWin<H>::W;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    double acc = fma(p.s0, v[q + W], p.zero);
+#pragma unroll
+    for (int j = -H; j <= H; ++j)
+      if (j != 0) acc = fma(p.s[0][j + H], v[q + W + j], acc);
+    r[q] = acc;
+  }
+}
+
 // Update the four points x0..x0+3 of row (y, z) (the forward step; AB: 0 forward Euler, 1 Adams-Bashforth, 2
 // AB2 with both levels stored, ab_combine's STEADY form).
-template <int DIM, int H, class LD, int AB = 0, bool OWN_SIDES = false>
+template <int DIM, int H, class LD, int AB = 0>
 __device__ __forceinline__ void group_update(const StepParams &p, const uint8_t *__restrict__ keff,
-                                             const double *__restrict__ un, double *__restrict__ out, int64_t n,
+                                             const double *__restrict__ un, double *__restrict__ out, int64_t n, int sn,
                                              int x0, int y, int z) {
   double r[4], uc[4];
   const int64_t i0 = (DIM == 3 ? ((int64_t)z * p.n[1] + y) * p.n[0] : 0) + x0;
@@ -415,21 +410,12 @@ __device__ __forceinline__ void group_update(const StepParams &p, const uint8_t 
   if constexpr (DIM == 1) {
     constexpr int W = XWin<H>::W;
     double v[XWin<H>::N];
-    window_1d<H, LD, OWN_SIDES>(p, keff, un, n, x0, v);
-    if (!group_fixed<H, AB != 0, 0>(p, v, r)) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double acc = fma(p.s0, v[q + W], p.zero);
-#pragma unroll
-        for (int j = -H; j <= H; ++j)
-          if (j != 0) acc = fma(p.s[0][j + H], v[q + W + j], acc);
-        r[q] = acc;
-      }
-    }
+    window_1d<H, LD>(p, keff, un, sn, x0, v);
+    if (!group_fixed<H, AB != 0, 0>(p, v, r)) linear_chain<H>(p, v, r);
 #pragma unroll
     for (int q = 0; q < 4; ++q) uc[q] = v[q + W];
   } else {
-    group_eval<DIM, H, LD, false, OWN_SIDES>(p, keff, un, n, x0, y, z, r, uc);
+    group_eval<DIM, H, LD, false>(p, keff, un, n, x0, y, z, r, uc);
   }
   if (AB) ab_combine<4, AB == 2>(p, n, i0, uc, r, old);
   reinterpret_cast<double2 *>(out + i0)[0] = make_double2(r[0], r[1]);
@@ -554,6 +540,39 @@ __device__ double point_update_space(const StepParams &p, const uint8_t *__restr
   return acc;
 }
 
+__device__ __forceinline__ void point_coords(const StepParams &p, int dim, int64_t i, int c[3]) {
+  c[0] = (int)i; c[1] = 0; c[2] = 0;
+  if (dim == 3) {
+    const int nx = p.n[0], ny = p.n[1];
+    const int64_t yz = i / nx;
+    c[0] = (int)(i - yz * nx);
+    c[2] = (int)(yz / ny);
+    c[1] = (int)(yz - (int64_t)c[2] * ny);
+  }
+}
+
+// One point of the forward step, any shape and scheme, as FMA chains.
+template <int DIM, int H, class LD, bool AB, int KIND>
+__device__ __forceinline__ void point_step(const StepParams &p, const uint8_t *__restrict__ keff,
+                                           const double *__restrict__ un, double *__restrict__ out, int64_t n, int64_t i) {
+  int c[3];
+  point_coords(p, DIM, i, c);
+  AbLevels<1> old;
+  if (AB) ab_fetch<1>(p, n, i, old);
+  const double u[1] = {LD::ld(un + i)};
+  double r[1];
+  if constexpr (DIM == 1 && KIND == 1) {
+    r[0] = point_update_burgers<H, LD>(p, keff, un, n, i);
+    if (!AB) r[0] = u[0] + r[0];
+  } else if constexpr (KIND == 2 && H == 1) {
+    r[0] = point_update_space<DIM, LD>(p, keff, un, n, i, c);
+  } else {
+    r[0] = point_update<DIM, H, LD>(p, keff, un, n, i, c);
+  }
+  if (AB) ab_combine<1>(p, n, i, u, r, old);
+  out[i] = r[0];
+}
+
 // Does the group x0..x0+3 of row (y, z) hold a PE-edge point of a split axis (AT_AT_SPACE2 / AT_AT_SPACE1)?
 template <int DIM>
 __device__ __forceinline__ bool group_at_space_edge(const StepParams &p, int x0, int y, int z) {
@@ -574,19 +593,81 @@ __device__ __forceinline__ bool group_at_space_edge(const StepParams &p, int x0,
   return false;
 }
 
+// Group k of a 1D shape without aligned groups of four (central and time-expanded rows, Burgers): every PE is cut into
+// groups of four from its first cell, the last one partial; 8-byte accesses.  The points beyond the PE that a partial
+// group sums are dropped.  As group_1d_order does, the groups that reach no buffer point come first (all of a PE's but
+// the first and the last two), then three per PE that do, so warps take one path.
+template <int H, class LD, int AB, int KIND>
+__device__ __forceinline__ void group_ragged(const StepParams &p, const uint8_t *__restrict__ keff,
+                                             const double *__restrict__ un, double *__restrict__ out, int64_t n, int sn,
+                                             int k) {
+  constexpr int W = XWin<H>::W;
+  const int nx = p.n[0], S = p.use_pe[0] ? p.S[0] : nx;
+  const int gS = (S + 3) >> 2, npe = p.use_pe[0] ? p.pe[0] : 1, n_in = gS > 3 ? npe * (gS - 3) : 0;
+  int pe, g;
+  if (k < n_in) {
+    pe = (int)fdiv((uint32_t)k, p.div_up);
+    g = 1 + k - pe * (gS - 3);
+  } else if (gS > 3) {
+    pe = (k - n_in) / 3;
+    g = k - n_in - 3 * pe;
+    g = g == 0 ? 0 : gS - 3 + g;
+  } else {
+    pe = k / gS;
+    g = k - pe * gS;
+  }
+  const int pos0 = 4 * g, x0 = pe * S + pos0;
+  const int nv = min(4, S - pos0);
+  AbLevels<1> old[4];
+  if (AB) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ab_fetch<1>(p, n, x0 + (q < nv ? q : 0), old[q]);
+  }
+  double v[XWin<H>::N], r[4];
+#pragma unroll
+  for (int t = 0; t < XWin<H>::N; ++t) {
+    int x = x0 - W + t;  // PEs are at least 2 h wide, a whole domain at least that: at most one wrap and W + 3 beyond
+    x = x < 0 ? x + nx : x;
+    x = x >= nx ? x - nx : x;
+    v[t] = LD::ld(un + (x < nx ? x : nx - 1));
+  }
+  if (p.use_pe[0] && (pos0 < H || pos0 + 3 >= S - H)) {
+    const int pidx[3] = {pe, 0, 0};
+    const int kl = keff[side_of<1>(p, pidx, 0, 0)], kr = keff[side_of<1>(p, pidx, 0, 1)];
+#pragma unroll
+    for (int t = W - H; t <= W + 3 + H; ++t) {
+      const int rel = pos0 - W + t;
+      const int kk = rel < 0 ? kl : (rel >= S && rel < S + H ? kr : 0);  // further cells no kept point reads
+      if (kk > 0) v[t] = halo_value<LD>(p, wrap_coord(x0 - W + t, nx), sn, kk);
+    }
+  }
+  if (!group_fixed<H, AB != 0, KIND>(p, v, r)) {
+    if (KIND) burgers_chain<H>(p, v, r);
+    else linear_chain<H>(p, v, r);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (q >= nv) continue;
+    const double u[1] = {v[W + q]};
+    if (AB) ab_combine<1>(p, n, x0 + q, u, r + q, old[q]);
+    else if (KIND) r[q] = u[0] + r[q];
+    out[x0 + q] = r[q];
+  }
+}
+
 // One group of the forward step for every scheme: groups holding a PE-edge point of a scheme expanded in space
 // go point by point through its edge rows, all others through the grouped central / time-expanded path.  KIND
 // selects the kernel variant -- 0: central and time-expanded rows, 1: Burgers' equation (1D), 2: rows expanded in
 // space -- so each kernel carries only its own path.
 template <int DIM, int H, class LD, int AB, int KIND = 0>
 __device__ __forceinline__ void group_step(const StepParams &p, const uint8_t *__restrict__ keff,
-                                           const double *__restrict__ un, double *__restrict__ out, int64_t n,
+                                           const double *__restrict__ un, double *__restrict__ out, int64_t n, int sn,
                                            int x0, int y, int z) {
   if (DIM == 1 && KIND == 1) {
     double v[XWin<H>::N], r[4], uc[4];
     AbLevels<4> old;
     if (AB) ab_fetch<4, AB == 2>(p, n, x0, old);
-    window_1d<H, LD>(p, keff, un, n, x0, v);
+    window_1d<H, LD>(p, keff, un, sn, x0, v);
     if (!group_fixed<H, AB != 0, 1>(p, v, r)) burgers_chain<H>(p, v, r);
 #pragma unroll
     for (int q = 0; q < 4; ++q) uc[q] = v[XWin<H>::W + q];
@@ -613,7 +694,7 @@ __device__ __forceinline__ void group_step(const StepParams &p, const uint8_t *_
     reinterpret_cast<double2 *>(out + i0)[1] = make_double2(r[2], r[3]);
     return;
   }
-  group_update<DIM, H, LD, AB>(p, keff, un, out, n, x0, y, z);
+  group_update<DIM, H, LD, AB>(p, keff, un, out, n, sn, x0, y, z);
 }
 
 }  // namespace atfd

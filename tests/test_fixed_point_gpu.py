@@ -32,6 +32,13 @@ PROBLEMS = [
     ("ab3_o6", lambda: W.wl_1d(64 * 20, 20, 6, 3, 0, 609, (1, 2), r_alpha=0.01, tsteps=3)[0]),
     ("burgers_ab2_o4", lambda: dict(W.wl_1d(64 * 20, 20, 4, 3, 0, 610, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
     ("burgers_euler_o2", lambda: dict(W.wl_1d(64 * 20, 20, 2, 3, 0, 611, (1, 2), c=0.0, r_alpha=0.02)[0], burgers=1)),
+    # large shapes without aligned groups: a last group of 1, 2 or 3 points per PE, narrow PEs, one PE
+    ("ragged_o2", lambda: W.wl_1d(197 * 1001, 1001, 2, 3, 0, 631, (1, 2))[0]),
+    ("ragged_o4", lambda: W.wl_1d(250 * 800, 800, 4, 4, 0, 632, (1, 2))[0]),
+    ("ragged_o4_narrow", lambda: W.wl_1d(5 * 40000, 40000, 4, 3, 0, 633, (1, 2))[0]),
+    ("ragged_o6_ab3", lambda: W.wl_1d(19 * 10500, 10500, 6, 3, 0, 634, (1, 2), r_alpha=0.01, tsteps=3)[0]),
+    ("ragged_o4_unsplit", lambda: W.wl_1d(200001, 1, 4, 3, 0, 635, (1, 2))[0]),
+    ("ragged_burgers_ab2_o4", lambda: dict(W.wl_1d(131 * 1600, 1600, 4, 3, 0, 636, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
     ("3d_o2", lambda: W.wl_3d([24, 20, 18], [2, 2, 3], 2, 3, 0, 612, c=(0.3, 0.2, 0.1))[0]),
     ("3d_o4", lambda: W.wl_3d([72, 18, 20], [2, 1, 2], 4, 3, 0, 613, c=(0.3, 0.2, 0.1))[0]),
     ("3d_o4_ragged", lambda: W.wl_3d([39, 22, 14], [3, 2, 1], 4, 3, 0, 614, c=(0.3, 0.2, 0.1))[0]),
@@ -132,6 +139,10 @@ SMALL = [
     ("n2048_o6_ab3", lambda: W.wl_1d(2048, 64, 6, 3, 0, 644, (1, 2), r_alpha=0.01, tsteps=3)[0]),
     ("n1288_o4_ab2_unsplit", lambda: W.wl_1d(1288, 1, 4, 3, 0, 645, (1, 2), r_alpha=0.02, tsteps=2)[0]),
     ("n640_o4_burgers", lambda: dict(W.wl_1d(640, 10, 4, 3, 0, 646, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
+    ("n250_o4_points", lambda: W.wl_1d(250, 5, 4, 3, 0, 648, (1, 2))[0]),
+    ("n1001_o6_ab3_points", lambda: W.wl_1d(1001, 7, 6, 3, 0, 649, (1, 2), r_alpha=0.01, tsteps=3)[0]),
+    ("n102_burgers_points", lambda: dict(W.wl_1d(102, 6, 2, 3, 0, 650, (1, 2), c=0.0, r_alpha=0.02)[0], burgers=1)),
+    ("n63_space_points", lambda: W.wl_1d(63, 9, 2, 3, 0, 651, (1, 2), scheme=W.AT_SPACE2)[0]),
     ("n640_space", lambda: W.wl_1d(640, 10, 2, 3, 0, 647, (1, 2), scheme=W.AT_SPACE2)[0]),
 ]
 
