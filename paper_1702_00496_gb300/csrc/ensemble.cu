@@ -43,6 +43,7 @@ struct MemberParams {
   // the same modes prepared for the recurrences over k (when ms_ic.rot), exactly as the single-problem path
   // prepares them, so a member's fields and statistics carry the same bits: t = 0, t_final, t = -dt, -2 dt
   ModeSet ms_ic, ms_fin, ms_pre[2];
+  ModeTable mt;                    // the same offsets at every time (the modes' order does not change)
 };
 
 constexpr int kStatFields = AT_STAT_FIELDS;
@@ -53,6 +54,21 @@ __device__ double wave_1d(const MemberParams &m, const ModeSet &ms, const double
   double s = 0.0;
   for (int q = 0; q < m.nmodes; ++q) s += amp[q] * sin(m.kappa[q] * (x - shift) + m.phase[q]);
   return s;
+}
+
+// The field of the modes ms at every point, by the block: in runs of 16 points as the single-problem path, or point by point.
+__device__ void member_field(const MemberParams &m, const ModeSet &ms, const double *amp, double shift, double *out) {
+  const int N = m.p.n[0];
+  if (!m.mt.on) {
+    for (int i = threadIdx.x; i < N; i += blockDim.x) out[i] = wave_1d(m, ms, amp, shift, i);
+    return;
+  }
+  for (int c = threadIdx.x; c < (N + 15) >> 4; c += blockDim.x) {
+    double v[16];
+    atfd::mode_run(ms, m.mt, m.nmodes, (double)(16 * (int64_t)c + 8) * m.xpi, v);
+    for (int j = 0; j < 16; j += 2)  // N is a multiple of 4
+      if (16 * c + j < N) *reinterpret_cast<double2 *>(out + 16 * c + j) = make_double2(v[j], v[j + 1]);
+  }
 }
 
 // Adams-Bashforth pre-history of a realization (the same start as a single problem): dt f of the analytic
@@ -66,7 +82,7 @@ __device__ void member_prehistory(MemberParams &m) {
   __syncthreads();
   if (threadIdx.x == 0) m.p.use_pe[0] = 0;
   for (int mm = 1; mm <= ns; ++mm) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tmp[i] = wave_1d(m, m.ms_pre[mm - 1], m.amp_pre[mm - 1], m.shift_pre[mm - 1], i);
+    member_field(m, m.ms_pre[mm - 1], m.amp_pre[mm - 1], m.shift_pre[mm - 1], tmp);
     __syncthreads();
     double *out = m.p.frhs + (int64_t)(((-mm) % ns + ns) % ns) * m.p.ntot;
     for (int k = threadIdx.x; k < (N >> 2); k += blockDim.x) {
@@ -130,7 +146,7 @@ __global__ void __launch_bounds__(1024, 1) ensemble_kernel(const MemberParams *_
     }
     __syncthreads();
     const int N = m.p.n[0];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) m.p.ring[i] = wave_1d(m, m.ms_ic, m.amp, 0.0, i);
+    member_field(m, m.ms_ic, m.amp, 0.0, m.p.ring);
     __syncthreads();
     if (AB && m.p.ts > 1) {
       if (m.p.h == 1) member_prehistory<1>(m);
@@ -149,8 +165,14 @@ __global__ void __launch_bounds__(1024, 1) ensemble_kernel(const MemberParams *_
     double acc[kStatFields];
 #pragma unroll
     for (int f = 0; f < kStatFields; ++f) acc[f] = 0.0;
+    // u_a goes through the ring slot after the final level's (its levels are not read any more)
+    double *sol = m.p.ring + (m.steps + 1) % m.p.R * m.p.ntot;
+    if (m.mt.on) {
+      member_field(m, m.ms_fin, m.amp_final, m.shift_final, sol);
+      __syncthreads();
+    }
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const double ua = wave_1d(m, m.ms_fin, m.amp_final, m.shift_final, i);
+      const double ua = m.mt.on ? sol[i] : wave_1d(m, m.ms_fin, m.amp_final, m.shift_final, i);
       const int pos = i % m.p.S[0];
       const bool inB = m.p.use_pe[0] && (pos < m.p.h || pos >= m.p.S[0] - m.p.h);
       const double e = u[i] - ua;
@@ -400,6 +422,7 @@ extern "C" int at_ensemble_create(const at_config_t *members, const at_member_t 
     fill_modes(&m.ms_fin, m.amp, m.phase, m.kappa, c.nmodes, c.alpha, c.c[0], tf);
     for (int mm = 1; mm <= 2; ++mm)
       fill_modes(&m.ms_pre[mm - 1], m.amp, m.phase, m.kappa, c.nmodes, c.alpha, c.c[0], -(double)mm * c.dt);
+    fill_mode_table(&m.mt, m.ms_ic, c.nmodes, c.n[0]);
     m.group = groups[key_of(r)];
     m.steps = nsteps;
     m.twin = runs[r].twin;

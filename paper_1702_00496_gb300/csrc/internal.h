@@ -136,6 +136,14 @@ struct ModeSet {
 void fill_modes(ModeSet *ms, const double *amp, const double *phase, const double *kappa, int nmodes, double alpha,
                 double c, double t);
 
+// cos and sin of k_q j dx, j = 1 .. 8, for the modes in ModeSet's order (sorted by wavenumber): the offsets of a run of 16
+// grid points from its ninth.  on = 1 when the modes run by recurrences and the grid is long enough for runs (1D).
+struct ModeTable {
+  int32_t on;
+  double cs[AT_MAX_MODES][8][2];
+};
+void fill_mode_table(ModeTable *t, const ModeSet &ms, int nmodes, int64_t n);
+
 // Initial-condition / analytic-solution parameters.
 struct WaveParams {
   int32_t dim, nmodes;
@@ -148,6 +156,7 @@ struct WaveParams {
   double kappa[3][AT_MAX_MODES];
   ModeSet ms[3];  // per axis, filled by the launchers for the time of the launch (fill_modes)
   double xpi[3];  // 2 / n: grid point i sits at x = pi (i xpi)
+  ModeTable mt;   // 1D: filled with ms
 };
 
 // Validate cfg and fill the step parameters (merged taps, extrapolation weights, delay process) for a problem

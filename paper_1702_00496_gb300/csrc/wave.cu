@@ -32,6 +32,8 @@ WaveParams at_time(const WaveParams &w0, double t) {
     if (a < w.dim) fill_modes(&w.ms[a], w0.amp[a], w0.phase[a], w0.kappa[a], w.nmodes, w0.alpha, w0.c[a], t);
     else w.ms[a].rot = 0;
   }
+  w.mt.on = 0;
+  if (w.dim == 1) fill_mode_table(&w.mt, w.ms[0], w.nmodes, w.n[0]);
   for (int a = 0; a < w.dim; ++a)
     for (int q = 0; q < w.nmodes; ++q)
       if (t != 0.0) w.amp[a][q] = w0.amp[a][q] * std::exp(-w0.alpha * w0.kappa[a][q] * w0.kappa[a][q] * t);
@@ -52,6 +54,24 @@ __global__ void field_1d_kernel(const WaveParams w, double t, double *out) {
     out[i] = axis_sum(w, 0, (int)i, t);
 }
 
+// The same in runs of 16 points (w.mt.on).
+__global__ void __launch_bounds__(256) field_runs_kernel(const WaveParams w, double *out) {
+  const int n = w.n[0], runs = (n + 15) >> 4;
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < runs; c += gridDim.x * blockDim.x) {
+    double v[16];
+    atfd::mode_run(w.ms[0], w.mt, w.nmodes, (double)(16 * (int64_t)c + 8) * w.xpi[0], v);
+    double *o = out + 16 * (int64_t)c;
+    if (16 * c + 16 <= n && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+#pragma unroll
+      for (int j = 0; j < 16; j += 2) *reinterpret_cast<double2 *>(o + j) = make_double2(v[j], v[j + 1]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (16 * c + j < n) o[j] = v[j];
+    }
+  }
+}
+
 __global__ void field_3d_kernel(const WaveParams w, const double *tables, double *out) {
   const int64_t nx = w.n[0], ny = w.n[1], ntot = nx * ny * w.n[2];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ntot; i += (int64_t)gridDim.x * blockDim.x) {
@@ -59,6 +79,25 @@ __global__ void field_3d_kernel(const WaveParams w, const double *tables, double
     const int x = (int)(i - yz * nx), z = (int)(yz / ny), y = (int)(yz - z * ny);
     out[i] = tables[x] * tables[w.n[0] + y] * tables[w.n[0] + w.n[1] + z];
   }
+}
+
+// The block's sums of acc (field 1: its largest value) to partials[blockIdx.x]; 256 threads.
+__device__ void block_partials(const double acc[AT_STAT_FIELDS], double *partials) {
+  __shared__ double red[AT_STAT_FIELDS][256];
+#pragma unroll
+  for (int f = 0; f < AT_STAT_FIELDS; ++f) red[f][threadIdx.x] = acc[f];
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) {
+#pragma unroll
+      for (int f = 0; f < AT_STAT_FIELDS; ++f) {
+        const double o = red[f][threadIdx.x + s];
+        red[f][threadIdx.x] = (f == 1) ? ((o != o) ? o : fmax(red[f][threadIdx.x], o)) : red[f][threadIdx.x] + o;
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < AT_STAT_FIELDS) partials[(int64_t)blockIdx.x * AT_STAT_FIELDS + threadIdx.x] = red[threadIdx.x][0];
 }
 
 // REF = false: E = U - u_a with u_a the analytic solution at time t; REF = true: E = U - V with V a reference field
@@ -101,21 +140,53 @@ __global__ void __launch_bounds__(256) stats_partial_kernel(const WaveParams w, 
     acc[6] += ua * ua;
     if (e != e) acc[1] = e;  // keep a NaN visible through the max
   }
-  __shared__ double red[AT_STAT_FIELDS][256];
+  block_partials(acc, partials);
+}
+
+// E = U - u_a in 1D, u_a in runs of 16 points (w.mt.on).  Five FP64 operations per point beside u_a's: the largest |E| is
+// found on the bits (a NaN's are above infinity's, so it stays visible), the sets are counted in integers, and the sum
+// over all points is that over the two sets.
+__global__ void __launch_bounds__(256) stats_runs_kernel(const WaveParams w, const StepParams p, const double *u,
+                                                         double *partials) {
+  const int n = w.n[0], runs = (n + 15) >> 4, S = p.S[0], h = p.h;
+  const bool split = p.use_pe[0] != 0, aligned = (reinterpret_cast<uintptr_t>(u) & 15) == 0;
+  double abs1 = 0.0, sum1 = 0.0, in2 = 0.0, bd2 = 0.0, ua2 = 0.0;
+  int64_t in = 0, bd = 0;
+  unsigned long long top = 0;
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < runs; c += gridDim.x * blockDim.x) {
+    double v[16], x[16];
+    const int64_t i0 = 16 * (int64_t)c;
+    const int valid = n - (int)i0 < 16 ? n - (int)i0 : 16;
+    if (valid == 16 && aligned) {
 #pragma unroll
-  for (int f = 0; f < AT_STAT_FIELDS; ++f) red[f][threadIdx.x] = acc[f];
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-#pragma unroll
-      for (int f = 0; f < AT_STAT_FIELDS; ++f) {
-        const double o = red[f][threadIdx.x + s];
-        red[f][threadIdx.x] = (f == 1) ? ((o != o) ? o : fmax(red[f][threadIdx.x], o)) : red[f][threadIdx.x] + o;
+      for (int j = 0; j < 16; j += 2) {
+        const double2 a = *reinterpret_cast<const double2 *>(u + i0 + j);
+        x[j] = a.x; x[j + 1] = a.y;
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) x[j] = u[i0 + (j < valid ? j : 0)];
     }
-    __syncthreads();
+    atfd::mode_run(w.ms[0], w.mt, w.nmodes, (double)(i0 + 8) * w.xpi[0], v);
+    int pos = split ? (int)i0 % S : h;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j < valid) {
+        const double e = x[j] - v[j];
+        const bool inB = split && (pos < h || pos >= S - h);
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(e) & 0x7fffffffffffffffull;
+        top = bits > top ? bits : top;
+        abs1 += fabs(e);
+        sum1 += e;
+        if (inB) { bd2 = fma(e, e, bd2); ++bd; } else { in2 = fma(e, e, in2); ++in; }
+        ua2 = fma(v[j], v[j], ua2);
+      }
+      if (split && ++pos == S) pos = 0;
+    }
   }
-  if (threadIdx.x < AT_STAT_FIELDS) partials[(int64_t)blockIdx.x * AT_STAT_FIELDS + threadIdx.x] = red[threadIdx.x][0];
+  double acc[AT_STAT_FIELDS] = {in2 + bd2, __longlong_as_double((long long)top), abs1, sum1, in2, bd2, ua2, (double)in,
+                                (double)bd};
+  block_partials(acc, partials);
 }
 
 __global__ void __launch_bounds__(AT_STAT_BLOCKS) stats_final_kernel(const double *partials, double *result) {
@@ -162,9 +233,24 @@ void fill_modes(ModeSet *ms, const double *amp, const double *phase, const doubl
   }
 }
 
+void fill_mode_table(ModeTable *t, const ModeSet &ms, int nmodes, int64_t n) {
+  // runs of 16 points leave short grids to too few threads
+  t->on = ms.rot && n >= 4096 ? 1 : 0;
+  if (!t->on) return;
+  for (int q = 0; q < nmodes; ++q)
+    for (int j = 0; j < 8; ++j) {
+      const double a = 6.283185307179586476925286766559005768 * (double)(ms.kr[q] * (j + 1)) / (double)n;
+      t->cs[q][j][0] = std::cos(a);
+      t->cs[q][j][1] = std::sin(a);
+    }
+}
+
 cudaError_t launch_wave_field(const WaveParams &w0, double t, double *tables, double *out, cudaStream_t st) {
   const WaveParams w = at_time(w0, t);
-  if (w.dim == 1) {
+  if (w.dim == 1 && w.mt.on) {
+    const int blocks = ((w.n[0] + 15) / 16 + 255) / 256;
+    field_runs_kernel<<<blocks < 152 * 16 ? blocks : 152 * 16, 256, 0, st>>>(w, out);
+  } else if (w.dim == 1) {
     const int64_t blocks = (w.n[0] + 255) / 256;
     field_1d_kernel<<<(int)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, st>>>(w, t, out);
   } else {
@@ -179,7 +265,9 @@ cudaError_t launch_wave_field(const WaveParams &w0, double t, double *tables, do
 cudaError_t launch_error_stats(const WaveParams &w0, const StepParams &p, const double *u, double t, double *tables,
                                double *partials, double *result, cudaStream_t st) {
   const WaveParams w = at_time(w0, t);
-  if (w.dim == 1) {
+  if (w.dim == 1 && w.mt.on) {
+    stats_runs_kernel<<<AT_STAT_BLOCKS, 256, 0, st>>>(w, p, u, partials);
+  } else if (w.dim == 1) {
     stats_partial_kernel<1, false><<<AT_STAT_BLOCKS, 256, 0, st>>>(w, p, u, t, tables, partials, nullptr, 1);
   } else {
     axis_table_kernel<<<8, 256, 0, st>>>(w, t, tables);
