@@ -774,6 +774,9 @@ bool adjoint_grouped(const AdjParams &a) {
 // and last): with x0 a multiple of 4 and h <= 3, x0 >= h implies x0 >= W and x0 + 3 + h < n implies
 // x0 + 3 + W < n, so the two definitions agree.
 cudaError_t launch_adjoint_step(const AdjParams &a, int64_t n, int nblk, cudaStream_t st) {
+  cudaError_t be = cudaSuccess;
+  if (a.f.dim == 3 && launch_adjoint_brick(a.f, a.akeff, a.lam, a.Rl, a.reach, a.mu, a.alpha != 0, a.g_blk, nblk, n, st, &be))
+    return be;
   const bool grouped = adjoint_grouped(a);
   if (a.f.dim == 1) {
     if (a.f.h == 1) launch_alpha<1, 1>(a, n, nblk, grouped, st);

@@ -19,6 +19,11 @@
 //    the march: done in place, one such group held its block's barrier for 52 DFMA (256^3: 411 us per step against 242
 //    without any).
 //
+// The backward sweep of the gradient runs on the same tiles: the transposed step's level-n part (taps reversed, cells
+// across a face counted only at delay 0), the alpha term (second-derivative taps of U^n times lambda, summed), and a
+// small kernel for what the cells at the faces send to older levels.  256^3 in 4^3 PEs, order 4: 1.01 -> 0.63 ms per
+// backward step with the alpha term, 0.52 -> 0.37 ms without.
+//
 // What bounds it: the issue of the integer pipes (at order 4 39 multiply-adds per point, 22 instructions for 1.4
 // conversions, 25 for the rounding, the rest addresses and control) and the barrier.  512^3 in 8^3 PEs, L = 3 on GB300:
 // order 4 3.51 -> 1.43 ms per step, order 2 1.83 -> 0.96 ms; 256^3 in 4^3 PEs 453 -> 247 and 236 -> 160 us.
@@ -50,25 +55,67 @@ struct BrickShape {
   int64_t blocks;
 };
 
-template <int H, int AB>
-__global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_kernel(const StepParams p, const BrickShape b,
-                                                                         const int64_t n_off, const int64_t *n_base) {
+// What the backward step's passes read and write beside the step parameters.
+struct BrickAdjoint {
+  const double *src;    // MODE 1: the field the transposed taps act on (lambda^{n+1}, or mu); MODE 2: the same, as a factor
+  const double *ident;  // MODE 1, Adams-Bashforth: lambda^{n+1}, which reaches lambda^n unchanged; else null
+  double *cur;          // MODE 1: lambda^n
+  double *fresh;        // MODE 1: the level this step initialises (zeros), or null
+  double *g_blk;        // MODE 2: per-block sums of dJ/dalpha
+  int32_t add;          // MODE 1: add to cur (else set it)
+};
+
+// One point of the transposed step's level-n part as an FMA chain: p.s holds the taps reversed, p.s0 the centre; a
+// neighbour across a face with a delay (kn: the delays of the neighbours' sides) contributes to older levels instead.
+template <int H>
+__device__ __noinline__ double transposed_point(const StepParams &p, const double *__restrict__ src, const int pidx[3],
+                                                const int kn[3][2], const int c[3]) {
+  const int64_t stride[3] = {1, (int64_t)p.n[0], (int64_t)p.n[0] * p.n[1]};
+  const int64_t i = c[2] * stride[2] + c[1] * stride[1] + c[0];
+  double acc = fma(p.s0, LdgNC::ld(src + i), p.zero);
+  for (int a = 0; a < 3; ++a) {
+    const int pos = c[a] - pidx[a] * p.S[a];
+    for (int j = -H; j <= H; ++j) {
+      if (j == 0) continue;
+      if (p.use_pe[a] && ((pos + j < 0 && kn[a][0] > 0) || (pos + j >= p.S[a] && kn[a][1] > 0))) continue;
+      const int cj = wrap_coord(c[a] + j, p.n[a]);
+      acc = fma(p.s[a][j + H], LdgNC::ld(src + i + (int64_t)(cj - c[a]) * stride[a]), acc);
+    }
+  }
+  return acc;
+}
+
+// MODE 0: the forward step.  MODE 1: the part of the transposed step that stays at level n, with the taps reversed; a
+// buffer point counts only where the neighbour's side that reads across has delay 0.  MODE 2: the alpha term's sum of
+// lambda x (the second-derivative taps of U^n), for which p.s0, p.s and p.f3 hold those taps; each block takes the same
+// tiles in the same order, so the sum is deterministic.
+template <int H, int AB, int MODE>
+__global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(const StepParams p, const BrickShape b,
+                                                                            const BrickAdjoint adj, const int64_t n_off,
+                                                                            const int64_t *n_base) {
   constexpr int NR = 2 * H + 2;  // ring planes
   extern __shared__ int2 ring[];
   __shared__ int mx[3], pm[8], later[kBrickLater], n_later;
   const int64_t n = n_off + (n_base ? *n_base : 0);
-  const double *__restrict__ un = p.ring + slot_of(n, p.R) * p.ntot;
-  double *__restrict__ out = p.ring + slot_of(n + 1, p.R) * p.ntot;
+  const double *__restrict__ un = MODE == 1 ? adj.src : p.ring + slot_of(n, p.R) * p.ntot;
+  double *__restrict__ out = MODE == 1 ? adj.cur : p.ring + slot_of(n + 1, p.R) * p.ntot;
   const uint8_t *keff = p.keff + (n & 1) * p.nb;
   const int tid = threadIdx.x;
-  draw_sides(p, n + 1, (int64_t)blockIdx.x * kBrickThreads + tid, (int64_t)gridDim.x * kBrickThreads,
-             p.keff + ((n + 1) & 1) * p.nb);
+  if (MODE == 0) {
+    draw_sides(p, n + 1, (int64_t)blockIdx.x * kBrickThreads + tid, (int64_t)gridDim.x * kBrickThreads,
+               p.keff + ((n + 1) & 1) * p.nb);
+  } else if (MODE == 1 && n >= 1) {
+    draw_sides(p, n - 1, (int64_t)blockIdx.x * kBrickThreads + tid, (int64_t)gridDim.x * kBrickThreads,
+               p.keff + ((n - 1) & 1) * p.nb);
+  }
+  double galpha = 0.0;
   const int nx = p.n[0], ny = p.n[1], nz = p.n[2], sn = (int)slot_of(n, p.R);
   const int64_t nxy = (int64_t)nx * ny;
+  for (int64_t tile = blockIdx.x; tile < b.blocks; tile += gridDim.x) {
   // tile: x fastest, then y, then chunk, then PE
   int pidx[3], x0, y0, zs, ze;
   {
-    int t = blockIdx.x;
+    int t = (int)tile;
     const int tx = t % b.tiles_x; t /= b.tiles_x;
     const int ty = t % b.tiles_y; t /= b.tiles_y;
     const int ch = t % b.chunks; t /= b.chunks;
@@ -86,8 +133,14 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
   int kside[3][2];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    kside[a][0] = p.use_pe[a] ? keff[side_of<3>(p, pidx, a, 0)] : 0;
-    kside[a][1] = p.use_pe[a] ? keff[side_of<3>(p, pidx, a, 1)] : 0;
+    // the PE's own sides; transposed: the side of the neighbour across each face that reads this PE's cells
+    int lo[3] = {pidx[0], pidx[1], pidx[2]}, hi[3] = {pidx[0], pidx[1], pidx[2]};
+    if (MODE == 1) {
+      lo[a] = pidx[a] == 0 ? p.pe[a] - 1 : pidx[a] - 1;
+      hi[a] = pidx[a] + 1 == p.pe[a] ? 0 : pidx[a] + 1;
+    }
+    kside[a][0] = p.use_pe[a] ? keff[side_of<3>(p, lo, a, MODE == 1 ? 1 : 0)] : 0;
+    kside[a][1] = p.use_pe[a] ? keff[side_of<3>(p, hi, a, MODE == 1 ? 0 : 1)] : 0;
   }
   // This thread's share of a plane's cells: kCore slots of the tile's own cells, row by row, then the cells around it --
   // left and right of the rows, then below and above them -- so that the buffer points, which cost T FP64 operations
@@ -133,7 +186,7 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
     const double *src = un + base;
 #pragma unroll
     for (int s = 0; s < kBrickSlots; ++s) v[s] = LdgNC::ld(src + goff[s]);
-    if (some) {
+    if (MODE != 1 && some) {
 #pragma unroll
       for (int s = kCore; s < kBrickSlots; ++s) {
         const int k = code[s] >> 16;
@@ -148,7 +201,11 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
   };
   auto extrapolate = [&](int zz) {
     const int kz = zz < pz0 ? kside[2][0] : (zz >= pz1 ? kside[2][1] : 0);
-    if (kz > 0) {  // a buffer plane: only the tile's own cells of it are read
+    if (MODE == 1) {  // what lies across a face with a delay goes to older levels (brick_faces_kernel)
+#pragma unroll
+      for (int s = 0; s < kBrickSlots; ++s)
+        if (s < kCore ? kz > 0 : (code[s] >> 16) > 0) v[s] = 0.0;
+    } else if (kz > 0) {  // a buffer plane: only the tile's own cells of it are read
       const int64_t base = (int64_t)wrap_coord(zz, nz) * nxy;
 #pragma unroll
       for (int s = 0; s < kCore; ++s) v[s] = halo_value<LdgNC>(p, base + goff[s], sn, kz);
@@ -180,7 +237,15 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
   const int64_t cell0 = (int64_t)(y0 + row) * nx + x0 + 4 * grp;
   // the FP64 chain for group g of tile row rr of plane o
   auto chain = [&](int rr, int g, int o, double r[4]) {
-    if (b.aligned) {
+    if (MODE == 1) {
+      const int valid = min(4, xlen - 4 * g);
+#pragma unroll 1
+      for (int q = 0; q < valid; ++q) {
+        const int c[3] = {x0 + 4 * g + q, y0 + rr, o};
+        const double w = transposed_point<H>(p, un, pidx, kside, c);
+        r[0] = q == 0 ? w : r[0]; r[1] = q == 1 ? w : r[1]; r[2] = q == 2 ? w : r[2]; r[3] = q == 3 ? w : r[3];
+      }
+    } else if (b.aligned) {
       double uc[4];
       group_eval<3, H, LdgNC, false>(p, keff, un, n, x0 + 4 * g, y0 + rr, o, r, uc);
     } else {
@@ -196,6 +261,41 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
   };
   // Adams-Bashforth combination and store of `valid` points from i0
   auto finish = [&](int64_t i0, int valid, double r[4], const AbLevels<1> old[4]) {
+    if (MODE == 2) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < valid) galpha = fma(LdgNC::ld(adj.src + i0 + q), r[q], galpha);
+      return;
+    }
+    if (MODE == 1 && b.aligned) {  // the workspace is 16-byte aligned
+      double2 *o = reinterpret_cast<double2 *>(out + i0);
+      double2 lo = make_double2(r[0], r[1]), hi = make_double2(r[2], r[3]);
+      if (adj.ident) {
+        const double2 a = LdgNC::ld2(adj.ident + i0), c = LdgNC::ld2(adj.ident + i0 + 2);
+        lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
+      }
+      if (adj.add) {
+        const double2 a = o[0], c = o[1];
+        lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
+      }
+      o[0] = lo;
+      o[1] = hi;
+      if (adj.fresh) {
+        double2 *z = reinterpret_cast<double2 *>(adj.fresh + i0);
+        z[0] = z[1] = make_double2(0.0, 0.0);
+      }
+      return;
+    }
+    if (MODE == 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (q >= valid) continue;
+        if (adj.ident) r[q] += LdgNC::ld(adj.ident + i0 + q);
+        out[i0 + q] = adj.add ? out[i0 + q] + r[q] : r[q];
+        if (adj.fresh) adj.fresh[i0 + q] = 0.0;
+      }
+      return;
+    }
     if (AB) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -242,7 +342,7 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
           const int g0 = (c4[0].x ^ (c4[0].x >> 31)) | (c4[1].x ^ (c4[1].x >> 31));
           int g1 = (c4[2].x ^ (c4[2].x >> 31)) | (c4[3].x ^ (c4[3].x >> 31));
           g1 = nv < 3 ? g0 : g1;
-          far = (min(g0, g1) >> (29 - kBrickGuard)) == 0;
+          far = MODE != 2 && (min(g0, g1) >> (29 - kBrickGuard)) == 0;  // a sum over all points needs no local bits
         }
         int64_t A[4], B[4], C[4];
         const FxTaps<6 * AT_MAX_H + 1> &t = p.f3;
@@ -366,6 +466,94 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) forward_brick_ker
     chain(rr, g, o, r);
     finish(i0, valid, r, old);
   }
+  __syncthreads();
+  }
+  if (MODE == 2) {
+    __shared__ double sums[kBrickThreads / 32];  // block sum in a fixed order
+    for (int d = 16; d > 0; d >>= 1) galpha += __shfl_down_sync(0xffffffffu, galpha, d);
+    if ((tid & 31) == 0) sums[tid >> 5] = galpha;
+    __syncthreads();
+    if (tid == 0) {
+      double t = sums[0];
+      for (int w = 1; w < kBrickThreads / 32; ++w) t += sums[w];
+      adj.g_blk[blockIdx.x] += t;
+    }
+  }
+}
+
+// The part of the transposed step that goes to older levels: a cell within h of a face whose far side's reader has delay
+// k > 0 sends sum_j s_j lambda_{c-j} over the taps that cross, times w_m(k), to level n-k-m.  One thread per such cell
+// (they are enumerated once each, face_cell), all its axes in turn.
+// (A problem has fewer than 2^31 points: 32-bit divisions.)
+struct FaceBoxes {
+  uint32_t part_z, part_y, total;  // cells near a z face; near a y face but no z face; near an x face only
+  uint32_t cs[3], cc[3];           // coordinates near a face and elsewhere, per axis
+  int32_t hw[3];
+};
+
+__device__ __forceinline__ int near_face(const StepParams &p, int a, int hw, uint32_t t) {
+  const uint32_t w = 2 * hw, pe = t / w;
+  const int r = (int)(t - pe * w);
+  return (int)pe * p.S[a] + (r < hw ? r : p.S[a] - (int)w + r);
+}
+__device__ __forceinline__ int off_face(const StepParams &p, int a, int hw, uint32_t t) {
+  if (hw == 0) return (int)t;
+  const uint32_t w = p.S[a] - 2 * hw, pe = t / w;
+  return (int)(pe * (uint32_t)p.S[a] + hw + (t - pe * w));
+}
+
+template <int H>
+__global__ void __launch_bounds__(256) brick_faces_kernel(const StepParams p, const FaceBoxes m, const double *__restrict__ src,
+                                                          double *lam, const int Rl, const int64_t n) {
+  const uint8_t *keff = p.keff + (n & 1) * p.nb;
+  const int snl = (int)slot_of(n, Rl);
+  const int64_t stride[3] = {1, (int64_t)p.n[0], (int64_t)p.n[0] * p.n[1]};
+  const uint32_t nx = p.n[0], ny = p.n[1];
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < m.total; e += gridDim.x * blockDim.x) {
+    int c[3];
+    if (e < m.part_z) {
+      const uint32_t row = e / nx, lay = row / ny;
+      c[0] = (int)(e - row * nx);
+      c[1] = (int)(row - lay * ny);
+      c[2] = near_face(p, 2, m.hw[2], lay);
+    } else if (e - m.part_z < m.part_y) {
+      const uint32_t k = e - m.part_z, row = k / nx, lay = row / m.cs[1];
+      c[0] = (int)(k - row * nx);
+      c[1] = near_face(p, 1, m.hw[1], row - lay * m.cs[1]);
+      c[2] = off_face(p, 2, m.hw[2], lay);
+    } else {
+      const uint32_t k = e - m.part_z - m.part_y, r = k / m.cs[0], lay = r / m.cc[1];
+      c[0] = near_face(p, 0, m.hw[0], k - r * m.cs[0]);
+      c[1] = off_face(p, 1, m.hw[1], r - lay * m.cc[1]);
+      c[2] = off_face(p, 2, m.hw[2], lay);
+    }
+    const int64_t i = c[2] * stride[2] + c[1] * stride[1] + c[0];
+    int pidx[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) pidx[a] = c[a] / p.S[a];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (!p.use_pe[a]) continue;
+      const int pos = c[a] - pidx[a] * p.S[a];
+      const bool lower = pos < H;
+      if (!lower && pos < p.S[a] - H) continue;
+      int nb[3] = {pidx[0], pidx[1], pidx[2]};
+      nb[a] = lower ? (pidx[a] == 0 ? p.pe[a] - 1 : pidx[a] - 1) : (pidx[a] + 1 == p.pe[a] ? 0 : pidx[a] + 1);
+      const int k = keff[side_of<3>(p, nb, a, lower ? 1 : 0)];
+      if (k == 0) continue;
+      double x = 0.0;
+#pragma unroll
+      for (int j = -H; j <= H; ++j) {  // reversed taps: tap j reads c + j
+        if (j == 0 || (pos + j >= 0 && pos + j < p.S[a])) continue;
+        const int cj = wrap_coord(c[a] + j, p.n[a]);
+        x = fma(p.s[a][j + H], LdgNC::ld(src + i + (int64_t)(cj - c[a]) * stride[a]), x);
+      }
+      for (int t = 0; t < p.T; ++t) {
+        double *o = lam + slot_back(snl, k + t, Rl) * p.ntot + i;
+        *o = fma(p.w[k][t], x, *o);
+      }
+    }
+  }
 }
 
 int brick_sms() {
@@ -437,24 +625,41 @@ bool brick_shape(const StepParams &p, BrickShape *b) {
   return b->blocks < (1ll << 31);
 }
 
-template <int H, int AB>
-cudaError_t launch_brick_typed(const StepParams &p, const BrickShape &b, int64_t n, const int64_t *n_base,
-                               cudaStream_t st) {
+template <int H, int AB, int MODE>
+cudaError_t launch_brick_typed(const StepParams &p, const BrickShape &b, const BrickAdjoint &adj, int64_t blocks, int64_t n,
+                               const int64_t *n_base, cudaStream_t st) {
   const int bytes = (2 * H + 2) * b.plane * 8;
-  auto kernel = forward_brick_kernel<H, AB>;
+  auto kernel = brick_kernel<H, AB, MODE>;
   if (bytes + 4096 > 48 * 1024) {  // with the static part
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
   }
-  kernel<<<(unsigned)b.blocks, kBrickThreads, bytes, st>>>(p, b, n, n_base);
+  kernel<<<(unsigned)blocks, kBrickThreads, bytes, st>>>(p, b, adj, n, n_base);
   return cudaGetLastError();
 }
 
-template <int AB>
-cudaError_t launch_brick_h(const StepParams &p, const BrickShape &b, int64_t n, const int64_t *n_base, cudaStream_t st) {
-  if (p.h == 1) return launch_brick_typed<1, AB>(p, b, n, n_base, st);
-  if (p.h == 2) return launch_brick_typed<2, AB>(p, b, n, n_base, st);
-  return launch_brick_typed<3, AB>(p, b, n, n_base, st);
+template <int AB, int MODE>
+cudaError_t launch_brick_h(const StepParams &p, const BrickShape &b, const BrickAdjoint &adj, int64_t blocks, int64_t n,
+                           const int64_t *n_base, cudaStream_t st) {
+  if (p.h == 1) return launch_brick_typed<1, AB, MODE>(p, b, adj, blocks, n, n_base, st);
+  if (p.h == 2) return launch_brick_typed<2, AB, MODE>(p, b, adj, blocks, n, n_base, st);
+  return launch_brick_typed<3, AB, MODE>(p, b, adj, blocks, n, n_base, st);
+}
+
+// p with the taps t (centre, then each axis in offset order) in place of the step's.
+void set_taps(StepParams *p, double s0, const double s[3][2 * AT_MAX_H + 1], bool reversed) {
+  const int h = p->h;
+  double t[6 * AT_MAX_H + 1] = {s0}, keep[3][2 * AT_MAX_H + 1];
+  int c = 1;
+  for (int a = 0; a < 3; ++a)
+    for (int j = -h; j <= h; ++j) {
+      keep[a][j + h] = s[a][reversed ? h - j : h + j];
+      if (j != 0) t[c++] = keep[a][j + h];
+    }
+  p->s0 = s0;
+  for (int a = 0; a < 3; ++a)
+    for (int j = 0; j <= 2 * h; ++j) p->s[a][j] = keep[a][j];
+  fx_prepare(t, c, &p->f3);
 }
 
 }  // namespace
@@ -462,6 +667,53 @@ cudaError_t launch_brick_h(const StepParams &p, const BrickShape &b, int64_t n, 
 bool launch_forward_brick(const StepParams &p, int64_t n, const int64_t *n_base, cudaStream_t st, cudaError_t *e) {
   BrickShape b;
   if (!brick_shape(p, &b)) return false;
-  *e = p.ts > 1 ? launch_brick_h<1>(p, b, n, n_base, st) : launch_brick_h<0>(p, b, n, n_base, st);
+  const BrickAdjoint none = {};
+  *e = p.ts > 1 ? launch_brick_h<1, 0>(p, b, none, b.blocks, n, n_base, st)
+                : launch_brick_h<0, 0>(p, b, none, b.blocks, n, n_base, st);
+  return true;
+}
+
+bool launch_adjoint_brick(const StepParams &f, uint8_t *akeff, double *lam, int Rl, int reach, const double *mu, bool alpha,
+                          double *g_blk, int nblk, int64_t n, cudaStream_t st, cudaError_t *e) {
+  BrickShape b;
+  if (!brick_shape(f, &b)) return false;
+  StepParams p = f;
+  p.keff = akeff;
+  const double *next = lam + (n + 1) % Rl * f.ntot, *src = mu ? mu : next;
+  if (alpha) {
+    // the second-derivative taps (no 1 in the centre), from the forward levels; before the next draws
+    StepParams q = p;
+    set_taps(&q, f.q0, f.q, false);
+    if (!q.f3.ok) return false;
+    BrickAdjoint a = {};
+    a.src = src;
+    a.g_blk = g_blk;
+    *e = launch_brick_h<0, 2>(q, b, a, b.blocks < nblk ? b.blocks : nblk, n, nullptr, st);
+    if (*e != cudaSuccess) return true;
+  }
+  set_taps(&p, f.s0, f.s, true);
+  BrickAdjoint a = {};
+  a.src = src;
+  a.ident = mu ? next : nullptr;
+  a.cur = lam + n % Rl * f.ntot;
+  a.add = reach > 0;
+  a.fresh = reach > 0 && n >= reach ? lam + (n - reach) % Rl * f.ntot : nullptr;
+  if ((*e = launch_brick_h<0, 1>(p, b, a, b.blocks, n, nullptr, st)) != cudaSuccess) return true;
+  FaceBoxes m;
+  for (int k = 0; k < 3; ++k) {
+    m.hw[k] = f.use_pe[k] ? f.h : 0;
+    m.cs[k] = f.use_pe[k] ? (uint32_t)(f.pe[k] * 2 * f.h) : 0;  // a PE is at least 2 h wide
+    m.cc[k] = f.n[k] - m.cs[k];
+  }
+  m.part_z = m.cs[2] * f.n[1] * f.n[0];
+  m.part_y = m.cc[2] * m.cs[1] * f.n[0];
+  m.total = m.part_z + m.part_y + m.cc[2] * m.cc[1] * m.cs[0];
+  if (m.total == 0 || f.scheme == AT_SYNC || reach == 0) return true;
+  const int64_t blocks = ((int64_t)m.total + 255) / 256, most = (int64_t)brick_sms() * 8;
+  const unsigned g = (unsigned)(blocks < most ? blocks : most);
+  if (f.h == 1) brick_faces_kernel<1><<<g, 256, 0, st>>>(p, m, src, lam, Rl, n);
+  else if (f.h == 2) brick_faces_kernel<2><<<g, 256, 0, st>>>(p, m, src, lam, Rl, n);
+  else brick_faces_kernel<3><<<g, 256, 0, st>>>(p, m, src, lam, Rl, n);
+  *e = cudaGetLastError();
   return true;
 }

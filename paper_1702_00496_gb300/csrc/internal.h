@@ -175,6 +175,12 @@ cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, c
 // 3D: the step in fixed point over tiles of the PEs (brick.cu); false: the shape or scheme is not one for it, nothing
 // launched.
 bool launch_forward_brick(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st, cudaError_t *e);
+// Backward step n of a 3D linear problem on the same tiles: the transposed step on the adjoint ring lam (Rl slots, levels
+// down to n - reach), with alpha the sum of dJ/dalpha's terms into g_blk (nblk sums); f: forward parameters whose ring
+// holds the levels the alpha term reads; akeff: the sweep's delay buffers (step n's in place, step n-1's drawn); mu:
+// Adams-Bashforth, else null.  false: not a shape for it, nothing launched.
+bool launch_adjoint_brick(const StepParams &f, uint8_t *akeff, double *lam, int Rl, int reach, const double *mu, bool alpha,
+                          double *g_blk, int nblk, int64_t n, cudaStream_t st, cudaError_t *e);
 // Largest block length K <= kmax (1: none) that the problem admits, and the block parameters for K (host).
 int fuse_max_k(const StepParams &p, const void *ring, int kmax);
 void fuse_setup(StepParams *p, int k);

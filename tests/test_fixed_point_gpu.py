@@ -167,3 +167,41 @@ def test_small_problems_in_one_launch_are_bitwise_single_steps(name, make, calle
         s.close()
     for u, d in runs[1:]:
         assert torch.equal(u, runs[0][0]) and torch.equal(d, runs[0][1])
+
+
+ADJOINT_TILES = [
+    ("o4_ragged", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 4, 3, 0, 661, c=(0.3, 0.2, 0.1))[0], False),
+    ("o2_aligned_unsplit_y", lambda: W.wl_3d([128, 128, 128], [2, 1, 2], 2, 4, 0, 662, c=(0.3, 0.2, 0.1))[0], False),
+    ("o6_std", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 6, 3, 0, 663, c=(0.3, 0.2, 0.1), scheme=W.ASYNC_STD,
+                               dt=0.01 * W.dx_of(150) ** 2 / 0.05)[0], False),
+    ("o4_ab2", lambda: W.wl_3d([128, 128, 128], [2, 2, 2], 4, 3, 0, 664, c=(0.3, 0.2, 0.1), tsteps=2,
+                               dt=0.02 * W.dx_of(128) ** 2 / 0.05)[0], True),
+]
+
+
+@pytest.mark.parametrize("name,make,callers_field", ADJOINT_TILES, ids=[c[0] for c in ADJOINT_TILES])
+def test_gradient_on_tiles_matches_the_cpu_adjoint(name, make, callers_field):
+    """The transposed step over the marched tiles (its level-n part, the faces' older levels, the alpha sum) against the
+    oracle's literal adjoint, with the bars of the other adjoint tests; and the initial field's gradient alone and other
+    checkpoint intervals give the same bits."""
+    from paper_1702_00496_gb300 import Solver
+    spec = make()
+    steps = 7
+    cfg = oracle.Config(spec)
+    u0 = oracle.initial(cfg) + (0.01 if callers_field else 0.0)
+    rng = np.random.default_rng(7)
+    target = 0.5 * u0 + 0.1 * rng.standard_normal(cfg.shape)
+    grads = []
+    for every, want_alpha in ((0, True), (steps, True), (2, False)):
+        s = Solver(spec)
+        s.reset(torch.as_tensor(u0, device="cuda"))
+        s.adjoint_forward(steps, every)
+        lam = s.field() - torch.as_tensor(target, device="cuda")
+        g, ga = s.adjoint_backward(lam.clone(), want_alpha)
+        grads.append((g.cpu().numpy(), ga))
+        s.close()
+    _, go, gao = oracle.adjoint(cfg, steps, target, u0=u0)
+    g, ga = grads[0]
+    assert np.linalg.norm(g - go) / np.linalg.norm(go) <= 1e-12
+    assert ga == pytest.approx(gao, rel=1e-10)
+    assert np.array_equal(grads[1][0], g) and grads[1][1] == ga and np.array_equal(grads[2][0], g)
