@@ -293,8 +293,9 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
       if (near) {
         block_sums<TK, C, true>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
       } else {
-        // every run of 8 cells must hold a value within kFxGuard bits of the tile's largest one
-        constexpr int G = C < 8 ? C : 8;
+        // every cell must have a value within kFxGuard bits of the tile's largest one in its own window of TK cells
+        // either side: two cells of each run are looked at, and no cell of the run is further than TK from either
+        constexpr int G = TK < 3 ? 2 : (C < 8 || TK < 6 ? 4 : 8);
 #pragma unroll
         for (int g = 0; g < C; g += G) {
           const int a = C * lane + TK + g + G / 8, b = C * lane + TK + g + G - 1 - G / 8;
