@@ -169,6 +169,7 @@ AT_FX_HD void fx_results(const int64_t R[N], int ex, double r[N]) {
 }
 
 // Weights of up to N taps; sw = 0 with ok = 0 when they cannot be represented (not finite, all zero, out of range).
+// w_low: what the weights have below their last bit (composed stencils), or null.
 // f1, f0: the same parts in FP32, in units of 2^3 of R, for sums whose cross terms go through the FP32 pipe.
 template <int N>
 struct FxTaps {
@@ -178,7 +179,7 @@ struct FxTaps {
 };
 
 template <int N>
-inline void fx_prepare(const double *w, int n, FxTaps<N> *t) {
+inline void fx_prepare(const double *w, int n, FxTaps<N> *t, const double *w_low = nullptr) {
   std::memset(t, 0, sizeof(*t));
   double sum = 0.0, big = 0.0;
   for (int i = 0; i < n; ++i) {
@@ -198,11 +199,17 @@ inline void fx_prepare(const double *w, int n, FxTaps<N> *t) {
   t->sw = 60 - k;
   for (int i = 0; i < n; ++i) {
     // w 2^sw exactly: sw is in 0..109
-    double v = w[i];
+    double v = w[i], vl = w_low ? w_low[i] : 0.0;
     int s = t->sw;
-    for (; s >= 60; s -= 60) v *= 1152921504606846976.0;
+    for (; s >= 60; s -= 60) {
+      v *= 1152921504606846976.0;
+      vl *= 1152921504606846976.0;
+    }
     v *= (double)(1ull << s);
-    const int64_t W = (int64_t)(v < 0 ? v - 0.5 : v + 0.5);
+    vl *= (double)(1ull << s);
+    const int64_t whole = (int64_t)v;
+    const double rest = (v - (double)whole) + vl;
+    const int64_t W = whole + (int64_t)(rest < 0 ? rest - 0.5 : rest + 0.5);
     const int64_t half = 1ll << (kFxLowBits - 1), mask = (1ll << kFxLowBits) - 1;
     const int64_t lo = ((W + half) & mask) - half;
     t->w0[i] = (int32_t)lo;

@@ -17,11 +17,16 @@
 // drawn from Philox (Sec. 5.1) keyed by (seed, step, side) once per step -- by the launch of the previous
 // step, into a double-buffered array -- and clamped so that no level before 0 is read.
 //
-// The kernel is bound by the FP64 pipe on GB300 (2 FP64 FMA lanes per SM per clock nominal; about 1.6 per
-// clock sustained for dependent FMA chains): each point costs the minimum 1 + 2 h dim FP64 operations, all of
-// them FMAs -- the chain starts with fma(s0, u_i, +0) on a runtime zero, because a DMUL occupies the FP64
-// pipe longer than a DFMA and the result is the same rounded product.
+// The FP64 pipe of GB300 does two FMAs per SM and clock, which bounded every step kernel at 9 to 25 % of the memory
+// rate while the sums were FP64 chains.  They are summed in block fixed point instead (fixed.cuh), three integer
+// multiply-adds of 16 lanes or more a clock per tap; windows the fixed point does not take are chains still: 1 + 2 h dim
+// FMAs per point, starting with fma(s0, u_i, +0) on a runtime zero (a DMUL occupies the pipe longer than a DFMA).
+//
+// Kernels of 1D: forward_block_kernel (K steps in one launch), forward_group_kernel (groups of four, one step),
+// forward_ragged_kernel (large shapes without aligned groups), forward_point_kernel (small ones); 3D: the marched tiles
+// (brick.cu) from the size on where they are faster, groups or points below; tiny 1D problems: small.cu.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "stencil.cuh"
@@ -408,6 +413,9 @@ cudaError_t launch_draw_delays(const StepParams &p, int64_t n, cudaStream_t st) 
 
 namespace {
 
+// 1D shapes without aligned groups of four from this many points on are summed in fixed point (launch_typed)
+constexpr int64_t kRaggedPoints = 196608;
+
 // groups of four x points must not straddle a PE and must start on 16 bytes
 bool grouped_shape(const StepParams &p, const void *base) {
   return p.n[0] % 4 == 0 && (!p.use_pe[0] || p.S[0] % 4 == 0) && (reinterpret_cast<uintptr_t>(base) % 16) == 0 &&
@@ -428,7 +436,7 @@ void launch_typed(const StepParams &p, bool grouped, int blocks, int threads, in
   constexpr int ABG = AB ? 1 : 0;
   // per step, tiny / per million points more, us: the per-point kernel 2.9 / 7.5 (order 2), 3.9 / 9.3 (order 4), 5.6 / 11.7
   // (order 6), 4.3 / 22 (AB2); groups in fixed point 3.1 / 4.6, 4.6 / 5.8, 6.4 / 6.6, 5.4 / 9.5
-  const bool ragged = p.ntot >= 196608;
+  const bool ragged = p.ntot >= kRaggedPoints;
   const int rblocks = (int)std::min<int64_t>((p.ntot / 2 + 255) / 256, (int64_t)sm_count() * 32);
   if (DIM == 1 && p.burgers) {
     if (grouped) forward_group_kernel<1, H, ABG, 1><<<blocks, threads, 0, st>>>(p, n, n_base);
@@ -544,7 +552,11 @@ static void fuse_radii(int h, int K, int *fe, int zr[]) {
 }
 
 int fuse_max_k(const StepParams &p, const void *ring, int kmax) {
-  if (p.dim != 1 || p.scheme > AT_AT || p.burgers || p.ts != 1 || !grouped_shape(p, ring)) return 1;
+  // The block kernel itself takes any PE width and alignment.  Small shapes without aligned groups of four run point by
+  // point, with one rounding per tap for any split of the steps; large ones take blocks like the others (750000 points in
+  // PEs of 250, order 4: 3.7 us per step in blocks of 4, 9.8 in single steps).
+  if (p.dim != 1 || p.scheme > AT_AT || p.burgers || p.ts != 1) return 1;
+  if (!grouped_shape(p, ring) && p.ntot < kRaggedPoints) return 1;
   for (int K = kmax < AT_MAX_FUSE ? kmax : AT_MAX_FUSE; K >= 2; --K) {
     if (p.R <= K) continue;  // U^n must stay in the ring while U^{n+K} is written
     int fe, zr[AT_MAX_FUSE];
@@ -574,20 +586,31 @@ void fuse_setup(StepParams *p, int k) {
   const int h = p->h;
   fuse_radii(h, k, &p->fe, p->zr);
   if (!p->use_pe[0]) p->fe = 0;
-  // K-fold composition of the merged taps (s0 at the centre), in a fixed order
-  double s[2 * AT_MAX_H + 1], c[2 * AT_MAX_H * AT_MAX_FUSE + 1] = {1.0}, t[2 * AT_MAX_H * AT_MAX_FUSE + 1];
+  // K-fold composition of the merged taps (s0 at the centre), in pairs of doubles: the fixed-point weights keep more bits
+  // than a double, and the roundings of a composition in doubles would pull every block the same way
+  constexpr int N = 2 * AT_MAX_H * AT_MAX_FUSE + 1;
+  double s[2 * AT_MAX_H + 1], c[N] = {1.0}, cl[N] = {0.0}, t[N], tl[N];
   for (int j = -h; j <= h; ++j) s[j + h] = j == 0 ? p->s0 : p->s[0][j + h];
-  int w = 0;  // c holds taps -w .. w at c[0 .. 2w]
+  int w = 0;  // c + cl holds taps -w .. w at 0 .. 2w
   for (int step = 0; step < k; ++step) {
     const int w2 = w + h;
-    for (int i = 0; i <= 2 * w2; ++i) t[i] = 0.0;
+    for (int i = 0; i <= 2 * w2; ++i) t[i] = tl[i] = 0.0;
     for (int i = 0; i <= 2 * w; ++i)
-      for (int j = 0; j <= 2 * h; ++j) t[i + j] += c[i] * s[j];
+      for (int j = 0; j <= 2 * h; ++j) {
+        const double m = c[i] * s[j], ml = std::fma(c[i], s[j], -m) + cl[i] * s[j];
+        double &sum = t[i + j];
+        const double next = sum + m, of_m = next - sum;
+        tl[i + j] += ((sum - (next - of_m)) + (m - of_m)) + ml;
+        sum = next;
+      }
     w = w2;
-    for (int i = 0; i <= 2 * w; ++i) c[i] = t[i];
+    for (int i = 0; i <= 2 * w; ++i) {
+      c[i] = t[i] + tl[i];
+      cl[i] = (t[i] - c[i]) + tl[i];
+    }
   }
   for (int i = 0; i <= 2 * w; ++i) p->ck[i] = c[i];
-  fx_prepare(p->ck, 2 * w + 1, &p->fck);
+  fx_prepare(p->ck, 2 * w + 1, &p->fck, cl);
 }
 
 cudaError_t launch_sync_rhs(const StepParams &p, const double *u, double *out, cudaStream_t st) {

@@ -7,10 +7,11 @@
 // that lies outside the group's PE (a buffer point, Sec. 2) by the halo value its PE side sees:
 //     u~ = sum_{m<T} w_m(k) U^{n-k-m}     (k: that side's effective delay for step n; k = 0 keeps U^n)
 // Groups never straddle a PE (PE widths are multiples of 4 on these paths), so each loaded value is either
-// inside the PE or a buffer point of exactly one side.  The update is then the same chain of FMAs for every
-// group:  r = fma(s0, u_i, +0), the taps of axis x in offset order, then axis y, then axis z.
+// inside the PE or a buffer point of exactly one side.  The update is then the same for every group: the taps of
+// all axes summed in block fixed point (fixed.cuh: exact, one rounding), or, where a window does not fit that, the chain
+//     r = fma(s0, u_i, +0), the taps of axis x in offset order, then axis y, then axis z.
 //
-// With Adams-Bashforth time stepping (Sec. 4.1, Eq. "time_disc" with two or three levels) the same chain,
+// With Adams-Bashforth time stepping (Sec. 4.1, Eq. "time_disc" with two or three levels) the same sum,
 // without the 1 in s0, gives dt f^n; the update adds the stored dt f^{n-1}, dt f^{n-2} with their weights and
 // keeps dt f^n in place of the oldest one.
 //

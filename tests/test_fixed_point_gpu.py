@@ -36,6 +36,12 @@ PROBLEMS = [
     ("ragged_o2", lambda: W.wl_1d(197 * 1001, 1001, 2, 3, 0, 631, (1, 2))[0]),
     ("ragged_o4", lambda: W.wl_1d(250 * 800, 800, 4, 4, 0, 632, (1, 2))[0]),
     ("ragged_o4_narrow", lambda: W.wl_1d(5 * 40000, 40000, 4, 3, 0, 633, (1, 2))[0]),
+    # blocks over PEs that are no multiple of four wide: the narrowest ones that take K = 4, a ring too short for K = 4,
+    # tiles that end one cell into the next, a domain of odd length that wraps
+    ("ragged_o2_blocks", lambda: W.wl_1d(73 * 2700, 2700, 2, 3, 0, 637, (1, 2))[0]),
+    ("ragged_o4_blocks", lambda: W.wl_1d(145 * 1357, 1357, 4, 2, 0, 638, (1, 2), scheme=W.ASYNC_STD)[0]),
+    ("ragged_o2_blocks_short_ring", lambda: W.wl_1d(257 * 801, 801, 2, 1, 0, 639, (1, 2))[0]),
+    ("ragged_o6_blocks", lambda: W.wl_1d(305 * 651, 651, 6, 3, 0, 640, (1, 2), r_alpha=0.01)[0]),
     ("ragged_o6_ab3", lambda: W.wl_1d(19 * 10500, 10500, 6, 3, 0, 634, (1, 2), r_alpha=0.01, tsteps=3)[0]),
     ("ragged_o4_unsplit", lambda: W.wl_1d(200001, 1, 4, 3, 0, 635, (1, 2))[0]),
     ("ragged_burgers_ab2_o4", lambda: dict(W.wl_1d(131 * 1600, 1600, 4, 3, 0, 636, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),

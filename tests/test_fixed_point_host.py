@@ -40,6 +40,12 @@ extern "C" int fx_sum(int n, const double *w, const double *v, int f32, double *
   *out = fx_to(R, E - 1023 - t.sw);
   return 1;
 }
+extern "C" int fx_weights(int n, const double *w, const double *low, int64_t *W) {
+  FxTaps<31> t;
+  fx_prepare(w, n, &t, low);
+  for (int i = 0; i < n; ++i) W[i] = (int64_t)t.w1[i] * (1ll << kFxLowBits) + t.w0[i];
+  return t.sw;
+}
 """
 
 
@@ -93,6 +99,23 @@ def test_sums_against_exact_rationals(lib, n, kind, f32):
         rep = size * Fraction(2 * n + 4, 2 ** 55) if f32 else size / 2 ** 58
         ulp = Fraction(math.ulp(abs(float(exact)))) if exact else Fraction(0)
         assert abs(Fraction(got) - exact) <= rep + ulp / 2 + (Fraction(math.ulp(got)) / 2 if got else 0)
+
+
+@pytest.mark.parametrize("low", [False, True])
+@pytest.mark.parametrize("n", [1, 17, 25])
+def test_weights_hold_the_low_parts_too(lib, n, low):
+    """Weights given as a double and what lies below its last bit come out as the nearest whole number of 2^-sw (and one
+    more rounding of 2^-53 of the part below a unit)."""
+    rng = np.random.default_rng([n, low])
+    for kind in ("stencil", "ones", "any"):
+        w = _weights(rng, n, kind)
+        wl = np.abs(w) * 2.0 ** -53 * rng.uniform(-1, 1, n)
+        W = (ctypes.c_int64 * n)()
+        D = ctypes.c_double * n
+        sw = lib.fx_weights(n, D(*w), D(*wl) if low else None, W)
+        for a, b, c in zip(w.tolist(), wl.tolist(), W):
+            exact = (Fraction(a) + (Fraction(b) if low else 0)) * 2 ** sw
+            assert abs(c - exact) <= Fraction(1, 2) + Fraction(1, 2 ** 40)
 
 
 def test_what_is_not_summed(lib):
