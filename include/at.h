@@ -161,8 +161,8 @@ int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_len, uint8_t 
  * same steps split into other calls give results equal up to rounding, not bit for bit.
  * Stencil sums run in block fixed point: a window's values scaled to its largest one, 62 bits each, exact to 2^-60 of
  * that value before the one rounding of the result; windows that fall steeply, hold infinities or NaN or lie at the
- * ends of the exponent range are summed as FP64 chains (large fields of any shape; small shapes whose PE width is no
- * multiple of 4 are chains throughout).  A problem of up to 2048 points without blocks of K >= 3 runs a call's steps in
+ * ends of the exponent range are summed as FP64 chains (single steps of fewer than
+ * 196608 points whose PE width is no multiple of 4 are chains throughout).  A problem of up to 2048 points without blocks of K >= 3 runs a call's steps in
  * one launch.
  * Adams-Bashforth runs from a caller's field take their first ts-1 steps (fewer stored levels, other weights) as
  * single launches; every later step -- every step after the analytic pre-history -- has all ts levels (with ts = 2
@@ -173,7 +173,7 @@ int at_step(at_handle_t *hd, int64_t nsteps);
 
 /* Block length of at_step for the following calls: the largest K <= k (1..4) the problem admits -- 1D, forward
  * Euler, AT_SYNC / AT_ASYNC_STD / AT_AT, not Burgers, n0 and the PE width multiples of 4 and the ring 16-byte aligned or
- * n0 >= 196608, more ring slots than K, and PEs wide enough that the zones stepped one step at a time (under 10 h + 16
+ * n0 > 1024, more ring slots than K, and PEs wide enough that the zones stepped one step at a time (under 10 h + 16
  * cells around each boundary for K = 4) do not meet and that a block saves at least 5 % of the multiply-adds of K
  * single steps (PEs of at least 144 cells for order 4 and K = 4, 72 for order 2) -- written to *k_used (1: single
  * steps).  at_init picks the largest

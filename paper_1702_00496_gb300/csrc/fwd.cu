@@ -559,11 +559,11 @@ static void fuse_radii(int h, int K, int *fe, int zr[]) {
 }
 
 int fuse_max_k(const StepParams &p, const void *ring, int kmax) {
-  // The block kernel itself takes any PE width and alignment.  Small shapes without aligned groups of four run point by
-  // point, with one rounding per tap for any split of the steps; large ones take blocks like the others (750000 points in
-  // PEs of 250, order 4: 3.7 us per step in blocks of 4, 9.8 in single steps).
+  // The block kernel itself takes any PE width and alignment.  Shapes without aligned groups of four that run a call's
+  // steps in one launch (small.cu) stay there; the others take blocks like the aligned ones (order 4, per step: 750000
+  // points in PEs of 250 9.8 us in single steps, 3.7 in blocks of 4; 30030 points in PEs of 143 4.4, 1.6 in blocks of 3).
   if (p.dim != 1 || p.scheme > AT_AT || p.burgers || p.ts != 1) return 1;
-  if (!grouped_shape(p, ring) && p.ntot < kRaggedPoints) return 1;
+  if (!grouped_shape(p, ring) && p.ntot <= kSmallPoints) return 1;
   for (int K = kmax < AT_MAX_FUSE ? kmax : AT_MAX_FUSE; K >= 2; --K) {
     if (p.R <= K) continue;  // U^n must stay in the ring while U^{n+K} is written
     int fe, zr[AT_MAX_FUSE];

@@ -167,9 +167,11 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
 // One forward step n = n_off + (*n_base if n_base else 0): reading the base from device memory lets a
 // captured graph of consecutive steps be replayed at any step.
 cudaError_t launch_forward_step(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
-// The fuse_k steps n .. n+fuse_k-1 of a block (n = n_off + *n_base): zone launches, then the block launch.
+// The fuse_k steps n .. n+fuse_k-1 of a block (n = n_off + *n_base), in one launch.
 cudaError_t launch_forward_block(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st);
-// nsteps steps n .. of a small 1D problem in one launch (small.cu), and whether the problem is one.
+// nsteps steps n .. of a small 1D problem in one launch (small.cu), and whether the problem is one: without aligned groups
+// of four, up to kSmallPoints points.
+constexpr int64_t kSmallPoints = 1024;
 bool small_steps_fit(const StepParams &p);
 cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t st);
 // 3D: the step in fixed point over tiles of the PEs (brick.cu); false: the shape or scheme is not one for it, nothing

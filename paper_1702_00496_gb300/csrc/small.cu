@@ -77,7 +77,7 @@ void launch_small_h(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t
 
 }  // namespace
 
-bool small_steps_fit(const StepParams &p) { return p.dim == 1 && p.n[0] <= (small_grouped(p) ? 2048 : 1024); }
+bool small_steps_fit(const StepParams &p) { return p.dim == 1 && p.n[0] <= (small_grouped(p) ? 2048 : kSmallPoints); }
 
 cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, cudaStream_t st) {
   const int64_t most = 4096;  // steps of one launch

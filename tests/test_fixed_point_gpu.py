@@ -42,6 +42,10 @@ PROBLEMS = [
     ("ragged_o4_blocks", lambda: W.wl_1d(145 * 1357, 1357, 4, 2, 0, 638, (1, 2), scheme=W.ASYNC_STD)[0]),
     ("ragged_o2_blocks_short_ring", lambda: W.wl_1d(257 * 801, 801, 2, 1, 0, 639, (1, 2))[0]),
     ("ragged_o6_blocks", lambda: W.wl_1d(305 * 651, 651, 6, 3, 0, 640, (1, 2), r_alpha=0.01)[0]),
+    # and small ones, from one point more than what one launch takes point by point
+    ("ragged_o4_blocks_smallest", lambda: W.wl_1d(205 * 5, 5, 4, 4, 0, 652, (1, 2))[0]),
+    ("ragged_o2_blocks_unsplit", lambda: W.wl_1d(1027, 1, 2, 3, 0, 653, (1, 2))[0]),
+    ("ragged_o6_blocks_odd", lambda: W.wl_1d(333 * 31, 31, 6, 3, 0, 654, (1, 2), r_alpha=0.01, scheme=W.ASYNC_STD)[0]),
     ("ragged_o6_ab3", lambda: W.wl_1d(19 * 10500, 10500, 6, 3, 0, 634, (1, 2), r_alpha=0.01, tsteps=3)[0]),
     ("ragged_o4_unsplit", lambda: W.wl_1d(200001, 1, 4, 3, 0, 635, (1, 2))[0]),
     ("ragged_burgers_ab2_o4", lambda: dict(W.wl_1d(131 * 1600, 1600, 4, 3, 0, 636, (1, 2), c=0.0, r_alpha=0.02, tsteps=2)[0], burgers=1)),
