@@ -39,32 +39,22 @@ import workloads as W  # noqa: E402
 
 METRIC = "grid-point updates/s (FP64)"
 FP64_FMA_LANES_PER_SM = 2  # FP64 FMA lanes per SM per clock on GB300 (nominal)
-# DRAM bytes (read + write) per launch of the step kernel, the mean of two launches of one ncu capture of the current
-# kernel source; None where no capture of the current source exists.
+# DRAM bytes (read + write) per launch of the step kernel, one ncu capture of the current kernel source; None where no
+# capture of the current source exists.
 MEASURED_TRAFFIC = {
-    ("1d_n16m", "forward_group_kernel<1,2,0>"): 136.95e6 + 80.50e6,
-    # blocks of 4 steps: one block launch (137.4 MB read, 79.2 MB written) and one zone launch (4.6 MB read) per
-    # block, per step
-    ("1d_n16m", "blocks of 4"): (137.4e6 + 79.2e6 + 4.6e6) / 4,
-    ("1d_n16m_case2", "forward_group_kernel<1,1,0>"): None,
-    ("1d_n16m_case3", "forward_group_kernel<1,1,0>"): 135.27e6 + 80.13e6,
-    ("1d_n16m_case4", "forward_group_kernel<1,2,2>"): 271.86e6 + 208.75e6,
-    ("1d_n16m_case5", "forward_group_kernel<1,3,1>"): 409.85e6 + 221.76e6,
-    ("1d_n16m_case6", "forward_group_kernel<1,2,1>"): 271.83e6 + 209.14e6,
-    # 3D: captured at 256^3 (the same 64^3 PEs; a 512^3 ring is 5-6 GB) over launches 5 and 6 of a 10-step run,
-    # scaled to 512^3 by the 8x points
-    ("3d_512_o2", "forward_group_kernel<3,1,0>"): 8 * (370.01e6 + 116.13e6),
-    ("3d_512_o4", "forward_group_kernel<3,2,0>"): 8 * (475.21e6 + 122.36e6),
+    ("1d_n16m", "blocks of 4"): (141.0e6 + 98.0e6) / 4,  # per step
+    ("1d_n16m_case3", "forward_group_kernel<1,1,0>"): 135.4e6 + 88.5e6,
+    ("1d_n16m_case4", "forward_group_kernel<1,2,2>"): 271.7e6 + 215.1e6,
+    ("1d_n16m_case5", "forward_group_kernel<1,3,1>"): 410.1e6 + 224.8e6,
+    ("1d_n16m_case6", "forward_group_kernel<1,2,1>"): 271.8e6 + 217.0e6,
+    # 3D: captured at 256^3 (the same 64^3 PEs; a 512^3 ring is 5-6 GB), scaled to 512^3 by the 8x points
+    ("3d_512_o2", "brick_kernel<1,0,0>"): 8 * (253.0e6 + 107.4e6),
+    ("3d_512_o4", "brick_kernel<2,0,0>"): 8 * (339.9e6 + 115.0e6),
 }
 TRAFFIC_NOTES = {
     "3d_512_o2": "DRAM read + write per launch from ncu at 256^3 in 4^3 PEs of 64^3, scaled by points to 512^3",
     "3d_512_o4": "DRAM read + write per launch from ncu at 256^3 in 4^3 PEs of 64^3, scaled by points to 512^3",
 }
-
-
-# The ensemble kernel's DRAM read + write per point update: ncu on a 100-step launch of the 1024 members (21.16 GB
-# read, 13.72 GB written, 1.794e9 updates); the full 5000-step launch scales with its updates.
-ENSEMBLE_DRAM_BYTES_PER_UPDATE = (21.16e9 + 13.72e9) / 1.7944576e9
 
 
 def measured_peaks():
@@ -194,9 +184,9 @@ def bytes_per_update(spec) -> int:
 def launches_per_run(spec, T: int, K: int = 1) -> int:
     """Kernels of this library one timed run launches: the reset (initial field, Adams-Bashforth pre-history and
     its history counter, the first delay draw), T forward steps (one counter update before the captured graphs,
-    each graph of G = 50 steps -- 48 in blocks of K = 4 or 3: whole blocks -- holding its step kernels, a block
-    being one zone launch and one block launch, and a counter kernel; the remainder launched one by one) and the
-    error statistics."""
+    each graph of G = 50 steps -- 48 in blocks of K = 4 or 3: whole blocks -- holding its step kernels, one launch per
+    block, and a counter kernel; the remainder launched one by one; small 1D problems without such blocks take a
+    launch per 4096 steps) and the error statistics."""
     dim, ts = spec["dim"], time_levels(spec)
     wave = 1 if dim == 1 else 2
     if spec.get("burgers", 0):  # no analytic pre-history: the history counter only
@@ -206,10 +196,12 @@ def launches_per_run(spec, T: int, K: int = 1) -> int:
     G = 50 // K * K if K > 1 else 50
 
     def launches(steps):
-        return (steps // K) * 2 + steps % K if K > 1 else steps
+        return steps // K + steps % K if K > 1 else steps
 
     chunks = T // G
     step = (1 + (launches(G) + 1) * chunks if chunks else 0) + launches(T - G * chunks)
+    if dim == 1 and K < 3 and spec["n"][0] <= 2048:
+        step = (T + 4095) // 4096
     stats = 2 if dim == 1 else 3
     return reset + step + stats
 
@@ -347,27 +339,24 @@ def measure_dgemm(local: int, n: int = 8192, reps: int = 3):
         return None
 
 
-def roofline_alu(flop_per_launch, bytes_per_launch, launch_ms, ops_per_launch, kernel, local, clocks, traffic=None,
-                 dgemm=None):
-    """FP64-pipe roofline of one kernel: achieved flop/s of its algorithmic work against the device's nominal FP64
-    rate; the FP64 lanes it issues per clock and SM (at the median SM clock sampled during the timed region); the
-    achieved HBM rate of its algorithmic bytes against the measured copy rate."""
+def roofline(flop_per_launch, bytes_per_launch, launch_ms, ops_per_launch, kernel, local, clocks, traffic=None,
+             dgemm=None):
+    """Roofline of one kernel.  The step kernels sum their stencils on the integer pipes (block fixed point), so the FP64
+    pipe is no ceiling any more: `achieved` is the HBM rate of the algorithmic bytes against the measured copy rate, and
+    beside it stands the rate of the algorithmic FP64 operations, as a multiple of what the FP64 pipe could do."""
     sms, mhz, peak = fp64_peak(local)
-    achieved = flop_per_launch / (launch_ms / 1e3)
-    mhz_run = (clocks or {}).get("sm_mhz") or mhz
-    hbm = measured_peaks().get("hbm_gbs")
+    hbm = measured_peaks().get("hbm_gbs") or 6800.0
     gbs = bytes_per_launch / (launch_ms / 1e3) / 1e9
-    out = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
-           "frac": achieved / peak, "traffic": traffic,
+    flops = flop_per_launch / (launch_ms / 1e3)
+    mhz_run = (clocks or {}).get("sm_mhz") or mhz
+    out = {"bound": "memory", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "traffic": traffic,
            "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
            "algorithmic_bytes_per_launch": bytes_per_launch, "kernel": kernel, "launch_ms": launch_ms,
-           "peak_source": f"nominal: {sms} SMs x {FP64_FMA_LANES_PER_SM} FP64 FMA lanes/clk x 2 flop x {mhz:.0f} MHz",
-           "fp64_lanes_per_clk_sm": ops_per_launch / (launch_ms / 1e3) / sms / (mhz_run * 1e6),
-           "fp64_lanes_clock_mhz": mhz_run,
-           "hbm_gbs": gbs, "hbm_frac_of_measured": (gbs / hbm) if hbm else None}
+           "peak_source": "measured copy bandwidth", "limit_now": "issue of the integer and FP32 pipes",
+           "algorithmic_tflops": flops / 1e12, "fp64_pipe_tflops": peak / 1e12, "multiple_of_fp64_pipe": flops / peak,
+           "fp64_operations_per_clk_sm": ops_per_launch / (launch_ms / 1e3) / sms / (mhz_run * 1e6)}
     if dgemm:
         out["dgemm_fp64_tflops"] = dgemm
-        out["frac_of_dgemm"] = achieved / 1e12 / dgemm
     return out
 
 
@@ -487,6 +476,10 @@ def measure_forward(spec, T, args, local, warmup, steps, world=1, e2e=False, flu
     ab = 0 if time_levels(spec) == 1 else (2 if time_levels(spec) == 2 and spec["dim"] == 1 and not spec.get("burgers")
                                            else 1)
     kname = f"forward_group_kernel<{spec['dim']},{spec['order'] // 2},{ab}>"
+    if spec["dim"] == 3:
+        kname = f"brick_kernel<{spec['order'] // 2},{ab},0>"
+    elif kblock < 3 and ntot <= 2048:
+        kname = f"small_steps_kernel<{spec['order'] // 2}> (a run of steps per launch; times are per step)"
     ops = fp64_ops_per_update(spec)
     bytes_update = bytes_per_update(spec)
     traffic = MEASURED_TRAFFIC.get((workload, kname))
@@ -494,20 +487,16 @@ def measure_forward(spec, T, args, local, warmup, steps, world=1, e2e=False, flu
         # blocks of K steps: 2 h K + 1 FP64 operations per point and block away from PE boundaries; U^n is read and
         # U^{n+K} written once per block
         traffic = MEASURED_TRAFFIC.get((workload, f"blocks of {kblock}"))
-        kname = (f"forward_block_kernel<{spec['order'] // 2},{kblock}> + forward_zones_kernel<{spec['order'] // 2},"
-                 f"{kblock}> (blocks of {kblock} steps)")
+        kname = f"forward_block_kernel<{spec['order'] // 2},{kblock}> (blocks of {kblock} steps; times are per step)"
         ops = (spec["order"] * kblock + 1) / kblock
         bytes_update = 16 / kblock
-    out["roofline"] = roofline_alu(flops_per_update(spec) * ntot, bytes_update * ntot, kern_ms,
+    out["roofline"] = roofline(flops_per_update(spec) * ntot, bytes_update * ntot, kern_ms,
                                    ops * ntot, kname, local, clocks, traffic, dgemm)
     if kblock > 1:
-        out["roofline"]["traffic_note"] = "DRAM read + write per step (a block launch and a zone launch per K steps, ncu)"
-    out["roofline"]["fp64_ops_per_update_executed"] = ops
-    if kblock > 1:
-        out["roofline"]["note"] = ("achieved counts the single step's algorithmic flop per update (1 multiply and "
-                                   "2 h FMAs); blocks of K steps execute 2 h K + 1 FP64 operations per point and "
-                                   "block away from PE boundaries (fp64_ops_per_update_executed), so the FP64 "
-                                   "lanes per clock use that count")
+        out["roofline"]["traffic_note"] = "DRAM read + write per step (one launch per K steps, ncu)"
+        out["roofline"]["note"] = ("algorithmic_tflops counts the single step's flop per update (1 multiply and 2 h FMAs); "
+                                   "U^n is read and U^{n+K} written once per block of K steps, whose composed stencil "
+                                   "has 2 h K + 1 taps (fp64_operations_per_clk_sm)")
     if workload in TRAFFIC_NOTES:
         out["roofline"]["traffic_note"] = TRAFFIC_NOTES[workload]
     out["gpu_launches"] = steps * launches_per_run(spec, T, kblock)
@@ -606,10 +595,8 @@ def measure_ensemble(args, local, specs, steps_list, T, groups_in, twins, warmup
            "one_at_a_time_ms": one, "speedup_vs_one_at_a_time": (one / ms) if one else None,
            "one_at_a_time_clocks": one_clocks, "groups": groups, "clocks": clocks, "gpu_launches": steps * 4}
     if T is not None:
-        rec["roofline"] = roofline_alu(flop, 16 * updates, ms, 5 * updates, "ensemble_kernel (whole graph launch)",
-                                       local, clocks, ENSEMBLE_DRAM_BYTES_PER_UPDATE * updates)
-        rec["roofline"]["traffic_note"] = ("DRAM read + write per update from one ncu capture of a 100-step launch of "
-                                           "the same members, scaled to this launch's updates")
+        rec["roofline"] = roofline(flop, 16 * updates, ms, 5 * updates, "ensemble_kernel (whole graph launch)", local,
+                                   clocks)
     return rec
 
 
@@ -676,7 +663,6 @@ def run_ensemble(args, rank: int, world: int, local: int):
 
 # --------------------------------------------------------------------------------------------- adjoint
 ADJ_FLOP_PER_CELL = 54  # 3D order 4, transposed step with the alpha term: 13 + 13 + 1 FMAs per cell
-ADJ_DRAM_BYTES_PER_LAUNCH = 1.67e9 + 0.32e9  # ncu, one backward step with the alpha term at 256^3
 
 
 def measure_adjoint(args, local, T, every, warmup, steps, rank=0, world=1, forward=True):
@@ -780,13 +766,11 @@ def adjoint_record(args, local, T, warmup, steps) -> dict:
                       "u0_only_ms": sq["adjoint_u0_only_ms"],
                       "u0_only_forward_ratio": sq["adjoint_u0_only_ms"] / f_ms, "clocks": sq["clocks"]},
            "grad_alpha": sq["grad_alpha"],
-           "fma_floor": {"alpha_resident": (13 + 27) / 13, "alpha_sqrt_t": (13 + 13 + 27) / 13,
+           "tap_ratio": {"alpha_resident": (13 + 27) / 13, "alpha_sqrt_t": (13 + 13 + 27) / 13,
                          "u0_only": (13 + 13) / 13,
-                         "note": "FP64 FMAs per cell: forward step 13, transposed step 13 (27 with the alpha term "
-                                 "<lambda, dt D2_AT U>), recompute of a checkpointed segment 13; the whole "
-                                 "gradient in dJ/dalpha cannot cost less than these multiples of the forward run on "
-                                 "the FP64 pipe, so <= 3x for dJ/dalpha is below what the pipe allows; dJ/du0 alone "
-                                 "needs no forward level and no recompute"}}
+                         "note": "multiply-adds per cell, as multiples of the forward run's: forward step 13, transposed "
+                                 "step 13 (27 with the alpha term <lambda, dt D2_AT U>), recompute of a checkpointed "
+                                 "segment 13; dJ/du0 alone needs no forward level and no recompute"}}
     free = torch.cuda.mem_get_info(local)[0]
     need = 8 * ntot * (T + 3 * R + 8)  # every level, the adjoint ring, the solver's ring and small fields
     if free > need:
@@ -796,11 +780,9 @@ def adjoint_record(args, local, T, warmup, steps) -> dict:
                            "backward_ms": rs["backward_ms"], "backward_forward_ratio": rs["backward_ms"] / f_ms,
                            "u0_only_ms": rs["adjoint_u0_only_ms"],
                            "u0_only_forward_ratio": rs["adjoint_u0_only_ms"] / f_ms, "clocks": rs["clocks"]}
-        rec["roofline"] = roofline_alu(ADJ_FLOP_PER_CELL * ntot, 8 * 8 * ntot, rs["backward_ms"] / T, 27 * ntot,
-                                       "adjoint_step_kernel (transposed step with the alpha term, every level "
-                                       "resident)", local, rs["clocks"], ADJ_DRAM_BYTES_PER_LAUNCH)
-        rec["roofline"]["traffic_note"] = ("DRAM read + write of one backward step at 256^3 from one ncu capture "
-                                           "(1.67 GB read, 0.32 GB written)")
+        rec["roofline"] = roofline(ADJ_FLOP_PER_CELL * ntot, 8 * 8 * ntot, rs["backward_ms"] / T, 27 * ntot,
+                                       "brick_kernel<2,0,2> + brick_kernel<2,0,1> + brick_faces_kernel<2> (a backward step with "
+                                       "the alpha term, every level resident)", local, rs["clocks"])
     else:
         rec["resident"] = {"skipped": f"needs {need / 1e9:.0f} GB free, {free / 1e9:.0f} GB free"}
         rec["roofline"] = None
@@ -851,12 +833,12 @@ def config_records(args, local, dgemm) -> dict:
         _free()
 
     def n256():
-        # 1D N = 256 (2000 steps): the whole ring is on chip, so one launch per step is bound by launch latency;
-        # the persistent engine runs the same problem (same delays, same field) inside one CTA without launches
+        # 1D N = 256 (2000 steps): latency of one CTA's step is all there is.  The value is Solver.step, which runs the
+        # steps of a call in one launch; beside it the same problem as a one-member ensemble
         spec, T = W.workload("1d_n256")
         r = forward_record("1d_n256", spec, T, args, local, sub_w, sub_k, 0,
-                           note="2 KB field: latency-bound, no HBM or FP64-pipe bound applies; value = one launch "
-                                "per step (Solver), persistent = the whole run in one CTA of the ensemble engine")
+                           note="2 KB field: latency-bound, no HBM or pipe bound applies; value = one launch "
+                                "per run of steps (Solver), persistent = the whole run in one CTA of the ensemble engine")
         r["persistent"] = persistent_single(spec, T, local, sub_w, sub_k)
         r["cpu_baseline"] = {"value": cpu_sample(spec, T, 1), "unit": "updates/s", "cores": 1, "kind": "oracle",
                              "cpu_model": cpu_model(), "sample": f"the whole {T}-step run on one thread"}
