@@ -297,8 +297,8 @@ int at_adjoint_backward(at_handle_t *hd, const double *lambda_dev, double *grad_
  *   need (members stored one after another; member r's ring holds its own at_ring_slots slots, its log
  *   nsteps_r x sides_r bytes).
  * at_ensemble_create: members and runs are copied; ring_dev (ring_len doubles, 16-byte aligned) and the optional
- *   log_dev (log_len bytes, NULL for no log) are borrowed.  threads per CTA is 128, 256, 512 or 1024 (0: 512 when there are more
- *   members than SMs, else 1024);
+ *   log_dev (log_len bytes, NULL for no log) are borrowed.  threads per CTA is 128, 256, 512 or 1024 (0: by the members' number
+ *   and size -- 1024, with at least four members per SM 512, or 256 if none has more than 1024 points);
  *   ctas_per_sm <= 0 takes the occupancy limit.  Every member starts from Eq. "IC" (with the analytic
  *   pre-history for Adams-Bashforth).  Errors: AT_ERR_ARG (non-1D member, n[0] or the PE width not a multiple
  *   of 4, bad nsteps, group or twin, sizes), AT_ERR_CUDA.

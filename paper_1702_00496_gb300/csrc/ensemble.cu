@@ -374,10 +374,16 @@ extern "C" int at_ensemble_create(const at_config_t *members, const at_member_t 
   if (reinterpret_cast<uintptr_t>(ring_dev) % 16)
     return fail(AT_ERR_ARG, "at_ensemble_create: ring not 16-byte aligned (the group kernels use 16-byte accesses)");
   if (log_dev && log_len < need_log) return fail(AT_ERR_ARG, "at_ensemble_create: log too small");
-  if (threads == 0) {  // two blocks of 512 per SM overlap their barriers (1024 members of 250 steps: 36.7 against 38.7 ms);
-    int dev = 0, sms = 152;  // one of 1024 where every member has an SM to itself
+  if (threads == 0) {
+    // Several members per SM hide each other's barriers and use what small members leave idle, but only while there are
+    // members enough to keep every SM at several (ms for 1024 x 1, 512 x 2, 256 x 4 threads and CTAs per SM: 1024
+    // members of 2^10..2^16 points 37.0, 34.7, 60.6; 1200 of 2^8..2^10 35.3, 22.0, 17.3; 200 of 2^13..2^15 6.0, 10.8, 13.7).
+    int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    threads = count > sms ? 512 : 1024;
+    int64_t largest = 0;
+    for (int r = 0; r < count; ++r) largest = std::max(largest, (int64_t)members[r].n[0]);
+    const bool many = count >= 4 * sms;
+    threads = many && largest <= 1024 ? 256 : (many || (count > sms && largest <= 2048) ? 512 : 1024);
   }
   if (threads != 128 && threads != 256 && threads != 512 && threads != 1024)
     return fail(AT_ERR_ARG, "threads must be 128, 256, 512 or 1024");
