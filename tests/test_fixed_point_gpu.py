@@ -215,3 +215,20 @@ def test_gradient_on_tiles_matches_the_cpu_adjoint(name, make, callers_field):
     assert np.linalg.norm(g - go) / np.linalg.norm(go) <= 1e-12
     assert ga == pytest.approx(gao, rel=1e-10)
     assert np.array_equal(grads[1][0], g) and grads[1][1] == ga and np.array_equal(grads[2][0], g)
+
+
+@pytest.mark.parametrize("n,count", [(64, 153), (64, 640), (1028, 640), (2052, 153)])
+def test_default_ensemble_shapes_give_the_same_members(n, count):
+    """The CTA shapes that the members' number and size choose by default (256, 512, 1024 threads) against one of 1024:
+    the fields bit for bit, the statistics up to the order of their sums (errors of 2^-53 per term, n terms)."""
+    from paper_1702_00496_gb300 import Ensemble
+    specs = [W.wl_1d(n, n // 4, 2, 3, 0, 700 + r, (1, 2))[0] for r in range(count)]
+    a, b = Ensemble(specs, 9), Ensemble(specs, 9, threads=1024)
+    for e in (a, b):
+        e.run()
+    for r in (0, 1, count // 2, count - 1):
+        assert torch.equal(a.field(r), b.field(r)), r
+    for x, y in zip(a.stats()[0], b.stats()[0]):
+        assert x["rms"] == pytest.approx(y["rms"], rel=n * 2.0 ** -52, abs=0)
+    a.close()
+    b.close()
