@@ -119,6 +119,7 @@ __device__ __forceinline__ void zone_steps(const StepParams &p, int64_t n, int s
     last = delay_clamp(raw, st, p.T);
     if (p.log != nullptr && st < p.log_steps) p.log[st * p.nb + side] = (uint8_t)raw;
   }
+  __syncwarp();  // for even K the delays of step n + K go where lanes 0 and 1 read those of step n; a shuffle orders no memory
   const int up = __shfl_up_sync(0xffffffffu, last, 2);
   if (lane >= 2) k = up;
   if (lane >= 2 * K - 2 && lane < 2 * K) p.keff[((n + K) & 1) * p.nb + side] = (uint8_t)last;
