@@ -10,7 +10,9 @@
 //  - Where the tile meets a face of its PE, the cells beyond are buffer points: they are extrapolated over the delayed
 //    levels (FP64, as everywhere) once per tile when their plane is loaded, with that side's delay.
 //  - One scale serves the planes of the ring.  A plane whose largest value exceeds it, or a ring that has fallen two
-//    bits below it, rescales the ring (a shift of every entry: rare, fields change little from plane to plane).
+//    bits below it, rescales the ring (a shift of every entry: rare, fields change little from plane to plane).  Planes cut
+//    at a scale that has fallen since lack the digits between: sums over them want values as many bits larger, and beyond
+//    kFxLift such bits they are not used (fixed.cuh, FxRing).
 //  - One barrier per plane: iteration i sums output plane i-2-h from planes the ring already holds (while the loads of
 //    plane i are in flight), publishes plane i's largest value, and after the barrier stores plane i.
 //  - A thread sums four x-consecutive points.  A group with a half more than kBrickGuard bits below the scale (where the
@@ -95,7 +97,8 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
                                                                             const int64_t *n_base) {
   constexpr int NR = 2 * H + 2;  // ring planes
   extern __shared__ int2 ring[];
-  __shared__ int mx[3], pm[8], later[kBrickLater], n_later;
+  __shared__ int mx[3], later[kBrickLater], n_later;
+  __shared__ FxPlanes planes;
   const int64_t n = n_off + (n_base ? *n_base : 0);
   const double *__restrict__ un = MODE == 1 ? adj.src : p.ring + slot_of(n, p.R) * p.ntot;
   double *__restrict__ out = MODE == 1 ? adj.cur : p.ring + slot_of(n + 1, p.R) * p.ntot;
@@ -224,9 +227,8 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
   };
   if (tid == 0) n_later = 0;
   if (tid < 3) mx[tid] = 0;
-  if (tid < 8) pm[tid] = 0;
-  int E = -1;
-  uint32_t bad = 0;  // planes (mod 32) that no sum may use
+  if (tid < 8) planes.top[tid] = planes.cut[tid] = 0;
+  FxRing scale;
   // this thread's points; a thread without any sums the tile's first group along
   int row = tid / b.gx, grp = tid - row * b.gx;
   const bool mine = row < ylen && 4 * grp < xlen;
@@ -329,8 +331,8 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
       const int2 *pl[2 * H + 1];
 #pragma unroll
       for (int d = 0; d <= 2 * H; ++d) pl[d] = ring + (cslot + d >= NR ? cslot + d - NR : cslot + d) * b.plane + col;
-      const uint32_t bits = __funnelshift_r(bad, bad, (uint32_t)(o - H) & 31u) & ((2u << (2 * H)) - 1u);
-      const bool usable = bits == 0;
+      const int E = scale.E, lift = fx_ring_lift(scale, planes, o, H);
+      const bool usable = lift <= kFxLift;
       double r[4] = {0.0, 0.0, 0.0, 0.0};
       bool far = false;
       if (usable && E >= 0) {  // the same for the whole block; E < 0: every plane so far is zero
@@ -339,10 +341,9 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
 #pragma unroll
         for (int q = 0; q < 4; ++q) c4[q] = mid[q];
         {
-          const int g0 = (c4[0].x ^ (c4[0].x >> 31)) | (c4[1].x ^ (c4[1].x >> 31));
-          int g1 = (c4[2].x ^ (c4[2].x >> 31)) | (c4[3].x ^ (c4[3].x >> 31));
-          g1 = nv < 3 ? g0 : g1;
-          far = MODE != 2 && (min(g0, g1) >> (29 - kBrickGuard)) == 0;  // a sum over all points needs no local bits
+          const uint32_t g0 = fx_upper(c4[0].x) | fx_upper(c4[1].x);
+          const uint32_t g1 = nv < 3 ? g0 : fx_upper(c4[2].x) | fx_upper(c4[3].x);
+          far = MODE != 2 && min(g0, g1) < fx_least(kBrickGuard, lift);  // a sum over all points needs no local bits
         }
         int64_t A[4], B[4], C[4];
         const FxTaps<6 * AT_MAX_H + 1> &t = p.f3;
@@ -413,38 +414,24 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
       continue;
     }
     __syncthreads();
-    const int m = mx[m3] >> 20;
+    const int m = mx[m3];
     if (tid == 0) mx[m3 == 0 ? 2 : m3 - 1] = 0;  // read by all before this barrier, used again two planes on
-    const bool ok = m == 0 || fx_usable(m);
-    const uint32_t bit = 1u << ((uint32_t)i & 31u);
-    bad = ok ? bad & ~bit : bad | bit;
-    int to = E;
-    if (ok && m > 0) {
-      if (m > E) {
-        to = m;
-      } else if (m <= E - 2) {  // has the whole ring fallen?
-        int top = m;
-        for (int d = 1; d < NR; ++d) top = max(top, pm[(i - d) & 7]);
-        if (top <= E - 2) to = top;
-      }
-    }
-    if (to != E && E >= 0) {
-      const int d = to - E;
+    const bool ok = fx_plane_usable(m);
+    const int top = ok ? m >> 20 : 0, d = fx_ring_join(scale, planes, i, top, H, ok);
+    if (tid == 0) fx_ring_note(planes, scale, i, top, d, ok);  // of planes that no output reads before the next barrier
+    if (d != 0) {
       for (int e = tid; e < NR * b.plane; e += kBrickThreads) {
         const int2 f = ring[e];
-        const int64_t x = (int64_t)f.x * 4294967296ll + f.y;
-        const Fx g = fx_split(d > 0 ? fx_shr(x, d) : (int64_t)((uint64_t)x << min(-d, 63)));
+        const Fx g = fx_split(fx_rescale((int64_t)f.x * 4294967296ll + f.y, d));
         ring[e] = make_int2(g.hi, g.lo);
       }
       __syncthreads();
     }
-    E = to;
-    if (tid == 0) pm[i & 7] = ok ? m : 0;
-    if (ok) {  // a zero plane, or one before the first scale: E is any, the values come out 0 (-1 for -0)
+    if (ok) {  // a zero plane, or one before the first scale: the scale is any, the values come out 0 (-1 for -0)
       int2 *dst = ring + wslot * b.plane;
 #pragma unroll
       for (int s = 0; s < kBrickSlots; ++s) {
-        const Fx f = fx_split(fx_from(v[s], E));
+        const Fx f = fx_split(fx_from(v[s], scale.E));
         dst[code[s] & 0xffff] = make_int2(f.hi, f.lo);
       }
     }

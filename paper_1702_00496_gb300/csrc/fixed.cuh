@@ -124,6 +124,13 @@ AT_FX_HD double fx_to(int64_t R, int ex) {
   return fx_assemble(a, sh, (int32_t)(sm >> 32), ex);
 }
 
+// |x|'s upper word (one less for an x below zero whose lower word is 0), given x's.
+AT_FX_HD uint32_t fx_upper(int32_t hi) { return (uint32_t)(hi ^ (hi >> 31)); }
+
+// Upper word from which on a value of an output's stencil is within `guard` bits of the largest there is, where entries
+// miss `lift` bits (guard >= lift).
+AT_FX_HD uint32_t fx_least(int guard, int lift) { return 1u << (30 - guard + lift); }
+
 AT_FX_HD double fx_to_wide(int64_t R, int ex, uint32_t *small) {
 #if defined(__CUDA_ARCH__)
   const int64_t sm = R >> 63;
@@ -166,6 +173,65 @@ AT_FX_HD void fx_results(const int64_t R[N], int ex, double r[N]) {
     for (int q = 0; q < N; ++q)
       if (R[q] < (1ll << 32) && R[q] > -(1ll << 32)) r[q] = fx_to(R[q], ex);
   }
+}
+
+// The scale of a ring of planes that a march lays down one by one (brick.cu), each cut at the scale of its moment.
+//
+// A larger plane raises the scale: every entry is shifted down and is then cut at the new scale, like the plane itself.
+// Once the ring has fallen two bits below it the scale falls and the entries are shifted up -- but the digits that were cut
+// at the old scale stay lost: they are `lift` bits short of what a plane cut at the new scale holds.  Callers ask that of
+// an output's planes and want values as many bits larger (fx_least), or take the FP64 chain.
+constexpr int kFxLift = 6;  // planes with more missing bits than this are not used
+
+struct FxRing {    // the same in every thread of a march
+  int E = -1;      // exponent of the scale; -1: no plane but zeros so far
+  int until = -8;  // planes up to this one may have been cut above it, or are not there
+};
+struct FxPlanes {          // of the last eight planes: plane i at i mod 8, written by one thread (fx_ring_note)
+  int top[8], cut[8];      // exponent of the largest value (0: zeros, or not usable) and of the scale it was cut at
+};
+constexpr int kFxNever = 1 << 20;  // cut of a plane that is not usable
+
+// Is a plane whose largest magnitude (fx_mag) is mag summed in fixed point?
+AT_FX_HD bool fx_plane_usable(int mag) { return (mag >> 20) == 0 || fx_usable(mag >> 20); }
+
+// Plane i joins; m: exponent of its largest value (0 as above), usable: fx_plane_usable; reach: planes on either side that
+// an output reads, so the 2 reach + 1 planes before i are still in use.  Returns by how much the scale rose: entries go down
+// by that, or up by its negative; 0 also for the first scale, before which every entry is 0 or -1.
+AT_FX_HD int fx_ring_join(FxRing &r, const FxPlanes &p, int i, int m, int reach, bool usable) {
+  int to = r.E;
+  if (m != 0 && m > r.E) {
+    to = m;
+  } else if (m != 0 && m <= r.E - 2) {  // has the whole ring fallen?
+    int most = m;
+    for (int q = 1; q <= 2 * reach + 1; ++q) most = p.top[(i - q) & 7] > most ? p.top[(i - q) & 7] : most;
+    if (most <= r.E - 2) to = most;
+  }
+  const int d = r.E < 0 ? 0 : to - r.E;
+  if (d < 0) r.until = i - 1;
+  if (!usable) r.until = i;
+  r.E = to;
+  return d;
+}
+
+AT_FX_HD void fx_ring_note(FxPlanes &p, const FxRing &r, int i, int m, int d, bool usable) {
+  if (d > 0)
+    for (int q = 0; q < 8; ++q) p.cut[q] = p.cut[q] > r.E ? p.cut[q] : r.E;
+  p.top[i & 7] = m;
+  p.cut[i & 7] = usable ? r.E : kFxNever;
+}
+
+// Bits that the planes o - reach .. o + reach of an output miss against the scale.
+AT_FX_HD int fx_ring_lift(const FxRing &r, const FxPlanes &p, int o, int reach) {
+  if (o - reach > r.until) return 0;
+  int most = r.E;
+  for (int q = o - reach; q <= o + reach; ++q) most = p.cut[q & 7] > most ? p.cut[q & 7] : most;
+  return most - r.E;
+}
+
+// A ring entry after the scale rose by d (fell by -d).
+AT_FX_HD int64_t fx_rescale(int64_t x, int d) {
+  return d > 0 ? fx_shr(x, d) : (int64_t)((uint64_t)x << (d < -63 ? 63 : -d));
 }
 
 // Weights of up to N taps; sw = 0 with ok = 0 when they cannot be represented (not finite, all zero, out of range).

@@ -1,0 +1,96 @@
+"""One launch of the fixed-point step kernels, every cell against its own stencil.
+
+A norm does not see a cell that is small beside another one; here each cell is held to the largest value of its own
+stencil.  As an FMA chain a sum of n taps may be off by n roundings of 2^-53 of that value times sum |w|, in fixed point by
+7 + n of them (test_fixed_ring_host.py derives it), and the weights, a few roundings each, by up to n more
+(both sides may contract them differently).  The reference applies the weights in extended precision.  The domains are
+unsplit, so every point takes the central taps; the kernels and their routes are those of split ones."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+CD1 = {2: [-1 / 2, 0.0, 1 / 2], 4: [1 / 12, -2 / 3, 0.0, 2 / 3, -1 / 12],
+       6: [-1 / 60, 3 / 20, -3 / 4, 0.0, 3 / 4, -3 / 20, 1 / 60]}
+CD2 = {2: [1.0, -2.0, 1.0], 4: [-1 / 12, 4 / 3, -5 / 2, 4 / 3, -1 / 12],
+       6: [1 / 90, -3 / 20, 3 / 2, -49 / 18, 3 / 2, -3 / 20, 1 / 90]}
+
+
+def _taps(spec):
+    """dt f's merged taps per axis."""
+    out = []
+    for a in range(spec["dim"]):
+        dx = 2.0 * np.pi / spec["n"][a]
+        c1, c2 = np.array(CD1[spec["order"]]), np.array(CD2[spec["order"]])
+        out.append((spec["dt"] * (-spec["c"][a] * c1 / dx + spec["alpha"] * c2 / (dx * dx))).astype(np.longdouble))
+    return out
+
+
+def _apply(u, taps, reverse=False):
+    """(sum of w v, largest |v|) of dt f at every cell; u of shape (.., nx) in extended precision."""
+    s, m = np.zeros_like(u), np.abs(u)
+    for a, t in enumerate(taps):
+        h = len(t) // 2
+        for j in range(-h, h + 1):
+            v = np.roll(u, j if reverse else -j, u.ndim - 1 - a)
+            s += t[j + h] * v
+            m = np.maximum(m, np.abs(v))
+    return s, m
+
+
+def _field(shape, kind, size, seed):
+    rng = np.random.default_rng([seed, len(kind)])
+    u = rng.uniform(0.5, 1.0, shape) * rng.choice([1.0, -1.0], shape)
+    z = np.arange(shape[0]).reshape((-1,) + (1,) * (len(shape) - 1))
+    if kind == "slab":  # two planes beside values of size 1, at every phase of a march
+        u = np.where(z % 23 < 2, u * size, u)
+    elif kind == "decay":  # falls and rises along z
+        u = u * size ** (-0.25 * np.minimum(z % 41, 40 - z % 41))
+    elif kind == "spikes":
+        u = np.where(rng.random(shape) < 2e-4, u * size, u)
+    return u
+
+
+TILES = [
+    ("o2", lambda: W.wl_3d([128, 96, 130], 1, 2, 3, 0, 901, c=(0.3, 0.2, 0.1))[0]),
+    ("o4", lambda: W.wl_3d([128, 96, 130], 1, 4, 3, 0, 902, c=(0.3, 0.2, 0.1))[0]),
+    ("o4_odd", lambda: W.wl_3d([125, 101, 127], 1, 4, 3, 0, 903, c=(0.3, 0.2, 0.1))[0]),
+    ("o6", lambda: W.wl_3d([128, 96, 130], 1, 6, 3, 0, 904, c=(0.3, 0.2, 0.1), dt=0.01 * W.dx_of(130) ** 2 / 0.05)[0]),
+    ("o4_ab2", lambda: W.wl_3d([128, 96, 130], 1, 4, 3, 0, 905, c=(0.3, 0.2, 0.1), tsteps=2)[0]),
+]
+FIELDS = [("slab", 1e4), ("slab", 1e8), ("slab", 1e16), ("slab", 1e20), ("decay", 4.0), ("decay", 1e4), ("decay", 1e8),
+          ("spikes", 1e8)]
+
+
+def _check(got, u, taps, n, reverse=False):
+    f, m = _apply(u, taps, reverse)
+    bar = (2 * n + 7) * np.longdouble(2.0) ** -53 * m * (1 + sum(np.abs(t).sum() for t in taps))
+    off = np.abs(got.astype(np.longdouble) - (u + f))
+    worst = np.unravel_index(np.argmax(off / bar), off.shape)
+    assert (off <= bar).all(), (worst, got[worst], float((u + f)[worst]))
+
+
+@pytest.mark.parametrize("kind,size", FIELDS, ids=[f"{k}_{s:g}" for k, s in FIELDS])
+@pytest.mark.parametrize("name,make", TILES, ids=[t[0] for t in TILES])
+def test_a_tiled_step_and_its_transpose_cell_by_cell(name, make, kind, size):
+    from paper_1702_00496_gb300 import Solver
+    spec = make()
+    shape = tuple(spec["n"][::-1])
+    u0, lam = _field(shape, kind, size, 1), _field(shape, kind, size, 2)
+    s = Solver(spec)
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.step(1)
+    s.sync()
+    got = s.field().cpu().numpy().copy()
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.adjoint_forward(1, 1)
+    g, _ = s.adjoint_backward(torch.as_tensor(lam, device="cuda"), False)
+    g = g.cpu().numpy()
+    s.close()
+    n = 1 + 3 * spec["order"]
+    _check(got, u0.astype(np.longdouble), _taps(spec), n)
+    _check(g, lam.astype(np.longdouble), _taps(spec), n, reverse=True)
