@@ -205,12 +205,7 @@ int at_prepare_params(const at_config_t *cfg, double *ring_dev, uint8_t *log_dev
     const uint32_t up = ((uint32_t)(p.use_pe[0] ? p.S[0] : p.n[0]) + 3) >> 2;
     p.div_up = atfd::fast_div(up > 3 ? up - 3 : 1);
   } else {
-    double t[6 * AT_MAX_H + 1] = {p.s0};
-    int c = 1;
-    for (int a = 0; a < 3; ++a)
-      for (int j = -h; j <= h; ++j)
-        if (j != 0) t[c++] = p.s[a][j + h];
-    atfd::fx_prepare(t, c, &p.f3);
+    fx_prepare_3d(&p, p.s0, p.s);
   }
   return AT_OK;
 }
@@ -338,7 +333,8 @@ extern "C" int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_le
       }
   }
   const size_t order_bytes = (order.size() * sizeof(int32_t) + 255) / 256 * 256;
-  const size_t bytes = 512 + keff_bytes + order_bytes +
+  const size_t listed_bytes = ((size_t)brick_listed_words(p) * sizeof(uint32_t) + 255) / 256 * 256;
+  const size_t bytes = 512 + keff_bytes + order_bytes + listed_bytes +
                        sizeof(double) * ((size_t)AT_STAT_BLOCKS * AT_STAT_FIELDS + 16 + n_tables);
   cudaError_t e = cudaMalloc(&hd->scratch, bytes);
   if (e != cudaSuccess) { delete hd; return cuda_fail(e, "at_init: cudaMalloc"); }
@@ -347,7 +343,8 @@ extern "C" int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_le
   p.keff = (uint8_t *)(base + 512);
   p.order = order.empty() ? nullptr : (const int32_t *)(base + 512 + keff_bytes);
   hd->n_interior = n_interior;
-  hd->d_partials = (double *)(base + 512 + keff_bytes + order_bytes);
+  p.listed = listed_bytes ? (uint32_t *)(base + 512 + keff_bytes + order_bytes) : nullptr;
+  hd->d_partials = (double *)(base + 512 + keff_bytes + order_bytes + listed_bytes);
   if (!order.empty() &&
       (e = cudaMemcpy((void *)p.order, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice)) !=
           cudaSuccess) {

@@ -11,15 +11,13 @@
 //    levels (FP64, as everywhere) once per tile when their plane is loaded, with that side's delay.
 //  - One scale serves the planes of the ring.  A plane whose largest value exceeds it, or a ring that has fallen two
 //    bits below it, rescales the ring (a shift of every entry: rare, fields change little from plane to plane).  Planes cut
-//    at a scale that has fallen since lack the digits between: sums over them want values as many bits larger, and beyond
-//    kFxLift such bits they are not used (fixed.cuh, FxRing).
+//    at a scale that has fallen since lack the digits between: their sums must be as much larger, and from kFxLift such
+//    bits on they are not used (fixed.cuh, FxRing).
 //  - One barrier per plane: iteration i sums output plane i-2-h from planes the ring already holds (while the loads of
 //    plane i are in flight), publishes plane i's largest value, and after the barrier stores plane i.
 //  - A thread sums four x-consecutive points.  A group with a half more than kBrickGuard bits below the scale (where the
-//    field changes sign along two axes at once, or falls steeply) takes the FP64 chain, as does every group of a plane
-//    near infinities, NaN or values at the ends of the exponent range.  The former are listed and done together after
-//    the march: done in place, one such group held its block's barrier for 52 DFMA (256^3: 411 us per step against 242
-//    without any).
+//    field changes sign along two axes at once, or falls steeply) is left to its FP64 chain, as is every group of a plane
+//    near infinities, NaN or values at the ends of the exponent range.  The march lists them, and a second launch does them.
 //
 // The backward sweep of the gradient runs on the same tiles: the transposed step's level-n part (taps reversed, cells
 // across a face counted only at delay 0), the alpha term (second-derivative taps of U^n times lambda, summed), and a
@@ -43,10 +41,10 @@ using namespace atfd;
 constexpr int kBrickThreads = 128;
 constexpr int kBrickX = 32;
 constexpr int kBrickBlocks = 4;
-constexpr int kBrickLater = 512; // groups a block can list for the FP64 chain
+constexpr int kBrickWarps = kBrickThreads / 32;  // words of a plane's listed groups
+constexpr int kBrickGuard = 10;  // bits below the scale that one of two x neighbours must be within
 constexpr int kCore = 4;         // values of the tile's own cells a thread loads per plane
 constexpr int kBrickSlots = 6;   // and with those around it
-constexpr int kBrickGuard = 10;  // a tile spans more cells than a 1D window: lines where the field changes sign meet in it
 
 struct BrickShape {
   int32_t tx, gx, rows;            // cells and groups of four per tile row, rows per tile
@@ -67,24 +65,336 @@ struct BrickAdjoint {
   int32_t add;          // MODE 1: add to cur (else set it)
 };
 
-// One point of the transposed step's level-n part as an FMA chain: p.s holds the taps reversed, p.s0 the centre; a
-// neighbour across a face with a delay (kn: the delays of the neighbours' sides) contributes to older levels instead.
-template <int H>
-__device__ __noinline__ double transposed_point(const StepParams &p, const double *__restrict__ src, const int pidx[3],
-                                                const int kn[3][2], const int c[3]) {
-  const int64_t stride[3] = {1, (int64_t)p.n[0], (int64_t)p.n[0] * p.n[1]};
-  const int64_t i = c[2] * stride[2] + c[1] * stride[1] + c[0];
-  double acc = fma(p.s0, LdgNC::ld(src + i), p.zero);
+// A tile.  The march keeps it in shared memory (registers are what it has least of).
+struct BrickTile {
+  int32_t pidx[3], x0, y0, zs, ze, xlen, ylen;  // its PE, its first cell, its planes zs .. ze - 1, its cells per plane
+  int32_t lo[3], hi[3];                         // the cells lo .. hi - 1 of its PE along each axis
+  int32_t k[3][2];  // delays of the PE's sides; transposed: of the neighbours' sides that read this PE's cells
+};
+
+__device__ __forceinline__ void tile_place(const StepParams &p, const BrickShape &b, int t, BrickTile *T) {
+  // x fastest, then y, then chunk, then PE
+  const int tx = t % b.tiles_x; t /= b.tiles_x;
+  const int ty = t % b.tiles_y; t /= b.tiles_y;
+  const int ch = t % b.chunks; t /= b.chunks;
+  T->pidx[0] = t % p.pe[0]; t /= p.pe[0];
+  T->pidx[1] = t % p.pe[1];
+  T->pidx[2] = t / p.pe[1];
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int pos = c[a] - pidx[a] * p.S[a];
-    for (int j = -H; j <= H; ++j) {
-      if (j == 0) continue;
-      if (p.use_pe[a] && ((pos + j < 0 && kn[a][0] > 0) || (pos + j >= p.S[a] && kn[a][1] > 0))) continue;
-      const int cj = wrap_coord(c[a] + j, p.n[a]);
-      acc = fma(p.s[a][j + H], LdgNC::ld(src + i + (int64_t)(cj - c[a]) * stride[a]), acc);
+    T->lo[a] = T->pidx[a] * p.S[a];
+    T->hi[a] = T->lo[a] + p.S[a];
+  }
+  T->x0 = T->lo[0] + tx * b.tx;
+  T->y0 = T->lo[1] + ty * b.rows;
+  T->zs = T->lo[2] + ch * b.zc;
+  T->ze = min(T->zs + b.zc, T->hi[2]);
+  T->xlen = min(b.tx, T->hi[0] - T->x0);
+  T->ylen = min(b.rows, T->hi[1] - T->y0);
+}
+
+template <int MODE>
+__device__ __forceinline__ void tile_delays(const StepParams &p, const uint8_t *keff, BrickTile *T) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int lo[3] = {T->pidx[0], T->pidx[1], T->pidx[2]}, hi[3] = {T->pidx[0], T->pidx[1], T->pidx[2]};
+    if (MODE == 1) {
+      lo[a] = lo[a] == 0 ? p.pe[a] - 1 : lo[a] - 1;
+      hi[a] = hi[a] + 1 == p.pe[a] ? 0 : hi[a] + 1;
+    }
+    T->k[a][0] = p.use_pe[a] ? keff[side_of<3>(p, lo, a, MODE == 1 ? 1 : 0)] : 0;
+    T->k[a][1] = p.use_pe[a] ? keff[side_of<3>(p, hi, a, MODE == 1 ? 0 : 1)] : 0;
+  }
+}
+
+// A thread's share of a plane's cells: kCore slots of the tile's own cells, row by row, then the cells around it -- left and
+// right of the rows, then below and above them -- so that the buffer points, which cost T FP64 operations each, fill few
+// warps.
+template <int H, int MODE>
+struct TileLoad {
+  int goff[kBrickSlots], code[kBrickSlots];  // cell within the plane; slot in the ring plane and delay
+  bool some;                                 // the warp has buffer points with a delay beside the tile
+  double v[kBrickSlots], hlev[kBrickSlots - kCore][H + 1];
+
+  __device__ __forceinline__ void setup(const StepParams &p, const BrickShape &b, const BrickTile &T, int tid) {
+    const int xlen = T.xlen, ylen = T.ylen;
+    bool buffers = false;
+#pragma unroll
+    for (int s = 0; s < kBrickSlots; ++s) {
+      int r, c, k = 0;
+      bool have;
+      if (s < kCore) {
+        const int l = tid + s * kBrickThreads;
+        have = l < ylen * xlen;
+        r = l / xlen;
+        c = l - r * xlen;
+      } else {
+        const int l = tid + (s - kCore) * kBrickThreads, side = 2 * H * ylen;
+        have = l < side + 2 * H * xlen;
+        if (l < side) {
+          const int hi = l >= H * ylen, m = l - hi * H * ylen;
+          r = m / H;
+          c = m - r * H + (hi ? xlen : -H);
+          if (hi ? T.x0 + c >= T.hi[0] : T.x0 + c < T.lo[0]) k = T.k[0][hi];
+        } else {
+          const int hi = l - side >= H * xlen, m = l - side - hi * H * xlen;
+          r = m / xlen;
+          c = m - r * xlen;
+          r += hi ? ylen : -H;
+          if (hi ? T.y0 + r >= T.hi[1] : T.y0 + r < T.lo[1]) k = T.k[1][hi];
+        }
+      }
+      const int cc = c + 4;  // columns -4 .. : group boundaries stay multiples of four
+      goff[s] = have ? wrap_coord(T.y0 + r, p.n[1]) * p.n[0] + wrap_coord(T.x0 + c, p.n[0]) : T.y0 * p.n[0] + T.x0;
+      code[s] = have ? ((r + H) * b.stride + cc + (cc >> 2)) | (k << 16) : b.plane - 1;  // a pad slot nobody reads
+      buffers = buffers || (have && k > 0);
+    }
+    some = __any_sync(0xffffffffu, buffers);
+  }
+
+  // Plane zz's values; of buffer points, levels n-k-m: fetched with the plane and combined after the sums in between.  A warp
+  // with a buffer point does it for all its halo slots (delay 0: level n, not used) without branches.
+  __device__ __forceinline__ void load(const StepParams &p, const double *__restrict__ un, int sn, int zz) {
+    const int64_t base = (int64_t)wrap_coord(zz, p.n[2]) * ((int64_t)p.n[0] * p.n[1]);
+    const double *src = un + base;
+#pragma unroll
+    for (int s = 0; s < kBrickSlots; ++s) v[s] = LdgNC::ld(src + goff[s]);
+    if (MODE != 1 && some) {
+#pragma unroll
+      for (int s = kCore; s < kBrickSlots; ++s) {
+        const int k = code[s] >> 16;
+        const double *h = p.ring + base + goff[s];
+        hlev[s - kCore][0] = LdgNC::ld(h + slot_back(sn, k, p.R) * p.ntot);
+        if (p.T > 1) {  // the time-expanded rows read H + 1 levels, the others one
+#pragma unroll
+          for (int m = 1; m <= H; ++m) hlev[s - kCore][m] = LdgNC::ld(h + slot_back(sn, k > 0 ? k + m : 0, p.R) * p.ntot);
+        }
+      }
     }
   }
+
+  __device__ __forceinline__ void extrapolate(const StepParams &p, const BrickTile &T, int sn, int zz) {
+    const int kz = zz < T.lo[2] ? T.k[2][0] : (zz >= T.hi[2] ? T.k[2][1] : 0);
+    if (MODE == 1) {  // what lies across a face with a delay goes to older levels (brick_faces_kernel)
+#pragma unroll
+      for (int s = 0; s < kBrickSlots; ++s)
+        if (s < kCore ? kz > 0 : (code[s] >> 16) > 0) v[s] = 0.0;
+    } else if (kz > 0) {  // a buffer plane: only the tile's own cells of it are read
+      const int64_t base = (int64_t)wrap_coord(zz, p.n[2]) * ((int64_t)p.n[0] * p.n[1]);
+#pragma unroll
+      for (int s = 0; s < kCore; ++s) v[s] = halo_value<LdgNC>(p, base + goff[s], sn, kz);
+    } else if (some) {
+#pragma unroll
+      for (int s = kCore; s < kBrickSlots; ++s) {
+        const int k = code[s] >> 16;  // halo_value's chain
+        double acc = fma(p.w[k][0], hlev[s - kCore][0], p.zero);
+        if (p.T > 1) {
+#pragma unroll
+          for (int m = 1; m <= H; ++m) acc = fma(p.w[k][m], hlev[s - kCore][m], acc);
+        }
+        v[s] = k > 0 ? acc : v[s];
+      }
+    }
+  }
+};
+
+// Four sums in fixed point: the taps in f3's order.
+template <int H>
+struct TileSums {
+  int64_t A[4], B[4], C[4];
+  __device__ __forceinline__ void centre(const FxTaps<6 * AT_MAX_H + 1> &t, int q, const int2 &f) {
+    A[q] = (int64_t)t.w1[0] * f.x;
+    B[q] = fx_mad(t.w1[0], f.y, kFxB0);
+    C[q] = fx_mad(t.w0[0], f.x, kFxC0);
+  }
+  __device__ __forceinline__ void tap(const FxTaps<6 * AT_MAX_H + 1> &t, int k, int q, const int2 &f) {
+    A[q] = fx_mad(t.w1[k], f.x, A[q]);
+    B[q] = fx_mad(t.w1[k], f.y, B[q]);
+    C[q] = fx_mad(t.w0[k], f.x, C[q]);
+  }
+  __device__ __forceinline__ void join() {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) A[q] = fx_join(A[q], B[q], C[q]);
+  }
+};
+__device__ __forceinline__ constexpr int tile_tap(int h, int a, int j) {  // f3's index of offset j != 0 of axis a
+  return 1 + 2 * h * a + (j < 0 ? j + h : j + h - 1);
+}
+
+// What becomes of the `valid` sums r of the points from i0: Adams-Bashforth's combination and the store, the transposed
+// step's, or (MODE 2) the sum galpha.
+template <int AB, int MODE>
+__device__ __forceinline__ void tile_finish(const StepParams &p, const BrickAdjoint &adj, bool aligned,
+                                            const double *__restrict__ un, double *__restrict__ out, int64_t n, int64_t i0,
+                                            int valid, double r[4], const AbLevels<1> old[4], double &galpha) {
+  if (MODE == 2) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < valid) galpha = fma(LdgNC::ld(adj.src + i0 + q), r[q], galpha);
+    return;
+  }
+  if (MODE == 1 && aligned) {  // the workspace is 16-byte aligned
+    double2 *o = reinterpret_cast<double2 *>(out + i0);
+    double2 lo = make_double2(r[0], r[1]), hi = make_double2(r[2], r[3]);
+    if (adj.ident) {
+      const double2 a = LdgNC::ld2(adj.ident + i0), c = LdgNC::ld2(adj.ident + i0 + 2);
+      lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
+    }
+    if (adj.add) {
+      const double2 a = o[0], c = o[1];
+      lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
+    }
+    o[0] = lo;
+    o[1] = hi;
+    if (adj.fresh) {
+      double2 *z = reinterpret_cast<double2 *>(adj.fresh + i0);
+      z[0] = z[1] = make_double2(0.0, 0.0);
+    }
+    return;
+  }
+  if (MODE == 1) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= valid) continue;
+      if (adj.ident) r[q] += LdgNC::ld(adj.ident + i0 + q);
+      out[i0 + q] = adj.add ? out[i0 + q] + r[q] : r[q];
+      if (adj.fresh) adj.fresh[i0 + q] = 0.0;
+    }
+    return;
+  }
+  if (AB) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= valid) continue;
+      const double u[1] = {LdgNC::ld(un + i0 + q)};
+      ab_combine<1>(p, n, i0 + q, u, r + q, old[q]);
+    }
+  }
+  if (aligned) {
+    reinterpret_cast<double2 *>(out + i0)[0] = make_double2(r[0], r[1]);
+    reinterpret_cast<double2 *>(out + i0)[1] = make_double2(r[2], r[3]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < valid) out[i0 + q] = r[q];
+  }
+}
+
+// The first `valid` points of a group as FMA chains: the centre, then the taps of x, y and z in offset order, across a face
+// with a delay the halo value (MODE 1: nothing, such a tap goes to older levels).  An axis' values are all in flight before
+// the first is used; r[q] of the points that are not there is any.
+template <int H, int MODE>
+__device__ __forceinline__ void tile_chain(const StepParams &p, const BrickTile &T, const double *__restrict__ un, int sn,
+                                           bool aligned, const int c[3], int valid, double r[4]) {
+  const int64_t nxy = (int64_t)p.n[0] * p.n[1], i = c[2] * nxy + (int64_t)c[1] * p.n[0] + c[0];
+  auto four = [&](int64_t cell, double v[4]) {
+    if (aligned) {
+      const double2 a = LdgNC::ld2(un + cell), b = LdgNC::ld2(un + cell + 2);
+      v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = LdgNC::ld(un + cell + (q < valid ? q : 0));
+    }
+  };
+  auto across = [&](int a, int at) { return at < T.lo[a] ? T.k[a][0] : (at >= T.hi[a] ? T.k[a][1] : 0); };
+  auto halo = [&](int64_t cell, int k) { return MODE == 1 ? 0.0 : halo_value<LdgNC>(p, cell, sn, k); };
+  {
+    double v[4 + 2 * H];
+    four(i, v + H);
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m) {  // the cells beside the valid points
+      const int at = c[0] + (m < H ? m - H : valid + m - H), k = across(0, at);
+      const int64_t cell = i + (wrap_coord(at, p.n[0]) - c[0]);
+      double x = LdgNC::ld(un + cell);
+      if (k > 0) x = halo(cell, k);
+      if (m < H) {
+        v[m] = x;
+      } else {
+        if (valid == 4) v[4 + m] = x;
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+          if (q == valid) v[q + m] = x;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      double acc = fma(p.s0, v[q + H], p.zero);
+#pragma unroll
+      for (int j = -H; j <= H; ++j)
+        if (j != 0) acc = fma(p.s[0][j + H], v[q + j + H], acc);
+      r[q] = acc;
+    }
+  }
+#pragma unroll
+  for (int a = 1; a < 3; ++a) {
+    const int64_t step = a == 1 ? (int64_t)p.n[0] : nxy;
+    auto cell = [&](int m) {
+      const int j = m < H ? m - H : m - H + 1;
+      return i + (int64_t)(wrap_coord(c[a] + j, p.n[a]) - c[a]) * step;
+    };
+    double v[2 * H][4];
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m) four(cell(m), v[m]);
+    if (c[a] - H < T.lo[a] || c[a] + H >= T.hi[a]) {
+#pragma unroll
+      for (int m = 0; m < 2 * H; ++m) {
+        const int k = across(a, c[a] + (m < H ? m - H : m - H + 1));
+        if (k > 0) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[m][q] = halo(cell(m) + (q < valid ? q : 0), k);
+        }
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = fma(p.s[a][m < H ? m : m + 1], v[m][q], r[q]);
+  }
+}
+
+// One point in the same way, with all of its values in flight together: few listed groups are waited for, not worked on.
+template <int H, int MODE>
+__device__ __forceinline__ double tile_point(const StepParams &p, const BrickTile &T, const double *__restrict__ un, int sn,
+                                             const int c[3]) {
+  const int64_t stride[3] = {1, (int64_t)p.n[0], (int64_t)p.n[0] * p.n[1]};
+  const int64_t i = c[2] * stride[2] + c[1] * stride[1] + c[0];
+  auto cell = [&](int a, int j) { return i + (int64_t)(wrap_coord(c[a] + j, p.n[a]) - c[a]) * stride[a]; };
+  double v[3][2 * H];
+  const double u = LdgNC::ld(un + i);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m) v[a][m] = LdgNC::ld(un + cell(a, m < H ? m - H : m - H + 1));
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (c[a] - H >= T.lo[a] && c[a] + H < T.hi[a]) continue;
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m) {
+      const int j = m < H ? m - H : m - H + 1;
+      const int k = c[a] + j < T.lo[a] ? T.k[a][0] : (c[a] + j >= T.hi[a] ? T.k[a][1] : 0);
+      if (k > 0) v[a][m] = MODE == 1 ? 0.0 : halo_value<LdgNC>(p, cell(a, j), sn, k);
+    }
+  }
+  double acc = fma(p.s0, u, p.zero);
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int m = 0; m < 2 * H; ++m) acc = fma(p.s[a][m < H ? m : m + 1], v[a][m], acc);
   return acc;
+}
+
+// *out += the block's sum of v, in a fixed order.
+template <int THREADS>
+__device__ __forceinline__ void block_total(double v, double *out) {
+  __shared__ double sums[THREADS / 32];
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+  if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = sums[0];
+    for (int w = 1; w < THREADS / 32; ++w) t += sums[w];
+    *out += t;
+  }
 }
 
 // MODE 0: the forward step.  MODE 1: the part of the transposed step that stays at level n, with the taps reversed; a
@@ -92,12 +402,14 @@ __device__ __noinline__ double transposed_point(const StepParams &p, const doubl
 // lambda x (the second-derivative taps of U^n), for which p.s0, p.s and p.f3 hold those taps; each block takes the same
 // tiles in the same order, so the sum is deterministic.
 template <int H, int AB, int MODE>
-__global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(const StepParams p, const BrickShape b,
-                                                                            const BrickAdjoint adj, const int64_t n_off,
+__global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(const __grid_constant__ StepParams p,
+                                                                            const __grid_constant__ BrickShape b,
+                                                                            const __grid_constant__ BrickAdjoint adj, const int64_t n_off,
                                                                             const int64_t *n_base) {
   constexpr int NR = 2 * H + 2;  // ring planes
   extern __shared__ int2 ring[];
-  __shared__ int mx[3], later[kBrickLater], n_later;
+  __shared__ int mx[3];
+  __shared__ BrickTile T;
   __shared__ FxPlanes planes;
   const int64_t n = n_off + (n_base ? *n_base : 0);
   const double *__restrict__ un = MODE == 1 ? adj.src : p.ring + slot_of(n, p.R) * p.ntot;
@@ -112,214 +424,33 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
                p.keff + ((n - 1) & 1) * p.nb);
   }
   double galpha = 0.0;
-  const int nx = p.n[0], ny = p.n[1], nz = p.n[2], sn = (int)slot_of(n, p.R);
-  const int64_t nxy = (int64_t)nx * ny;
-  for (int64_t tile = blockIdx.x; tile < b.blocks; tile += gridDim.x) {
-  // tile: x fastest, then y, then chunk, then PE
-  int pidx[3], x0, y0, zs, ze;
-  {
-    int t = (int)tile;
-    const int tx = t % b.tiles_x; t /= b.tiles_x;
-    const int ty = t % b.tiles_y; t /= b.tiles_y;
-    const int ch = t % b.chunks; t /= b.chunks;
-    pidx[0] = t % p.pe[0]; t /= p.pe[0];
-    pidx[1] = t % p.pe[1];
-    pidx[2] = t / p.pe[1];
-    x0 = pidx[0] * p.S[0] + tx * b.tx;
-    y0 = pidx[1] * p.S[1] + ty * b.rows;
-    zs = pidx[2] * p.S[2] + ch * b.zc;
-    ze = min(zs + b.zc, (pidx[2] + 1) * p.S[2]);
+  const int sn = (int)slot_of(n, p.R), lane = tid & 31, warp = tid >> 5;
+  const bool aligned = b.aligned != 0;
+  for (int tile = (int)blockIdx.x; tile < (int)b.blocks; tile += (int)gridDim.x) {
+  if (tid == 0) {
+    tile_place(p, b, tile, &T);
+    tile_delays<MODE>(p, keff, &T);
   }
-  const int px1 = (pidx[0] + 1) * p.S[0], py1 = (pidx[1] + 1) * p.S[1];
-  const int pz0 = pidx[2] * p.S[2], pz1 = pz0 + p.S[2];
-  const int xlen = min(b.tx, px1 - x0), ylen = min(b.rows, py1 - y0);
-  int kside[3][2];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    // the PE's own sides; transposed: the side of the neighbour across each face that reads this PE's cells
-    int lo[3] = {pidx[0], pidx[1], pidx[2]}, hi[3] = {pidx[0], pidx[1], pidx[2]};
-    if (MODE == 1) {
-      lo[a] = pidx[a] == 0 ? p.pe[a] - 1 : pidx[a] - 1;
-      hi[a] = pidx[a] + 1 == p.pe[a] ? 0 : pidx[a] + 1;
-    }
-    kside[a][0] = p.use_pe[a] ? keff[side_of<3>(p, lo, a, MODE == 1 ? 1 : 0)] : 0;
-    kside[a][1] = p.use_pe[a] ? keff[side_of<3>(p, hi, a, MODE == 1 ? 0 : 1)] : 0;
-  }
-  // This thread's share of a plane's cells: kCore slots of the tile's own cells, row by row, then the cells around it --
-  // left and right of the rows, then below and above them -- so that the buffer points, which cost T FP64 operations
-  // each, fill few warps.  goff: cell within the plane; code: slot in the ring plane, delay; -1: none.
-  int goff[kBrickSlots], code[kBrickSlots];
-  bool buffers = false;  // some of this thread's halo cells are buffer points with a delay
-#pragma unroll
-  for (int s = 0; s < kBrickSlots; ++s) {
-    int r, c, k = 0;
-    bool have;
-    if (s < kCore) {
-      const int l = tid + s * kBrickThreads;
-      have = l < ylen * xlen;
-      r = l / xlen;
-      c = l - r * xlen;
-    } else {
-      const int l = tid + (s - kCore) * kBrickThreads, side = 2 * H * ylen;
-      have = l < side + 2 * H * xlen;
-      if (l < side) {
-        const int hi = l >= H * ylen, m = l - hi * H * ylen;
-        r = m / H;
-        c = m - r * H + (hi ? xlen : -H);
-        if (hi ? x0 + c >= px1 : x0 + c < pidx[0] * p.S[0]) k = kside[0][hi];
-      } else {
-        const int hi = l - side >= H * xlen, m = l - side - hi * H * xlen;
-        r = m / xlen;
-        c = m - r * xlen;
-        r += hi ? ylen : -H;
-        if (hi ? y0 + r >= py1 : y0 + r < pidx[1] * p.S[1]) k = kside[1][hi];
-      }
-    }
-    const int cc = c + 4;  // columns -4 .. : group boundaries stay multiples of four
-    goff[s] = have ? wrap_coord(y0 + r, ny) * nx + wrap_coord(x0 + c, nx) : y0 * nx + x0;
-    code[s] = have ? ((r + H) * b.stride + cc + (cc >> 2)) | (k << 16) : b.plane - 1;  // a pad slot nobody reads
-    buffers = buffers || (have && k > 0);
-  }
-  // Buffer points: level n-k-m of halo slot s is hlev[s][m], fetched with the plane and combined after the sums in
-  // between.  A warp with a buffer point does it for all its halo slots (delay 0: level n, not used) without branches.
-  const bool some = __any_sync(0xffffffffu, buffers), deep = p.T > 1;
-  double v[kBrickSlots], hlev[kBrickSlots - kCore][H + 1];
-  auto load = [&](int zz) {
-    const int64_t base = (int64_t)wrap_coord(zz, nz) * nxy;
-    const double *src = un + base;
-#pragma unroll
-    for (int s = 0; s < kBrickSlots; ++s) v[s] = LdgNC::ld(src + goff[s]);
-    if (MODE != 1 && some) {
-#pragma unroll
-      for (int s = kCore; s < kBrickSlots; ++s) {
-        const int k = code[s] >> 16;
-        const double *h = p.ring + base + goff[s];
-        hlev[s - kCore][0] = LdgNC::ld(h + slot_back(sn, k, p.R) * p.ntot);
-        if (deep) {  // the time-expanded rows read H + 1 levels, the others one
-#pragma unroll
-          for (int m = 1; m <= H; ++m) hlev[s - kCore][m] = LdgNC::ld(h + slot_back(sn, k > 0 ? k + m : 0, p.R) * p.ntot);
-        }
-      }
-    }
-  };
-  auto extrapolate = [&](int zz) {
-    const int kz = zz < pz0 ? kside[2][0] : (zz >= pz1 ? kside[2][1] : 0);
-    if (MODE == 1) {  // what lies across a face with a delay goes to older levels (brick_faces_kernel)
-#pragma unroll
-      for (int s = 0; s < kBrickSlots; ++s)
-        if (s < kCore ? kz > 0 : (code[s] >> 16) > 0) v[s] = 0.0;
-    } else if (kz > 0) {  // a buffer plane: only the tile's own cells of it are read
-      const int64_t base = (int64_t)wrap_coord(zz, nz) * nxy;
-#pragma unroll
-      for (int s = 0; s < kCore; ++s) v[s] = halo_value<LdgNC>(p, base + goff[s], sn, kz);
-    } else if (some) {
-#pragma unroll
-      for (int s = kCore; s < kBrickSlots; ++s) {
-        const int k = code[s] >> 16;  // halo_value's chain
-        double acc = fma(p.w[k][0], hlev[s - kCore][0], p.zero);
-        if (deep) {
-#pragma unroll
-          for (int m = 1; m <= H; ++m) acc = fma(p.w[k][m], hlev[s - kCore][m], acc);
-        }
-        v[s] = k > 0 ? acc : v[s];
-      }
-    }
-  };
-  if (tid == 0) n_later = 0;
   if (tid < 3) mx[tid] = 0;
   if (tid < 8) planes.top[tid] = planes.cut[tid] = 0;
+  __syncthreads();
+  TileLoad<H, MODE> in;
+  in.setup(p, b, T, tid);
   FxRing scale;
   // this thread's points; a thread without any sums the tile's first group along
-  int row = tid / b.gx, grp = tid - row * b.gx;
-  const bool mine = row < ylen && 4 * grp < xlen;
-  row = mine ? row : 0;
-  grp = mine ? grp : 0;
-  const int nv = min(4, xlen - 4 * grp);
-  const int col = (row + H) * b.stride + 4 * grp + 4 + grp + 1;  // its slot in a ring plane (pad slot per four)
-  const int64_t cell0 = (int64_t)(y0 + row) * nx + x0 + 4 * grp;
-  // the FP64 chain for group g of tile row rr of plane o
-  auto chain = [&](int rr, int g, int o, double r[4]) {
-    if (MODE == 1) {
-      const int valid = min(4, xlen - 4 * g);
-#pragma unroll 1
-      for (int q = 0; q < valid; ++q) {
-        const int c[3] = {x0 + 4 * g + q, y0 + rr, o};
-        const double w = transposed_point<H>(p, un, pidx, kside, c);
-        r[0] = q == 0 ? w : r[0]; r[1] = q == 1 ? w : r[1]; r[2] = q == 2 ? w : r[2]; r[3] = q == 3 ? w : r[3];
-      }
-    } else if (b.aligned) {
-      double uc[4];
-      group_eval<3, H, LdgNC, false>(p, keff, un, n, x0 + 4 * g, y0 + rr, o, r, uc);
-    } else {
-      const int valid = min(4, xlen - 4 * g);
-      const int64_t i0 = (int64_t)o * nxy + (int64_t)(y0 + rr) * nx + x0 + 4 * g;
-#pragma unroll 1
-      for (int q = 0; q < valid; ++q) {
-        const int c[3] = {x0 + 4 * g + q, y0 + rr, o};
-        const double w = point_update<3, H, LdgNC>(p, keff, un, n, i0 + q, c);
-        r[0] = q == 0 ? w : r[0]; r[1] = q == 1 ? w : r[1]; r[2] = q == 2 ? w : r[2]; r[3] = q == 3 ? w : r[3];
-      }
-    }
-  };
-  // Adams-Bashforth combination and store of `valid` points from i0
-  auto finish = [&](int64_t i0, int valid, double r[4], const AbLevels<1> old[4]) {
-    if (MODE == 2) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < valid) galpha = fma(LdgNC::ld(adj.src + i0 + q), r[q], galpha);
-      return;
-    }
-    if (MODE == 1 && b.aligned) {  // the workspace is 16-byte aligned
-      double2 *o = reinterpret_cast<double2 *>(out + i0);
-      double2 lo = make_double2(r[0], r[1]), hi = make_double2(r[2], r[3]);
-      if (adj.ident) {
-        const double2 a = LdgNC::ld2(adj.ident + i0), c = LdgNC::ld2(adj.ident + i0 + 2);
-        lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
-      }
-      if (adj.add) {
-        const double2 a = o[0], c = o[1];
-        lo.x += a.x; lo.y += a.y; hi.x += c.x; hi.y += c.y;
-      }
-      o[0] = lo;
-      o[1] = hi;
-      if (adj.fresh) {
-        double2 *z = reinterpret_cast<double2 *>(adj.fresh + i0);
-        z[0] = z[1] = make_double2(0.0, 0.0);
-      }
-      return;
-    }
-    if (MODE == 1) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= valid) continue;
-        if (adj.ident) r[q] += LdgNC::ld(adj.ident + i0 + q);
-        out[i0 + q] = adj.add ? out[i0 + q] + r[q] : r[q];
-        if (adj.fresh) adj.fresh[i0 + q] = 0.0;
-      }
-      return;
-    }
-    if (AB) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= valid) continue;
-        const double u[1] = {LdgNC::ld(un + i0 + q)};
-        ab_combine<1>(p, n, i0 + q, u, r + q, old[q]);
-      }
-    }
-    if (b.aligned) {
-      reinterpret_cast<double2 *>(out + i0)[0] = make_double2(r[0], r[1]);
-      reinterpret_cast<double2 *>(out + i0)[1] = make_double2(r[2], r[3]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < valid) out[i0 + q] = r[q];
-    }
-  };
-  load(zs - H);
-  __syncthreads();
+  const int row = tid / b.gx, grp = tid - row * b.gx;
+  const bool mine = row < T.ylen && 4 * grp < T.xlen;
+  const int nv = min(4, mine ? T.xlen - 4 * grp : 4);
+  const int col = mine ? (row + H) * b.stride + 5 * grp + 5 : H * b.stride + 5;  // its slot in a ring plane (pad slot per four)
+  const int64_t cell0 = (int64_t)(T.y0 + (mine ? row : 0)) * p.n[0] + T.x0 + (mine ? 4 * grp : 0);
+  const int64_t nxy = (int64_t)p.n[0] * p.n[1];
+  const int zs = T.zs, ze = T.ze;
+  int heavy = 0;  // planes in a row with most groups listed
+  in.load(p, un, sn, zs - H);
   int wslot = 0, cslot = 0, m3 = 0;  // ring slots of plane i and of plane o - H of the output; i - (zs - H) mod 3
   for (int i = zs - H; i < ze + H + 2; ++i) {
     const int o = i - 2 - H;
+    bool list = false;
     if (o >= zs) {
       const int64_t i0 = (int64_t)o * nxy + cell0;
       AbLevels<1> old[4];
@@ -345,19 +476,10 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
           const uint32_t g1 = nv < 3 ? g0 : fx_upper(c4[2].x) | fx_upper(c4[3].x);
           far = MODE != 2 && min(g0, g1) < fx_least(kBrickGuard, lift);  // a sum over all points needs no local bits
         }
-        int64_t A[4], B[4], C[4];
         const FxTaps<6 * AT_MAX_H + 1> &t = p.f3;
+        TileSums<H> sum;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          A[q] = (int64_t)t.w1[0] * c4[q].x;
-          B[q] = fx_mad(t.w1[0], c4[q].y, kFxB0);
-          C[q] = fx_mad(t.w0[0], c4[q].x, kFxC0);
-        }
-        auto tap = [&](int k, int q, const int2 &f) {
-          A[q] = fx_mad(t.w1[k], f.x, A[q]);
-          B[q] = fx_mad(t.w1[k], f.y, B[q]);
-          C[q] = fx_mad(t.w0[k], f.x, C[q]);
-        };
+        for (int q = 0; q < 4; ++q) sum.centre(t, q, c4[q]);
         // x: cells -H .. 3 + H of the row; the pad slots lie before cells 0 and 4
 #pragma unroll
         for (int d = -H; d <= 3 + H; ++d) {
@@ -365,7 +487,7 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int j = d - q;  // tap j of point q reads cell q + j
-            if (j != 0 && j >= -H && j <= H) tap(1 + (j < 0 ? j + H : j + H - 1), q, f);
+            if (j != 0 && j >= -H && j <= H) sum.tap(t, tile_tap(H, 0, j), q, f);
           }
         }
 #pragma unroll
@@ -373,47 +495,56 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
           if (j == 0) continue;
           const int2 *s = mid + j * b.stride;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) tap(1 + 2 * H + (j < 0 ? j + H : j + H - 1), q, s[q]);
+          for (int q = 0; q < 4; ++q) sum.tap(t, tile_tap(H, 1, j), q, s[q]);
         }
 #pragma unroll
         for (int j = -H; j <= H; ++j) {
           if (j == 0) continue;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) tap(1 + 4 * H + (j < 0 ? j + H : j + H - 1), q, pl[H + j][q]);
+          for (int q = 0; q < 4; ++q) sum.tap(t, tile_tap(H, 2, j), q, pl[H + j][q]);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) A[q] = fx_join(A[q], B[q], C[q]);
+        sum.join();
         const int ex = E - 1023 - p.f3.sw;
         if (AB) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) r[q] = fx_to_any(A[q], ex);
+          for (int q = 0; q < 4; ++q) r[q] = fx_to_any(sum.A[q], ex);
         } else {
-          fx_results<4>(A, ex, r);
+          fx_results<4>(sum.A, ex, r);
         }
       }
-      bool put = mine;
-      if (mine && (far || !usable)) {
-        const int at = usable ? atomicAdd(&n_later, 1) : kBrickLater;
-        put = at >= kBrickLater;
-        if (put) chain(row, grp, o, r);
-        else later[at] = (o - zs) << 16 | row << 8 | grp;
+      list = mine && (far || !usable);
+      uint32_t who = __ballot_sync(0xffffffffu, list);
+      if (who != 0) {
+        int top = usable ? 0 : 1;  // sums of zeros are zero
+#pragma unroll
+        for (int q = o - H; q <= o + H; ++q) top |= planes.top[q & 7];
+        if (top == 0) {
+          who = 0;
+          list = false;
+          r[0] = r[1] = r[2] = r[3] = 0.0;
+        }
       }
-      if (put) finish(i0, nv, r, old);
+      if (lane == 0) p.listed[(tile * b.zc + (o - zs)) * kBrickWarps + warp] = who;
+      if (mine && !list) tile_finish<AB, MODE>(p, adj, aligned, un, out, n, i0, nv, r, old, galpha);
       cslot = cslot + 1 == NR ? 0 : cslot + 1;
     }
     if (i < ze + H) {
-      extrapolate(i);
+      in.extrapolate(p, T, sn, i);
       int mag = 0;
 #pragma unroll
-      for (int s = 0; s < kBrickSlots; ++s) mag = max(mag, fx_mag(v[s]));
+      for (int s = 0; s < kBrickSlots; ++s) mag = max(mag, fx_mag(in.v[s]));
       mag = __reduce_max_sync(0xffffffffu, mag);
       if ((tid & 31) == 0) atomicMax(&mx[m3], mag);
     }
-    if (i >= ze + H) {
-      if (i == ze + H) __syncthreads();  // the last plane stored is read in the next iteration
-      continue;
+    const int count = __syncthreads_count(list);
+    // a steep tile, not the planes around a fall of the scale: the rest of it is listed at once
+    heavy = 2 * count > T.ylen * ((T.xlen + 3) >> 2) ? heavy + (o - H > scale.until ? 3 : 1) : 0;
+    if (heavy >= 9) {
+      const uint32_t all = __ballot_sync(0xffffffffu, mine);
+      for (int z = o + 1 + lane; z < ze; z += 32) p.listed[(tile * b.zc + (z - zs)) * kBrickWarps + warp] = all;
+      break;
     }
-    __syncthreads();
+    if (i >= ze + H) continue;
     const int m = mx[m3];
     if (tid == 0) mx[m3 == 0 ? 2 : m3 - 1] = 0;  // read by all before this barrier, used again two planes on
     const bool ok = fx_plane_usable(m);
@@ -431,41 +562,122 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
       int2 *dst = ring + wslot * b.plane;
 #pragma unroll
       for (int s = 0; s < kBrickSlots; ++s) {
-        const Fx f = fx_split(fx_from(v[s], scale.E));
-        dst[code[s] & 0xffff] = make_int2(f.hi, f.lo);
+        const Fx f = fx_split(fx_from(in.v[s], scale.E));
+        dst[in.code[s] & 0xffff] = make_int2(f.hi, f.lo);
       }
     }
     wslot = wslot + 1 == NR ? 0 : wslot + 1;
     m3 = m3 == 2 ? 0 : m3 + 1;
-    if (i + 1 < ze + H) load(i + 1);
+    if (i + 1 < ze + H) in.load(p, un, sn, i + 1);
   }
   __syncthreads();
-#pragma unroll 1
-  for (int e = tid; e < min(n_later, kBrickLater); e += kBrickThreads) {
-    const int rr = (later[e] >> 8) & 0xff, g = later[e] & 0xff, o = zs + (later[e] >> 16), valid = min(4, xlen - 4 * g);
-    const int64_t i0 = (int64_t)o * nxy + (int64_t)(y0 + rr) * nx + x0 + 4 * g;
-    double r[4];
-    AbLevels<1> old[4];
-    if (AB) {
+  }
+  if (MODE == 2) block_total<kBrickThreads>(galpha, adj.g_blk + blockIdx.x);
+}
+
+// The groups that the march listed (a bit per group, four words per plane of a tile, every word written anew), as FMA
+// chains.  A block takes up to kListWords words, every gridDim.x-th one (tiles with many listed groups are spread), makes a
+// list of their groups in shared memory -- those away from the PE's faces from its front, those at a face, for which a warp
+// reads delayed levels, from its end -- and shares it out.  A launch of its own, started while the march ends: the march's
+// blocks have next to no L1 beside the ring and no registers to spare, a few of them hold most of a field's listed groups,
+// and past what they could list they held their barriers for the chains.  256^3 in 4^3 PEs, us per step (order 4 / 2; all
+// FP64 chains 438 / 235): a Gaussian of 13 cells 830 / 465 -> 637 / 372, a ball of ones in zeros 607 / 332 -> 228 / 149, noise
+// with spikes 832 / 457 -> 542 / 297; a field that is zero in half of the box 645 / 357 -> 287 / 198; smooth fields, with 0.5 %
+// of their groups listed, pay 10 us for it (226 -> 248, 160 -> 175).
+constexpr int kListThreads = 256;
+constexpr int kListWords = 512;  // 32 KB of list
+
+template <int H, int AB, int MODE>
+__global__ void __launch_bounds__(kListThreads, 2) brick_listed_kernel(const StepParams p, const BrickShape b,
+                                                                       const BrickAdjoint adj,
+                                                                       const int64_t n_off, const int64_t *n_base) {
+  __shared__ uint16_t list[kListWords * 32];
+  __shared__ uint32_t sums[kListThreads / 32];
+  cudaGridDependencySynchronize();
+  const int64_t n = n_off + (n_base ? *n_base : 0);
+  const int sn = (int)slot_of(n, p.R);
+  const double *__restrict__ un = MODE == 1 ? adj.src : p.ring + sn * p.ntot;
+  double *__restrict__ out = MODE == 1 ? adj.cur : p.ring + slot_of(n + 1, p.R) * p.ntot;
+  const uint8_t *keff = p.keff + (n & 1) * p.nb;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, per_tile = b.zc * kBrickWarps;
+  const int words = (int)b.blocks * per_tile;
+  double galpha = 0.0;
+  for (int w0 = (int)blockIdx.x; w0 < words; w0 += (int)gridDim.x * kListWords) {
+    // this thread's words: their groups away from faces and at faces
+    constexpr int W = kListWords / kListThreads;
+    uint32_t inner[W], face[W], count = 0;  // count: low half away from faces, high half at faces
 #pragma unroll
-      for (int q = 0; q < 4; ++q) ab_fetch<1>(p, n, i0 + (q < valid ? q : 0), old[q]);
+    for (int v = 0; v < W; ++v) {
+      const int64_t at = w0 + (int64_t)(tid * W + v) * gridDim.x;
+      const int w = (int)at;
+      inner[v] = at < words ? p.listed[w] : 0u;
+      face[v] = 0u;
+      if (inner[v] != 0) {
+        BrickTile T;
+        tile_place(p, b, w / per_tile, &T);
+        const int k = w % per_tile, z = T.zs + k / kBrickWarps;
+        if (z >= T.ze) inner[v] = 0;  // planes that a PE's last chunk has not: their words are not written
+        for (uint32_t left = inner[v]; left != 0; left &= left - 1) {
+          const int bit = __ffs(left) - 1, t = k % kBrickWarps * 32 + bit, row = t / b.gx;
+          const int x = T.x0 + 4 * (t - row * b.gx), y = T.y0 + row;
+          if (x - H < T.lo[0] || x + 3 + H >= T.hi[0] || y - H < T.lo[1] || y + H >= T.hi[1] || z - H < T.lo[2] || z + H >= T.hi[2])
+            face[v] |= 1u << bit;
+        }
+        inner[v] &= ~face[v];
+      }
+      count += __popc(inner[v]) | __popc(face[v]) << 16;
     }
-    chain(rr, g, o, r);
-    finish(i0, valid, r, old);
-  }
-  __syncthreads();
-  }
-  if (MODE == 2) {
-    __shared__ double sums[kBrickThreads / 32];  // block sum in a fixed order
-    for (int d = 16; d > 0; d >>= 1) galpha += __shfl_down_sync(0xffffffffu, galpha, d);
-    if ((tid & 31) == 0) sums[tid >> 5] = galpha;
+    uint32_t upto = count;
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, upto, d);
+      if (lane >= d) upto += v;
+    }
+    if (lane == 31) sums[warp] = upto;
     __syncthreads();
-    if (tid == 0) {
-      double t = sums[0];
-      for (int w = 1; w < kBrickThreads / 32; ++w) t += sums[w];
-      adj.g_blk[blockIdx.x] += t;
+    uint32_t all = 0, before = upto - count;
+    for (int q = 0; q < kListThreads / 32; ++q) {
+      if (q < warp) before += sums[q];
+      all += sums[q];
     }
+    uint32_t front = before & 0xffff, back = kListWords * 32 - 1 - (before >> 16);
+#pragma unroll
+    for (int v = 0; v < W; ++v) {
+      for (uint32_t left = inner[v]; left != 0; left &= left - 1)
+        list[front++] = (uint16_t)((tid * W + v) << 5 | (__ffs(left) - 1));
+      for (uint32_t left = face[v]; left != 0; left &= left - 1)
+        list[back--] = (uint16_t)((tid * W + v) << 5 | (__ffs(left) - 1));
+    }
+    __syncthreads();
+    // A group per thread, or, up to what keeps every thread busy once or twice, a point; those at faces, which take longest,
+    // first.
+    const int n_inner = (int)(all & 0xffff), n_face = (int)(all >> 16), each = n_inner + n_face <= kListThreads / 2 ? 4 : 1;
+    const int from = (n_face * each + 31) / 32 * 32;
+#pragma unroll 1
+    for (int e = tid; e < from + n_inner * each; e += kListThreads) {
+      if (e >= n_face * each && e < from) continue;
+      const int at = (e < from ? e : e - from) / each, entry = list[e < from ? kListWords * 32 - 1 - at : at];
+      const int w = w0 + (entry >> 5) * (int)gridDim.x, k = w % per_tile;
+      BrickTile T;
+      tile_place(p, b, w / per_tile, &T);
+      tile_delays<MODE>(p, keff, &T);
+      const int t = k % kBrickWarps * 32 + (entry & 31), row = t / b.gx, g = t - row * b.gx;
+      const int c[3] = {T.x0 + 4 * g + (each == 4 ? e & 3 : 0), T.y0 + row, T.zs + k / kBrickWarps};
+      const int valid = each == 4 ? min(1, T.x0 + T.xlen - c[0]) : min(4, T.xlen - 4 * g);
+      if (valid < 1) continue;
+      const int64_t i = ((int64_t)c[2] * p.n[1] + c[1]) * p.n[0] + c[0];
+      double r[4] = {0.0, 0.0, 0.0, 0.0};
+      AbLevels<1> old[4];
+      if (AB) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ab_fetch<1>(p, n, i + (q < valid ? q : 0), old[q]);
+      }
+      if (each == 4) r[0] = tile_point<H, MODE>(p, T, un, sn, c);
+      else tile_chain<H, MODE>(p, T, un, sn, b.aligned != 0, c, valid, r);
+      tile_finish<AB, MODE>(p, adj, each == 1 && b.aligned, un, out, n, i, valid, r, old, galpha);
+    }
+    __syncthreads();
   }
+  if (MODE == 2) block_total<kListThreads>(galpha, adj.g_blk + blockIdx.x);
 }
 
 // The part of the transposed step that goes to older levels: a cell within h of a face whose far side's reader has delay
@@ -609,7 +821,7 @@ bool brick_shape(const StepParams &p, BrickShape *b) {
   const bool grouped = p.n[0] % 4 == 0 && p.S[0] % 4 == 0;
   if (least > 0.95 * (double)p.ntot * (1 + 6 * p.h) * 1.08 / ((grouped ? 1.6 : 1.0) * sms * clock)) return false;
   b->aligned = p.n[0] % 4 == 0 && p.S[0] % 4 == 0 && reinterpret_cast<uintptr_t>(p.ring) % 16 == 0;
-  return b->blocks < (1ll << 31);
+  return b->blocks * b->zc * kBrickWarps < (1ll << 31);
 }
 
 template <int H, int AB, int MODE>
@@ -622,6 +834,23 @@ cudaError_t launch_brick_typed(const StepParams &p, const BrickShape &b, const B
     if (e != cudaSuccess) return e;
   }
   kernel<<<(unsigned)blocks, kBrickThreads, bytes, st>>>(p, b, adj, n, n_base);
+  const int64_t words = b.blocks * b.zc * kBrickWarps, want = (words + 63) / 64;
+  int64_t grid = 2 * brick_sms();
+  if (want < grid) grid = want;
+  if (MODE == 2 && blocks < grid) grid = blocks;
+  if (grid > 1) grid = (grid - 1) | 1;  // odd: every block's words come from all parts of the tiles
+  // launched while the march ends; it waits for the march's memory itself
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kListThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, brick_listed_kernel<H, AB, MODE>, p, b, adj, n, n_base);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
@@ -636,20 +865,21 @@ cudaError_t launch_brick_h(const StepParams &p, const BrickShape &b, const Brick
 // p with the taps t (centre, then each axis in offset order) in place of the step's.
 void set_taps(StepParams *p, double s0, const double s[3][2 * AT_MAX_H + 1], bool reversed) {
   const int h = p->h;
-  double t[6 * AT_MAX_H + 1] = {s0}, keep[3][2 * AT_MAX_H + 1];
-  int c = 1;
+  double keep[3][2 * AT_MAX_H + 1];
   for (int a = 0; a < 3; ++a)
-    for (int j = -h; j <= h; ++j) {
-      keep[a][j + h] = s[a][reversed ? h - j : h + j];
-      if (j != 0) t[c++] = keep[a][j + h];
-    }
+    for (int j = 0; j <= 2 * h; ++j) keep[a][j] = s[a][reversed ? 2 * h - j : j];
   p->s0 = s0;
   for (int a = 0; a < 3; ++a)
     for (int j = 0; j <= 2 * h; ++j) p->s[a][j] = keep[a][j];
-  fx_prepare(t, c, &p->f3);
+  fx_prepare_3d(p, s0, keep);
 }
 
 }  // namespace
+
+int64_t brick_listed_words(const StepParams &p) {
+  BrickShape b;
+  return brick_shape(p, &b) ? b.blocks * b.zc * kBrickWarps : 0;
+}
 
 bool launch_forward_brick(const StepParams &p, int64_t n, const int64_t *n_base, cudaStream_t st, cudaError_t *e) {
   BrickShape b;

@@ -120,10 +120,23 @@ struct StepParams {
   atfd::FxTaps<2 * AT_MAX_H + 1> fs, fb1, fb2;
   // 3D step in fixed point: s0, then the merged taps of x, y and z, each in offset order.
   atfd::FxTaps<6 * AT_MAX_H + 1> f3;
+  // 3D tiles: the groups that a step's march leaves to the chains (brick.cu), brick_listed_words words.
+  uint32_t *listed;
   // Division by the groups of a PE (S/4) and by its groups without the first and the last (1D).
   atfd::FastDiv div_g, div_in;
   atfd::FastDiv div_up;           // and, when the last one is partial, by ceil(S/4) - 3
 };
+
+// 3D: f3 of the taps s0, s (the centre, then each axis in offset order).
+inline void fx_prepare_3d(StepParams *p, double s0, const double s[3][2 * AT_MAX_H + 1]) {
+  const int h = p->h;
+  double t[6 * AT_MAX_H + 1] = {s0};
+  int c = 1;
+  for (int a = 0; a < 3; ++a)
+    for (int j = -h; j <= h; ++j)
+      if (j != 0) t[c++] = s[a][j + h];
+  atfd::fx_prepare(t, c, &p->f3);
+}
 
 // The modes of one axis at one time t, prepared on the host for the recurrences over k: sorted by wavenumber,
 // with A exp(-alpha kappa^2 t) and the phase phi - kappa c t folded into ac = A cos(.), as = A sin(.).  rot = 1 when
@@ -177,6 +190,7 @@ cudaError_t launch_small_steps(const StepParams &p, int64_t n, int64_t nsteps, c
 // 3D: the step in fixed point over tiles of the PEs (brick.cu); false: the shape or scheme is not one for it, nothing
 // launched.
 bool launch_forward_brick(const StepParams &p, int64_t n_off, const int64_t *n_base, cudaStream_t st, cudaError_t *e);
+int64_t brick_listed_words(const StepParams &p);
 // Backward step n of a 3D linear problem on the same tiles: the transposed step on the adjoint ring lam (Rl slots, levels
 // down to n - reach), with alpha the sum of dJ/dalpha's terms into g_blk (nblk sums); f: forward parameters whose ring
 // holds the levels the alpha term reads; akeff: the sweep's delay buffers (step n's in place, step n-1's drawn); mu:

@@ -94,3 +94,52 @@ def test_a_tiled_step_and_its_transpose_cell_by_cell(name, make, kind, size):
     n = 1 + 3 * spec["order"]
     _check(got, u0.astype(np.longdouble), _taps(spec), n)
     _check(g, lam.astype(np.longdouble), _taps(spec), n, reverse=True)
+
+
+SPLIT = [
+    ("o2_ragged", lambda: W.wl_3d([150, 126, 90], [3, 3, 2], 2, 3, 0, 911, c=(0.3, 0.2, 0.1))[0]),
+    ("o4", lambda: W.wl_3d([128, 128, 128], [2, 2, 2], 4, 3, 0, 912, c=(0.3, 0.2, 0.1))[0]),
+    ("o4_ab2", lambda: W.wl_3d([128, 128, 128], [2, 2, 2], 4, 3, 0, 913, c=(0.3, 0.2, 0.1), tsteps=2,
+                               dt=0.02 * W.dx_of(128) ** 2 / 0.05)[0]),
+]
+
+
+@pytest.mark.parametrize("kind", ["half_zero", "ball", "pulse", "one_steep_tile"])
+@pytest.mark.parametrize("name,make", SPLIT, ids=[s[0] for s in SPLIT])
+def test_tiles_with_few_many_and_all_groups_listed_match_the_oracle(name, make, kind):
+    """Groups that the tiles leave to the chains, in some planes of a tile, in most, in the rest of one: across faces with
+    delays, in partial groups.  Bars as for the other routes: 1e-12 of the largest value, and 256 ulp of the largest value
+    that a cell can depend on."""
+    import os
+
+    import oracle
+    from paper_1702_00496_gb300 import Solver
+    spec, steps = make(), 7
+    cfg = oracle.Config(spec)
+    rng = np.random.default_rng(spec["seed"])
+    x = [(np.arange(n) / n - 0.5) for n in cfg.shape]
+    r2 = x[0][:, None, None] ** 2 + x[1][None, :, None] ** 2 + x[2][None, None, :] ** 2
+    noise = 1.0 + 0.1 * rng.standard_normal(cfg.shape)
+    if kind == "half_zero":
+        u0 = np.where(x[2][None, None, :] > 0.11, noise, 0.0)
+    elif kind == "ball":
+        u0 = np.where(r2 < 0.06, noise, 0.0)
+    elif kind == "pulse":
+        u0 = noise * np.exp(-r2 / 0.002)
+    else:
+        u0 = noise.copy()
+        u0[10:40, 5:20, 3:30] *= 10.0 ** rng.uniform(-12, 0, (30, 15, 27))
+    s = Solver(spec, log_steps=steps)
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.step(steps)
+    s.sync()
+    u, d = s.field().cpu().numpy().copy(), s.delays().cpu().numpy().copy()
+    s.close()
+    ref, dref, _ = oracle.run(oracle.Config(spec), steps, threads=os.cpu_count() or 1, u0=u0)
+    assert np.array_equal(d, dref)
+    assert np.abs(u - ref).max() <= 1e-12 * np.abs(ref).max()
+    m = np.abs(u0)
+    for ax in range(3):
+        reach = spec["order"] // 2 * steps
+        m = np.max([np.roll(m, k, ax) for k in range(-reach, reach + 1)], axis=0)
+    assert (np.abs(u - ref) <= 256 * 2.0 ** -52 * np.maximum(m, np.abs(ref))).all()
