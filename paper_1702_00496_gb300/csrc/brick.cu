@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
         {
           const uint32_t g0 = fx_upper(c4[0].x) | fx_upper(c4[1].x);
           const uint32_t g1 = nv < 3 ? g0 : fx_upper(c4[2].x) | fx_upper(c4[3].x);
-          far = MODE != 2 && min(g0, g1) < fx_least(kBrickGuard, lift);  // a sum over all points needs no local bits
+          far = min(g0, g1) < fx_least(kBrickGuard, lift);
         }
         const FxTaps<6 * AT_MAX_H + 1> &t = p.f3;
         TileSums<H> sum;

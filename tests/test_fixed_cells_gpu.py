@@ -143,3 +143,29 @@ def test_tiles_with_few_many_and_all_groups_listed_match_the_oracle(name, make, 
         reach = spec["order"] // 2 * steps
         m = np.max([np.roll(m, k, ax) for k in range(-reach, reach + 1)], axis=0)
     assert (np.abs(u - ref) <= 256 * 2.0 ** -52 * np.maximum(m, np.abs(ref))).all()
+
+
+@pytest.mark.parametrize("bits", [0, 12, 24, 36, 48])
+@pytest.mark.parametrize("name,make", [t for t in TILES if t[0] != "o4_ab2"], ids=[t[0] for t in TILES if t[0] != "o4_ab2"])
+def test_the_diffusivity_gradient_of_a_field_that_is_small_where_the_seed_is_not(name, make, bits):
+    """dJ/dalpha of one step is the sum of lambda dt D2 U over the cells, and lambda here is nonzero only in a box where U is
+    2^-bits of what it is elsewhere in the same tiles.  Each term is held to its own stencil as above, the sum of 512 terms
+    to 512 roundings more."""
+    from paper_1702_00496_gb300 import Solver
+    spec = make()
+    shape = tuple(spec["n"][::-1])
+    rng = np.random.default_rng([spec["seed"], bits])
+    u0 = rng.uniform(0.5, 1.0, shape)
+    u0[40:60, 40:60, 40:60] *= 2.0 ** -bits
+    lam = np.zeros(shape)
+    lam[46:54, 46:54, 46:54] = rng.standard_normal((8, 8, 8))
+    s = Solver(spec)
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.adjoint_forward(1, 1)
+    _, ga = s.adjoint_backward(torch.as_tensor(lam, device="cuda"), True)
+    s.close()
+    q = [(spec["dt"] * np.array(CD2[spec["order"]]) / (2.0 * np.pi / n) ** 2).astype(np.longdouble) for n in spec["n"]]
+    f, m = _apply(u0.astype(np.longdouble), q)
+    n = 1 + 3 * spec["order"]
+    bar = (2 * n + 7 + 512) * np.longdouble(2.0) ** -53 * (np.abs(lam) * m).sum() * sum(np.abs(t).sum() for t in q)
+    assert abs(np.longdouble(ga) - (lam * f).sum()) <= bar
