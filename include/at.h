@@ -159,10 +159,15 @@ int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_len, uint8_t 
  * time; the delays, the delay log and the levels a later step reads at delayed levels are those of single steps.
  * Blocks start at the first step of each call (and of each captured graph inside it, 48 steps for K = 4), so the
  * same steps split into other calls give results equal up to rounding, not bit for bit.
- * Stencil sums run in block fixed point: a window's values scaled to its largest one, 62 bits each, exact to 2^-60 of
- * that value before the one rounding of the result; windows that fall steeply, hold infinities or NaN or lie at the
- * ends of the exponent range are summed as FP64 chains (single steps of fewer than
- * 196608 points whose PE width is no multiple of 4 are chains throughout).  A problem of up to 2048 points without blocks of K >= 3 runs a call's steps in
+ * Stencil sums run in block fixed point: values scaled to the largest one of their window (of a tile in blocks and in 3D),
+ * 62 bits each, weights to 2^-60 of their sum.  Before the one rounding of the result a sum is off by a few 2^-61 of that
+ * largest value; in blocks whose values lie within a factor of four, where part of it is FP32, by 2^-54 rms and 2^-51.5 at
+ * worst, which is under the FMA chain's own error.  Windows and groups whose own values are far below it, and such as hold
+ * infinities or NaN or lie at the ends of the exponent range, are summed as FP64 chains (single steps of fewer than 196608
+ * points whose PE width is no multiple of 4 are chains throughout).  So every cell is good to a few ulp of the largest value
+ * of its own stencil; a cell that is smaller than those beside it does not keep 53 bits of its own, as it would in a chain
+ * with small taps.
+ * A problem of up to 2048 points without blocks of K >= 3 runs a call's steps in
  * one launch.
  * Adams-Bashforth runs from a caller's field take their first ts-1 steps (fewer stored levels, other weights) as
  * single launches; every later step -- every step after the analytic pre-history -- has all ts levels (with ts = 2

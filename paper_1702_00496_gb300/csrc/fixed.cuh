@@ -30,11 +30,14 @@
 
 namespace atfd {
 
-// The cross terms, 2^-31 of A, can also be summed in FP32 (fx_mad_f32: one integer multiply-add and two FFMA per tap
-// instead of three multiply-adds, half the issue time).  Their rounding is then 2^-57 of the window's largest value:
-// under an FMA chain's error where every value of the window is within kFxNear bits of the largest.
+// The cross terms, 2^-31 of A, can also be summed in FP32 (fx_cross: one integer multiply-add and two FFMA per tap instead
+// of three multiply-adds, half the issue time).  Each of those FFMA then rounds at 2^-24 of its sum, 2^-55 of the window's
+// largest value and less: before the one rounding of the result 2^-54 rms and up to 2^-51.5 for the 17 taps of four steps at
+// order 4.  That is still under the FMA chain's error, rms and at worst, as long as every value of the window lies within
+// kFxNear bits of the largest and the taps go from the outermost pair to the centre, in a sum for either part
+// (test_fixed_cross_host.py; in one sum, in offset order, it was above the chain's from two bits on).
 constexpr int kFxGuard = 8;      // bits of a window's range within which the fixed-point sum is at least as exact
-constexpr int kFxNear = 2;       // the same with the cross terms in FP32
+constexpr int kFxNear = 1;       // the same with the cross terms in FP32
 constexpr int kFxLowBits = 29;   // bits of a weight's low part
 
 // Can windows whose largest value has biased exponent E be summed in fixed point?  Not with infinities or NaN (2047);
@@ -243,6 +246,30 @@ struct FxTaps {
   float f1[N], f0[N];
   int32_t sw, ok;
 };
+
+// The FP32 sums of the cross terms, of the values' lower and upper words, and what they make of A.
+struct FxCross {
+  float lo, hi;
+};
+template <int N>
+AT_FX_HD void fx_cross(FxCross &c, const FxTaps<N> &t, int j, float lo, float hi) {
+#if defined(__CUDA_ARCH__)
+  c.lo = fmaf(t.f1[j], lo, c.lo);
+  c.hi = fmaf(t.f0[j], hi, c.hi);
+#else
+  c.lo = __builtin_fmaf(t.f1[j], lo, c.lo);
+  c.hi = __builtin_fmaf(t.f0[j], hi, c.hi);
+#endif
+}
+AT_FX_HD int64_t fx_join_cross(int64_t A, const FxCross &c) {
+#if defined(__CUDA_ARCH__)
+  return A + (int64_t)(__float2int_rn(c.lo) + __float2int_rn(c.hi)) * 8;
+#else
+  return A + (int64_t)(__builtin_lrintf(c.lo) + __builtin_lrintf(c.hi)) * 8;
+#endif
+}
+// Tap m of n in the order that adds the largest terms last: the outermost pair, the next one, ..., the centre (n odd).
+AT_FX_HD constexpr int fx_inward(int m, int n) { return m & 1 ? n - 1 - m / 2 : m / 2; }
 
 template <int N>
 inline void fx_prepare(const double *w, int n, FxTaps<N> *t, const double *w_low = nullptr) {

@@ -198,21 +198,21 @@ __device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, 
 #pragma unroll
   for (int q0 = 0; q0 < C; q0 += 4) {
     int64_t A[4], B[4], D[4];
-    float c[4];
+    FxCross c[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       A[q] = 0; B[q] = kFxB0; D[q] = kFxC0;
-      c[q] = 0.0f;
+      c[q] = {0.0f, 0.0f};
     }
 #pragma unroll
-    for (int j = 0; j <= 2 * TK; ++j) {
+    for (int m = 0; m <= 2 * TK; ++m) {
+      const int j = fx_inward(m, 2 * TK + 1);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = q0 + q + j;
         A[q] = fx_mad(t.w1[j], w[i].x, A[q]);
         if (F32) {
-          c[q] = fmaf(t.f1[j], __int_as_float(w[i].y), c[q]);
-          c[q] = fmaf(t.f0[j], h[i], c[q]);
+          fx_cross(c[q], t, j, __int_as_float(w[i].y), h[i]);
         } else {
           B[q] = fx_mad(t.w1[j], w[i].y, B[q]);
           D[q] = fx_mad(t.w0[j], w[i].x, D[q]);
@@ -220,7 +220,7 @@ __device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, 
       }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) A[q] = F32 ? A[q] + (int64_t)__float2int_rn(c[q]) * 8 : fx_join(A[q], B[q], D[q]);
+    for (int q = 0; q < 4; ++q) A[q] = F32 ? fx_join_cross(A[q], c[q]) : fx_join(A[q], B[q], D[q]);
     fx_results<4>(A, ex, r + q0);
   }
 }
