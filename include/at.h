@@ -162,11 +162,11 @@ int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_len, uint8_t 
  * Stencil sums run in block fixed point: values scaled to the largest one of their window (of a tile in blocks and in 3D),
  * 62 bits each, weights to 2^-60 of their sum.  Before the one rounding of the result a sum is off by a few 2^-61 of that
  * largest value; in blocks whose values lie within a factor of four, where part of it is FP32, by 2^-54 rms and 2^-51.5 at
- * worst, which is under the FMA chain's own error.  Windows and groups whose own values are far below it, and such as hold
- * infinities or NaN or lie at the ends of the exponent range, are summed as FP64 chains (single steps of fewer than 196608
- * points whose PE width is no multiple of 4 are chains throughout).  So every cell is good to a few ulp of the largest value
- * of its own stencil; a cell that is smaller than those beside it does not keep 53 bits of its own, as it would in a chain
- * with small taps.
+ * worst, which is under the FMA chain's own error.  1D cells whose sum (Adams-Bashforth, Burgers: whose value) is so small
+ * beside it that a chain of FP64 operations could be more exact are summed as that chain, and so is what holds infinities
+ * or NaN or lies at the ends of the exponent range (single steps of fewer than 196608 points whose PE width is no multiple
+ * of 4 are chains throughout).  3D groups of four go by their values and are good to a few ulp of the largest value of each
+ * cell's own stencil: a cell that is much smaller than those beside it does not keep 53 bits of its own there.
  * A problem of up to 2048 points without blocks of K >= 3 runs a call's steps in
  * one launch.
  * Adams-Bashforth runs from a caller's field take their first ts-1 steps (fewer stored levels, other weights) as

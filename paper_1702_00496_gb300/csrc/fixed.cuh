@@ -14,10 +14,13 @@
 //            window's largest value for all taps together, is left out.
 //            R = A + B 2^-32 + C 2^-29 = sum W X 2^-61, rounded once to the nearest FP64 value R 2^(E - 1023 - sw).
 //
-// The error of R is below 2^-60 of the window's largest value times sum |w|, then there is one rounding; an FMA chain
-// of n terms rounds n times at 2^-53 of its partial sums.  A cell whose own neighbourhood is smaller than the window's
-// largest value by more than 2^-kFxGuard would lose by it: callers test that and take the FMA chain there, as they do
-// for windows that hold an infinity or a NaN, or that lie at the ends of the exponent range (fx_usable).
+// R is off by a few units: at most one for the cut values and one for the joins, a quarter per tap for w0 lo and half of
+// |X| 2^-61 per tap for its rounded weight.  Then there is one rounding, where an FMA chain of n terms rounds n times at 2^-53
+// of its partial sums.  A cell that is small against the window's largest value loses by it, so callers look at the sum
+// itself (1D; kFxLeast) or, where it is a small difference that is added to the cell's value, at that value: from 2^53 units
+// on the result's own rounding is one of them.  3D tiles look at two neighbours' values (brick.cu).  Cells that are too
+// small take the FMA chain, as do windows that hold an infinity or a NaN, or that lie at the ends of the exponent range
+// (fx_usable).
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -36,8 +39,9 @@ namespace atfd {
 // order 4.  That is still under the FMA chain's error, rms and at worst, as long as every value of the window lies within
 // kFxNear bits of the largest and the taps go from the outermost pair to the centre, in a sum for either part
 // (test_fixed_cross_host.py; in one sum, in offset order, it was above the chain's from two bits on).
-constexpr int kFxGuard = 8;      // bits of a window's range within which the fixed-point sum is at least as exact
-constexpr int kFxNear = 1;       // the same with the cross terms in FP32
+constexpr uint32_t kFxLeast = 1u << 21;      // upper word of a sum that is at least as exact as the chain
+constexpr uint32_t kFxLeastNear = 1u << 27;  // the same with the cross terms in FP32, for windows ...
+constexpr int kFxNear = 1;                   // ... whose values lie within these bits of the largest
 constexpr int kFxLowBits = 29;   // bits of a weight's low part
 
 // Can windows whose largest value has biased exponent E be summed in fixed point?  Not with infinities or NaN (2047);
@@ -161,15 +165,27 @@ AT_FX_HD double fx_to_any(int64_t R, int ex) {
 #endif
 }
 
-// N results at once: the rare ones below 2^32 are done again.
+// N results at once; returns the upper word of the smallest |R|, below 2^32 of which (0) a result is not valid.
 template <int N>
-AT_FX_HD void fx_results(const int64_t R[N], int ex, double r[N]) {
+AT_FX_HD uint32_t fx_results_wide(const int64_t R[N], int ex, double r[N]) {
   uint32_t small = 0xffffffffu;
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif
-  for (int q = 0; q < N; ++q) r[q] = fx_to_wide(R[q], ex, &small);
-  if (small == 0) {
+  for (int q = 0; q < N; ++q) {
+    r[q] = fx_to_wide(R[q], ex, &small);
+#if !defined(__CUDA_ARCH__)
+    const uint32_t up = (uint32_t)((uint64_t)(R[q] < 0 ? -R[q] : R[q]) >> 32);
+    small = up < small ? up : small;
+#endif
+  }
+  return small;
+}
+
+// The same where such results are valid too: the rare ones are done again.
+template <int N>
+AT_FX_HD void fx_results(const int64_t R[N], int ex, double r[N]) {
+  if (fx_results_wide<N>(R, ex, r) == 0) {
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif

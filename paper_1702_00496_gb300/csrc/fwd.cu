@@ -162,13 +162,20 @@ __device__ __forceinline__ void zone_steps(const StepParams &p, int64_t n, int s
   }
 }
 
-// One inner cell of a block as an FP64 chain: U^{n+K}_x = sum ck_j U^n_{x+j}, the centre first, then j ascending.
+// One inner cell of a block as an FP64 chain: U^{n+K}_x = sum ck_j U^n_{x+j}, the centre first, then j ascending.  The cells of
+// a warp are consecutive ones, or some of them.
 template <int TK>
 __device__ __noinline__ double block_cell(const StepParams &p, const double *__restrict__ u0, int x) {
   const int nx = p.n[0];
   double acc = fma(p.ck[TK], LdgNC::ld(u0 + x), p.zero);
-  for (int j = -TK; j <= TK; ++j)
-    if (j != 0) acc = fma(p.ck[j + TK], LdgNC::ld(u0 + wrap_coord(x + j, nx)), acc);
+  if (x >= TK && x + TK < nx) {
+#pragma unroll
+    for (int j = -TK; j <= TK; ++j)
+      if (j != 0) acc = fma(p.ck[j + TK], LdgNC::ld(u0 + x + j), acc);
+  } else {
+    for (int j = -TK; j <= TK; ++j)
+      if (j != 0) acc = fma(p.ck[j + TK], LdgNC::ld(u0 + wrap_coord(x + j, nx)), acc);
+  }
   return acc;
 }
 
@@ -185,9 +192,11 @@ constexpr int block_warp_bytes() {  // of a warp, for a zone or a tile
 }
 
 // The C outputs of a lane from its window in shared memory, four at a time (independent chains for the pipe's latency).
-// F32: the low parts are there as FP32 and the cross terms are summed in FP32.
+// F32: the low parts are there as FP32 and the cross terms are summed in FP32.  Returns a bit for every four cells that are
+// for the chain (fixed.cuh, kFxLeast).
 template <int TK, int C, bool F32, int NT>
-__device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, int lane, int ex, double r[C]) {
+__device__ __forceinline__ uint32_t block_sums(const FxTaps<NT> &t, const int2 *sm, int lane, int ex, double r[C]) {
+  uint32_t small = 0;
   int2 w[C + 2 * TK];
   float h[C + 2 * TK];
 #pragma unroll
@@ -221,8 +230,9 @@ __device__ __forceinline__ void block_sums(const FxTaps<NT> &t, const int2 *sm, 
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) A[q] = F32 ? fx_join_cross(A[q], c[q]) : fx_join(A[q], B[q], D[q]);
-    fx_results<4>(A, ex, r + q0);
+    if (fx_results_wide<4>(A, ex, r + q0) < (F32 ? kFxLeastNear : kFxLeast)) small |= 1u << (q0 / 4);
   }
+  return small;
 }
 
 // A block: zones near the PE boundaries, inner cells U^{n+K} = ck * U^n.
@@ -284,8 +294,9 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
     }
     const int E = __reduce_max_sync(0xffffffffu, hi) >> 20;
     const bool near = (__reduce_min_sync(0xffffffffu, lo) >> 20) >= E - kFxNear;
-    bool fixed = p.fck.ok && fx_usable(E);  // the same for the whole warp
+    const bool fixed = p.fck.ok && fx_usable(E);  // the same for the whole warp
     double r[C];
+    uint32_t chain = 0;  // a bit for every four of this lane's cells that are for the chain
     __syncwarp();
     if (fixed) {
 #pragma unroll
@@ -296,25 +307,15 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
         if (q < C || lane < 2 * TK) sm[i + i / C] = make_int2(f.hi, low);
       }
       __syncwarp();
-      if (near) {
-        block_sums<TK, C, true>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
-      } else {
-        // every cell must have a value within kFxGuard bits of the tile's largest one in its own window of TK cells
-        // either side: two cells of each run are looked at, and no cell of the run is further than TK from either
-        constexpr int G = TK < 3 ? 2 : (C < 8 || TK < 6 ? 4 : 8);
+      if (near) chain = block_sums<TK, C, true>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
+      else chain = block_sums<TK, C, false>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
+    } else {
+      int low = 0;
 #pragma unroll
-        for (int g = 0; g < C; g += G) {
-          const int a = C * lane + TK + g + G / 8, b = C * lane + TK + g + G - 1 - G / 8;
-          const int ha = sm[a + a / C].x, hb = sm[b + b / C].x;
-          if ((((ha ^ (ha >> 31)) | (hb ^ (hb >> 31))) >> (29 - kFxGuard)) == 0) fixed = false;
-        }
-        if (fixed) block_sums<TK, C, false>(p.fck, sm, lane, E - 1023 - p.fck.sw, r);
-      }
-    }
-    if (!fixed) {
+      for (int q = 0; q <= C; ++q) low |= fx_mag(v[q]) | fx_word(v[q], 0);
+      chain = __any_sync(0xffffffffu, low != 0) ? ~0u : 0u;  // sums of zeros are zero, as the chain's
 #pragma unroll
-      for (int q = 0; q < C; ++q)
-        if (C * lane + q < len) r[q] = block_cell<TK>(p, u0, x0 + C * lane + q);
+      for (int q = 0; q < C; ++q) r[q] = 0.0;
     }
     __syncwarp();
     double *ro = reinterpret_cast<double *>(sm) + lane * (C + 1);
@@ -323,7 +324,14 @@ __global__ void __launch_bounds__(256, 3) forward_block_kernel(const StepParams 
     __syncwarp();
     ro = reinterpret_cast<double *>(sm);
     double *dst = out + x0 + lane;
-    if (len == Tile::CELLS) {
+    if (__any_sync(0xffffffffu, chain != 0)) {
+#pragma unroll 1
+      for (int q = 0; q < C; ++q) {
+        const int i = lane + 32 * q;
+        const uint32_t owner = __shfl_sync(0xffffffffu, chain, i / C);
+        if (i < len) dst[32 * q] = owner >> (i % C / 4) & 1 ? block_cell<TK>(p, u0, x0 + i) : ro[i + i / C];
+      }
+    } else if (len == Tile::CELLS) {
 #pragma unroll
       for (int q = 0; q < C; ++q) dst[32 * q] = ro[lane + 32 * q + (lane + 32 * q) / C];
     } else {

@@ -274,8 +274,9 @@ __device__ __forceinline__ void ab_combine(const StepParams &p, int64_t n, int64
 // the FP64 pipe can do meanwhile stays with it: the outermost pair of taps of an Euler step (fx_reach), the
 // combination of an Adams-Bashforth step.
 //
-// A group is taken only when both halves of it hold a value within kFxGuard bits of the window's largest; the others
-// (and windows that hold infinities or NaN, or lie at the ends of the exponent range) go through the chain.
+// A group is taken only when its four sums (Adams-Bashforth, Burgers: its four values) are large enough against the window
+// for that (fixed.cuh, kFxLeast); the others, and windows that hold infinities or NaN or lie at the ends of the exponent
+// range, go through the chain.
 
 // x window of a 1D group: cells x0-W .. x0+3+W, buffer points replaced by the halo values of step n (its level is in
 // slot sn).
@@ -307,15 +308,21 @@ __device__ __forceinline__ void window_1d(const StepParams &p, const uint8_t *__
   }
 }
 
-// Scale of a 1D window (the cells within HI of the group), or -1 when the group goes through the chain.
+// Exponent of the largest value of a 1D window (the cells within HI of the group).
 template <int W, int HI>
-__device__ __forceinline__ int window_scale(const double v[4 + 2 * W]) {
+__device__ __forceinline__ int window_exponent(const double v[4 + 2 * W]) {
   int mag = 0;
 #pragma unroll
   for (int t = W - HI; t <= W + 3 + HI; ++t) mag = max(mag, fx_mag(v[t]));
-  const int E = mag >> 20;
-  const int near = min(max(fx_mag(v[W]), fx_mag(v[W + 1])), max(fx_mag(v[W + 2]), fx_mag(v[W + 3]))) >> 20;
-  return fx_usable(E) && near >= E - kFxGuard ? E : -1;
+  return mag >> 20;
+}
+
+// Are the four values x large enough for a sum with taps t that is added to them?  A unit of the sum is 2^(61 - sw) of theirs.
+template <int NT>
+__device__ __forceinline__ bool values_enough(const FxTaps<NT> &t, const Fx x[4]) {
+  const int more = max(61 - t.sw, 0);
+  const uint32_t least = more < 8 ? kFxLeast << more : 0x7fffffffu;
+  return min(min(fx_upper(x[0].hi), fx_upper(x[1].hi)), min(fx_upper(x[2].hi), fx_upper(x[3].hi))) >= least;
 }
 
 // R of the four points for the 2 HI + 1 taps t; x[i] is cell i - HI of the group.
@@ -351,13 +358,20 @@ template <int H, bool AB, int KIND>
 __device__ __forceinline__ bool group_fixed(const StepParams &p, const double v[XWin<H>::N], double r[4]) {
   constexpr int W = XWin<H>::W, HI = KIND ? H : fx_reach(H, AB);
   if (KIND ? !(p.fb1.ok && p.fb2.ok) : !p.fs.ok) return false;
-  const int E = window_scale<W, HI>(v);
-  if (E < 0) return false;
+  const int E = window_exponent<W, HI>(v);
+  if (!fx_usable(E)) {
+    int any = 0;  // sums of zeros are zero, as the chain's
+#pragma unroll
+    for (int t = W - H; t <= W + 3 + H; ++t) any |= fx_mag(v[t]) | fx_word(v[t], 0);
+    r[0] = r[1] = r[2] = r[3] = 0.0;
+    return any == 0;
+  }
   const int sh = KIND ? p.fb1.sw - p.fb2.sw - (E - 1023) - 1 : 0;
   if (KIND && (sh < 1 || sh > 200)) return false;
   Fx x[4 + 2 * HI];
 #pragma unroll
   for (int t = 0; t < 4 + 2 * HI; ++t) x[t] = fx_split(fx_from(v[W - HI + t], E));
+  if ((AB || KIND) && !values_enough(KIND ? p.fb2 : p.fs, x + HI)) return false;
   int64_t R[4];
   if (KIND) {
     int64_t R1[4];
@@ -373,7 +387,7 @@ __device__ __forceinline__ bool group_fixed(const StepParams &p, const double v[
 #pragma unroll
     for (int q = 0; q < 4; ++q) r[q] = fx_to_any(R[q], ex);
   } else {
-    fx_results<4>(R, ex, r);
+    if (fx_results_wide<4>(R, ex, r) < kFxLeast) return false;
     if (HI < H) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) r[q] = fma(p.s[0][0], v[q + W - H], r[q]);

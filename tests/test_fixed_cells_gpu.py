@@ -169,3 +169,71 @@ def test_the_diffusivity_gradient_of_a_field_that_is_small_where_the_seed_is_not
     n = 1 + 3 * spec["order"]
     bar = (2 * n + 7 + 512) * np.longdouble(2.0) ** -53 * (np.abs(lam) * m).sum() * sum(np.abs(t).sum() for t in q)
     assert abs(np.longdouble(ga) - (lam * f).sum()) <= bar
+
+
+LINES = [
+    ("block_o2", 8192, 2, 4, {}),
+    ("block_o4", 8200, 4, 4, {}),
+    ("block_o6", 8192, 6, 4, dict(r_alpha=0.02)),
+    ("block_o4_k3", 8192, 4, 3, {}),
+    ("block_o4_wide_tiles", 655364, 4, 4, {}),
+    ("block_o4_odd", 8193, 4, 4, {}),
+    ("block_o4_small_taps", 8192, 4, 4, dict(r_alpha=1e-6, c=0.0)),
+    ("single_o2", 8192, 2, 1, {}),
+    ("single_o4", 8192, 4, 1, {}),
+    ("single_o6", 8192, 6, 1, dict(r_alpha=0.02)),
+    ("single_o2_small_taps", 8192, 2, 1, dict(r_alpha=1e-6, c=0.0)),
+    ("single_o4_ragged", 200001, 4, 1, {}),
+    ("ab2_o4", 8192, 4, 1, dict(tsteps=2, r_alpha=0.02)),
+    ("ab3_o6", 8192, 6, 1, dict(tsteps=3, r_alpha=0.01)),
+    ("ab2_o2_ragged", 200001, 2, 1, dict(tsteps=2, r_alpha=0.02)),
+]
+
+
+@pytest.mark.parametrize("kind", ["ones", "noise", "spikes_1e6", "spikes_1e14", "steep", "half_zero", "waves"])
+@pytest.mark.parametrize("name,n,order,K,kw", LINES, ids=[c[0] for c in LINES])
+def test_a_1d_step_or_block_cell_by_cell(name, n, order, K, kw, kind):
+    """Each cell of one step, or one block of K, to what the chain of its m taps may be off: 2^-53 of sum |w v| over its own
+    stencil (Adams-Bashforth: and of its value) for each rounding, m more for the weights, and four for the fixed point."""
+    from paper_1702_00496_gb300 import Solver, at_set_fusion
+    spec = W.wl_1d(n, 1, order, 4, 0, 921, (1, 2), **kw)[0]
+    rng = np.random.default_rng([921, len(name), len(kind)])
+    u = rng.uniform(0.5, 1.0, n)
+    x = np.arange(n)
+    if kind == "ones":
+        u = np.ones(n)
+    elif kind == "noise":
+        u = rng.standard_normal(n)
+    elif kind.startswith("spikes"):
+        u = np.where(rng.random(n) < 0.01, u * float(kind[7:]), u)
+    elif kind == "steep":
+        u = u * np.exp(-((x % 257) - 100.0) ** 2 / 200.0)
+    elif kind == "half_zero":
+        u = np.where(x > n // 3, u, 0.0)
+    elif kind == "waves":
+        u = np.sin(2 * np.pi * x / 97.0)
+    s = Solver(spec)
+    assert at_set_fusion(s.h, K) == K
+    s.reset(torch.as_tensor(u, device="cuda"))
+    s.step(K)
+    s.sync()
+    got = s.field().cpu().numpy().copy()
+    s.close()
+    f = _taps(spec)[0]
+    one = f.copy()
+    one[order // 2] += 1
+    w = np.array([1], dtype=np.longdouble)
+    for _ in range(K):
+        w = np.convolve(w, one)
+    v, h, m = u.astype(np.longdouble), len(w) // 2, len(w)
+    want, size = np.zeros_like(v), np.zeros_like(v)
+    for j in range(-h, h + 1):
+        t = w[j + h] * np.roll(v, -j)
+        want += t
+        size += np.abs(t)
+    if spec["tsteps"] > 1:  # dt f is added to the value
+        size = np.abs(v) + sum(np.abs(f[j + order // 2] * np.roll(v, -j)) for j in range(-(order // 2), order // 2 + 1))
+    bar = (2 * m + 4) * np.longdouble(2.0) ** -53 * size
+    off = np.abs(got.astype(np.longdouble) - want)
+    worst = int(np.argmax(off - bar))
+    assert (off <= bar).all(), (worst, got[worst], float(want[worst]), float(off[worst] / bar[worst]) if bar[worst] else "")
