@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
       list = mine && (far || !usable);
       uint32_t who = __ballot_sync(0xffffffffu, list);
       if (who != 0) {
-        int top = usable ? 0 : 1;  // sums of zeros are zero
+        int top = usable ? 0 : 1;  // sums of zeros are zero (a plane that is not usable has no top either)
 #pragma unroll
         for (int q = o - H; q <= o + H; ++q) top |= planes.top[q & 7];
         if (top == 0) {
@@ -530,10 +530,13 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
     }
     if (i < ze + H) {
       in.extrapolate(p, T, sn, i);
-      int mag = 0;
+      int mag = 0, low = 0;
 #pragma unroll
-      for (int s = 0; s < kBrickSlots; ++s) mag = max(mag, fx_mag(in.v[s]));
-      mag = __reduce_max_sync(0xffffffffu, mag);
+      for (int s = 0; s < kBrickSlots; ++s) {
+        mag = max(mag, fx_mag(in.v[s]));
+        low |= fx_word(in.v[s], 0);
+      }
+      mag = __reduce_max_sync(0xffffffffu, max(mag, low != 0 ? 1 : 0));
       if ((tid & 31) == 0) atomicMax(&mx[m3], mag);
     }
     const int count = __syncthreads_count(list);

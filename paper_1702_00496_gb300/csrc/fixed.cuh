@@ -211,8 +211,9 @@ struct FxPlanes {          // of the last eight planes: plane i at i mod 8, writ
 };
 constexpr int kFxNever = 1 << 20;  // cut of a plane that is not usable
 
-// Is a plane whose largest magnitude (fx_mag) is mag summed in fixed point?
-AT_FX_HD bool fx_plane_usable(int mag) { return (mag >> 20) == 0 || fx_usable(mag >> 20); }
+// Is a plane whose largest magnitude (fx_mag; 1 where that is 0 but the values are not) is mag summed in fixed point?  Zeros
+// are; denormal numbers are not zeros.
+AT_FX_HD bool fx_plane_usable(int mag) { return mag == 0 || fx_usable(mag >> 20); }
 
 // Plane i joins; m: exponent of its largest value (0 as above), usable: fx_plane_usable; reach: planes on either side that
 // an output reads, so the 2 reach + 1 planes before i are still in use.  Returns by how much the scale rose: entries go down

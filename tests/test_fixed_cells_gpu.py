@@ -237,3 +237,29 @@ def test_a_1d_step_or_block_cell_by_cell(name, n, order, K, kw, kind):
     off = np.abs(got.astype(np.longdouble) - want)
     worst = int(np.argmax(off - bar))
     assert (off <= bar).all(), (worst, got[worst], float(want[worst]), float(off[worst] / bar[worst]) if bar[worst] else "")
+
+
+@pytest.mark.parametrize("size", [1e-305, 1e-310, 1e-321])
+@pytest.mark.parametrize("name,make", TILES, ids=[t[0] for t in TILES])
+def test_a_tiled_step_and_its_transpose_of_denormal_numbers(name, make, size):
+    """Fields whose largest value is denormal, or holds no bit of its upper word, are not zero.  As a chain each of the taps'
+    roundings is at most half the smallest number there is, or 2^-53 of the values where those are larger."""
+    from paper_1702_00496_gb300 import Solver
+    spec = make()
+    shape = tuple(spec["n"][::-1])
+    u0 = _field(shape, "noise", 1.0, 3) * size
+    s = Solver(spec)
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.step(1)
+    s.sync()
+    got = s.field().cpu().numpy().copy()
+    s.reset(torch.as_tensor(u0, device="cuda"))
+    s.adjoint_forward(1, 1)
+    g, _ = s.adjoint_backward(torch.as_tensor(u0, device="cuda"), False)
+    g = g.cpu().numpy()
+    s.close()
+    n, u = 1 + 3 * spec["order"], u0.astype(np.longdouble)
+    for out, reverse in ((got, False), (g, True)):
+        f, m = _apply(u, _taps(spec), reverse)
+        bar = (n + 2) * np.longdouble(2.0) ** -1075 + (2 * n + 7) * np.longdouble(2.0) ** -53 * 2 * m
+        assert (np.abs(out.astype(np.longdouble) - (u + f)) <= bar).all()
