@@ -484,7 +484,7 @@ extern "C" int at_ensemble_create(const at_config_t *members, const at_member_t 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t dyn_smem = (size_t)(2 * max_nb + 15) / 16 * 16;
   if (dyn_smem > 48 * 1024) {
-    delete e;
+    cudaFree(e->scratch); delete e;
     return fail(AT_ERR_ARG, "at_ensemble_create: a member has too many PE sides");
   }
   e->dyn_smem = dyn_smem;
@@ -503,10 +503,19 @@ extern "C" int at_ensemble_create(const at_config_t *members, const at_member_t 
     kernel = hmax <= 2 ? (any_ab ? ensemble_kernel<2, true, true> : ensemble_kernel<2, false, true>)
                        : (any_ab ? ensemble_kernel<3, true, true> : ensemble_kernel<3, false, true>);
   }
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, threads, dyn_smem);
+  // the delays lie beside the member's parameters: together they may pass the 48 KB that need no leave
+  cudaFuncAttributes attr;
+  err = cudaFuncGetAttributes(&attr, kernel);
+  if (err == cudaSuccess && attr.sharedSizeBytes + dyn_smem > 48 * 1024)
+    err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem);
+  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, threads, dyn_smem);
+  if (err != cudaSuccess || fit < 1) {
+    cudaFree(e->scratch); delete e;
+    return err != cudaSuccess ? cuda_fail(err, "at_ensemble_create: kernel")
+                              : fail(AT_ERR_ARG, "at_ensemble_create: no SM holds a CTA of this shape");
+  }
   if (ctas_per_sm <= 0) ctas_per_sm = fit;
   if (ctas_per_sm > fit) ctas_per_sm = fit;
-  if (ctas_per_sm < 1) ctas_per_sm = 1;
   e->blocks = sms * ctas_per_sm;
   if (e->blocks > count) e->blocks = count;
   // capture: counter reset, persistent kernel, summary
@@ -523,7 +532,9 @@ extern "C" int at_ensemble_create(const at_config_t *members, const at_member_t 
     twin_diff_kernel<<<count, 256, 0, cap>>>(e->d_members, e->d_member_diff);
     summary_kernel<<<1, 128, 0, cap>>>(e->d_member_stats, e->d_member_diff, e->d_members, count, e->ngroups,
                                        e->d_summary);
+    const cudaError_t launched = cudaGetLastError();
     err = cudaStreamEndCapture(cap, &e->graph);
+    if (launched != cudaSuccess) err = launched;
   }
   if (err == cudaSuccess) err = cudaGraphInstantiate(&e->exec, e->graph, 0);
   cudaStreamDestroy(cap);
