@@ -165,16 +165,7 @@ __global__ void __launch_bounds__(1024, 1) ensemble_kernel(const MemberParams *_
     double acc[kStatFields];
 #pragma unroll
     for (int f = 0; f < kStatFields; ++f) acc[f] = 0.0;
-    // u_a goes through the ring slot after the final level's (its levels are not read any more)
-    double *sol = m.p.ring + (m.steps + 1) % m.p.R * m.p.ntot;
-    if (m.mt.on) {
-      member_field(m, m.ms_fin, m.amp_final, m.shift_final, sol);
-      __syncthreads();
-    }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const double ua = m.mt.on ? sol[i] : wave_1d(m, m.ms_fin, m.amp_final, m.shift_final, i);
-      const int pos = i % m.p.S[0];
-      const bool inB = m.p.use_pe[0] && (pos < m.p.h || pos >= m.p.S[0] - m.p.h);
+    auto point = [&](int i, double ua, bool inB) {
       const double e = u[i] - ua;
       acc[0] += e * e;
       acc[1] = fmax(acc[1], fabs(e));
@@ -183,6 +174,23 @@ __global__ void __launch_bounds__(1024, 1) ensemble_kernel(const MemberParams *_
       if (inB) { acc[5] += e * e; acc[8] += 1.0; } else { acc[4] += e * e; acc[7] += 1.0; }
       acc[6] += ua * ua;
       if (e != e) acc[1] = e;
+    };
+    if (m.mt.on) {  // in runs, as member_field; the ring keeps its levels
+      for (int c = threadIdx.x; c < (N + 15) >> 4; c += blockDim.x) {
+        double v[16];
+        atfd::mode_run(m.ms_fin, m.mt, m.nmodes, (double)(16 * (int64_t)c + 8) * m.xpi, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int i = 16 * c + j, pos = i % m.p.S[0];
+          if (i < N) point(i, v[j], m.p.use_pe[0] && (pos < m.p.h || pos >= m.p.S[0] - m.p.h));
+        }
+      }
+    } else {
+      for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const int pos = i % m.p.S[0];
+        point(i, wave_1d(m, m.ms_fin, m.amp_final, m.shift_final, i),
+              m.p.use_pe[0] && (pos < m.p.h || pos >= m.p.S[0] - m.p.h));
+      }
     }
     // warp partials by shuffles, then warp 0 combines them in warp order (deterministic)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;

@@ -1,4 +1,4 @@
-"""Members with as many PE sides as the ensemble's shared memory takes: the delays of all sides, two buffers of a byte each,
+"""What an ensemble leaves in the caller's memory, and members with as many PE sides as its shared memory takes: the delays of all sides, two buffers of a byte each,
 lie beside the member's parameters.  The fields are those of single steps of the same problem, bit for bit."""
 import pytest
 
@@ -35,3 +35,23 @@ def test_more_sides_than_that_are_refused():
     from paper_1702_00496_gb300 import Ensemble
     with pytest.raises(Exception, match="too many PE sides"):
         Ensemble([_spec(12292)], 20)
+
+
+@pytest.mark.parametrize("n", [64, 4096, 6000])
+def test_the_ring_keeps_every_level_that_a_single_run_keeps(n):
+    """Level m lies in slot m mod (L + T) after the run too, the oldest one included: as after single steps, bit for bit."""
+    from paper_1702_00496_gb300 import Ensemble, Solver, at_set_fusion
+    specs = [W.wl_1d(n, n // 8, 2, 3, 0, 941 + r, (1, 2))[0] for r in range(2)]
+    e = Ensemble(specs, 17)
+    e.run()
+    torch.cuda.synchronize()
+    at = 0
+    for spec in specs:
+        s = Solver(spec)
+        at_set_fusion(s.h, 1)
+        s.step(17)
+        s.sync()
+        assert torch.equal(e.ring[at:at + s.ring.numel()], s.ring)
+        at += s.ring.numel()
+        s.close()
+    e.close()
