@@ -191,10 +191,12 @@ int at_set_fusion(at_handle_t *hd, int32_t k, int32_t *k_used);
  * replays from step 0.  Enqueued on the handle's stream.  Errors: AT_ERR_ARG, AT_ERR_CUDA. */
 int at_reset(at_handle_t *hd, const double *u0_dev);
 
-/* Launch shape of the per-step kernel for the following at_step calls: threads per block (128, 256 or 512)
- * and a cap of blocks_per_sm (1..64) blocks per SM on its grid-stride loop.  Defaults 256 and 32
- * (1D problems in aligned groups of four: blocks of 128 in whole waves, at most 40 per SM).  Waits for the stream and
- * drops the captured step graph.  Used by the autotuner.  Errors: AT_ERR_ARG. */
+/* Launch shape of the grouped and per-point kernels for the following at_step calls: threads per block (128, 256 or 512)
+ * and a cap of blocks_per_sm (1..64) blocks per SM on their grid-stride loops.  Defaults 256 and 32; 128 and 40 for 1D
+ * problems in aligned groups of four, where blocks of 128 come in whole waves of eight per SM (also when they are set
+ * here).  Blocks of K steps take 128 or 256 threads and the cap.  The 3D tiles, the kernel of large 1D shapes without
+ * aligned groups and the one-launch kernel of small 1D problems have a shape of their own, which this does not change.
+ * Waits for the stream and drops the captured step graph.  Used by the autotuner.  Errors: AT_ERR_ARG. */
 int at_set_launch(at_handle_t *hd, int32_t threads, int32_t blocks_per_sm);
 
 /* Wait for the handle's stream.  Returns AT_OK, or AT_ERR_CUDA with the runtime's message when the stream reports

@@ -16,7 +16,8 @@ import torch
 from . import binding as B
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_lib", "autotune.json")
-FORWARD_CANDIDATES = [(t, b) for t in (128, 256, 512) for b in (4, 8, 16, 32)]
+# (128, 40) and (256, 32) are what the kernels take by default (1D groups; the others)
+FORWARD_CANDIDATES = [(128, 40)] + [(t, b) for t in (128, 256, 512) for b in (4, 8, 16, 32)]
 ENSEMBLE_CANDIDATES = [(1024, 1), (512, 2), (512, 1), (256, 4), (256, 2)]
 
 

@@ -488,7 +488,7 @@ cudaError_t launch_forward_step(const StepParams &p, int64_t n, const int64_t *n
   // 1D groups: blocks of 128, eight resident per SM, in whole waves -- a last wave of few blocks costs as much as a full
   // one, a second group per thread much less.  Per step, blocks of 256 capped at 32 per SM -> this: 2^22 points AB3 order 6
   // 48.5 -> 37.7 us, Burgers AB2 order 4 43.5 -> 35.8; 2^24 points AB2 103.6 -> 100.0; 2^20 points AB2 12.0 -> 10.1.
-  if (own && blocks > 8 * sms) blocks -= blocks % (8 * sms);
+  if (p.dim == 1 && grouped && threads == 128 && blocks > 8 * sms) blocks -= blocks % (8 * sms);
   // a launch inside a captured graph (n_base set) runs only at steps at or after ab_steady
   const bool ab = p.ts > 1, steady = p.ts == 2 && (n_base != nullptr || n >= p.ab_steady);
   if (p.dim == 1) {
@@ -527,7 +527,7 @@ void launch_block_typed(const StepParams &p, int max_blocks, int threads, int64_
   // and fill tiles of 128; instructions per tile: C + 1 conversions and C outputs.
   const int64_t t8 = block_tiles(p, 8), t4 = block_tiles(p, 4);
   const int taps = 3 * (2 * H * K + 1) + 22;
-  if (t8 >= 152 * 16 && t8 * (9 * 11 + 8 * taps) <= t4 * (5 * 11 + 4 * (taps + 8)))
+  if (t8 >= sm_count() * 16 && t8 * (9 * 11 + 8 * taps) <= t4 * (5 * 11 + 4 * (taps + 8)))
     launch_block_tiles<H, K, 8>(p, max_blocks, t8, threads, n_off, n_base, st);
   else
     launch_block_tiles<H, K, 4>(p, max_blocks, t4, threads, n_off, n_base, st);
