@@ -796,13 +796,18 @@ bool brick_shape(const StepParams &p, BrickShape *b) {
   if (b->plane >= 65536 || p.S[2] > 32767) return false;
   // Planes per chunk, and whether to take this kernel at all.  A block's iteration (one plane) takes kIter whether one or
   // four blocks share the SM -- it is a chain of shared-memory round trips, conversions and a barrier -- so a launch
-  // takes as many of them as it has waves times planes, 2 h + 2 of which only fill the ring (512^3 in 8^3 PEs: 6.7 waves
-  // of 70 planes, 1.43 ms at order 4; 256^3 in 8^3 PEs at order 6, where every tile meets three faces with T = 4 levels
-  // each, 6 us per plane).  The grouped kernel (or the
-  // per-point one, for shapes without groups of four) does one FP64 operation per tap and 8 % more for the halo, at 1.6
-  // (1.0) lanes per SM and clock.
+  // takes as many of them as it has waves times planes, 2 h + 2 of which only fill the ring, and 5 us for the launch after
+  // it.  At order 6 tiles that meet three faces, with T = 4 levels each, take 6 us per plane.  The grouped kernel (or the
+  // per-point one, for shapes without groups of four) does one FP64 operation per tap and 17 % more for the halo, at 1.6
+  // (1.0) lanes per SM and clock; Adams-Bashforth costs it 1.8 (1.4) times that and more, a tile's iteration 1.4 times.
+  // us per step, tiles against groups or points, where the line lies: order 2, 128^3 in 2^3 PEs 37 against 35, 192 x 192 x 64
+  // in 4 x 4 x 1 43 against 38, 150 x 126 x 90 in 3 x 3 x 2 (points) 43 against 43, 160^3 in 2^3 60 against 62, 200 x 168 x 140
+  // in 4^3 (points) 85 against 115; order 4, 128^3 51 against 69, 100^3 in 5^3 43 in groups; order 2 with AB2, 128^3 50
+  // against 65, 192 x 192 x 64 63 against 92.
+  const bool grouped = p.n[0] % 4 == 0 && p.S[0] % 4 == 0, multi = p.ts > 1;
   const bool narrow = p.h == 3 && ((p.use_pe[0] && p.S[0] < 40) || (p.use_pe[1] && p.S[1] < 40));
-  const double kIter[4] = {0.0, 2.1e-6, 3.1e-6, narrow ? 6e-6 : 3.0e-6}, clock = 2.07e9;
+  const double kIter[4] = {0.0, 2.7e-6, 3.4e-6, narrow ? 6e-6 : 3.0e-6}, clock = 2.07e9;
+  const double iteration = kIter[p.h] * (multi ? 1.4 : 1.0), chains = !multi ? 1.0 : (grouped ? 1.8 : 1.4);
   const int sms = brick_sms(), bytes = (2 * p.h + 2) * b->plane * 8 + 4096;
   int resident = 227 * 1024 / bytes;
   if (resident > kBrickBlocks) resident = kBrickBlocks;
@@ -813,7 +818,7 @@ bool brick_shape(const StepParams &p, BrickShape *b) {
     const int zc = (p.S[2] + chunks - 1) / chunks;
     const double fill = (double)(columns * ((p.S[2] + zc - 1) / zc)) / (sms * resident);
     const double waves = fill <= 3.0 ? std::ceil(fill) : fill + 0.5;
-    const double t = waves * (zc + 2 * p.h + 2) * kIter[p.h];
+    const double t = waves * (zc + 2 * p.h + 2) * iteration;
     if (least == 0.0 || t < least) {
       least = t;
       b->zc = zc;
@@ -821,8 +826,7 @@ bool brick_shape(const StepParams &p, BrickShape *b) {
   }
   b->chunks = (p.S[2] + b->zc - 1) / b->zc;
   b->blocks = columns * b->chunks;
-  const bool grouped = p.n[0] % 4 == 0 && p.S[0] % 4 == 0;
-  if (least > 0.95 * (double)p.ntot * (1 + 6 * p.h) * 1.08 / ((grouped ? 1.6 : 1.0) * sms * clock)) return false;
+  if (5e-6 + least > 0.9 * chains * (double)p.ntot * (1 + 6 * p.h) * 1.17 / ((grouped ? 1.6 : 1.0) * sms * clock)) return false;
   b->aligned = p.n[0] % 4 == 0 && p.S[0] % 4 == 0 && reinterpret_cast<uintptr_t>(p.ring) % 16 == 0;
   return b->blocks * b->zc * kBrickWarps < (1ll << 31);
 }

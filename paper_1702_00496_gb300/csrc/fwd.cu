@@ -41,8 +41,10 @@ using namespace atfd;
 //
 // 1D groups are summed in fixed point (stencil.cuh); two blocks of 512 per SM (64 registers) hide the latency of their
 // integer chains: at N = 2^24 the AB2 step of order 4 takes 105 us against 133 us with the 88 registers it would use.
+// The chains of 3D groups want the same but with Adams-Bashforth (160^3 in 8^3 PEs, order 2: 70.3 against 74.5 us with the 76
+// registers they would use).
 template <int DIM, int H, int AB, int KIND>
-__global__ void __launch_bounds__(512, DIM == 1 ? 2 : 1) forward_group_kernel(const StepParams p, const int64_t n_off,
+__global__ void __launch_bounds__(512, DIM == 1 || !AB ? 2 : 1) forward_group_kernel(const StepParams p, const int64_t n_off,
                                                             const int64_t *n_base) {
   const int64_t n = n_off + (n_base ? *n_base : 0);
   const int sn = (int)slot_of(n, p.R);
