@@ -275,6 +275,10 @@ extern "C" int at_init(const at_config_t *cfg, double *ring_dev, int64_t ring_le
     }
   }
 
+  if (w.dim == 1) {
+    fill_modes(&w.ms[0], w.amp[0], w.phase[0], w.kappa[0], w.nmodes, w.alpha, w.c[0], 0.0);
+    fill_mode_table(&w.mt, w.ms[0], w.nmodes, w.n[0]);
+  }
   const size_t n_tables = (size_t)(cfg->n[0] + cfg->n[1] + cfg->n[2]);
   const size_t keff_bytes = (size_t)(2 * p.nb + 255) / 256 * 256;
   // 3D grouped shapes: visit interior groups first (every cell and stencil neighbour inside the group's PE and the

@@ -54,12 +54,19 @@ __device__ __forceinline__ double mode_sum(const ModeSet &ms, int nmodes, double
 // both sums shared by the pair: 16 FMAs per mode and run instead of a sincospi, two recurrences and two FMAs per mode
 // for every point (2^24 points, 10 modes: 17 FP64 operations per point instead of about 70).  The cosines and sines of
 // the offsets come from the host; an error there or in P, Q enters each point once.
-__device__ __forceinline__ void mode_run(const ModeSet &ms, const ModeTable &mt, int nmodes, double xpi, double out[16]) {
+//
+// G threads share a run: thread `part` of them has the pairs j = part + G i (i < 8 / G; points 7 - j and 9 + j of the run, E - O
+// and E + O), and s0, the ninth point, is every thread's.  The operations of a point are the same for every G, so its bits are.
+// cs: the table's cosines and sines, cs[q][j] (G > 1: in shared memory, as the threads of a warp read different ones).
+template <int G>
+__device__ __forceinline__ void mode_pairs(const ModeSet &ms, const double (*cs)[8][2], int nmodes, double xpi, int part,
+                                           double E[8 / G], double O[8 / G], double &s0) {
   double sx, cx;
   sincospi(xpi, &sx, &cx);
-  double sk = sx, ck = cx, s0 = 0.0, E[8], O[8];
+  double sk = sx, ck = cx;
+  s0 = 0.0;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) E[j] = O[j] = 0.0;
+  for (int j = 0; j < 8 / G; ++j) E[j] = O[j] = 0.0;
   const double tc = cx + cx;
   double sp = 0.0, cp = 1.0;  // sin, cos of (k-1)x
   int q = 0;
@@ -80,14 +87,19 @@ __device__ __forceinline__ void mode_run(const ModeSet &ms, const ModeTable &mt,
       const double P = fma(ms.as[q], ck, ms.ac[q] * sk), Q = fma(ms.ac[q], ck, -(ms.as[q] * sk));
       s0 += P;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        E[j] = fma(P, mt.cs[q][j][0], E[j]);
-        O[j] = fma(Q, mt.cs[q][j][1], O[j]);
+      for (int j = 0; j < 8 / G; ++j) {
+        E[j] = fma(P, cs[q][part + G * j][0], E[j]);
+        O[j] = fma(Q, cs[q][part + G * j][1], O[j]);
       }
       ++q;
     }
   }
-  out[8] = s0;
+}
+
+// All 16 points by one thread.
+__device__ __forceinline__ void mode_run(const ModeSet &ms, const ModeTable &mt, int nmodes, double xpi, double out[16]) {
+  double E[8], O[8];
+  mode_pairs<1>(ms, mt.cs, nmodes, xpi, 0, E, O, out[8]);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     out[7 - j] = E[j] - O[j];
