@@ -42,14 +42,15 @@ FP64_FMA_LANES_PER_SM = 2  # FP64 FMA lanes per SM per clock on GB300 (nominal)
 # DRAM bytes (read + write) per launch of the step kernel, one ncu capture of the current kernel source; None where no
 # capture of the current source exists.
 MEASURED_TRAFFIC = {
-    ("1d_n16m", "blocks of 4"): (141.0e6 + 98.0e6) / 4,  # per step
-    ("1d_n16m_case3", "forward_group_kernel<1,1,0>"): 135.4e6 + 88.5e6,
-    ("1d_n16m_case4", "forward_group_kernel<1,2,2>"): 271.7e6 + 215.1e6,
-    ("1d_n16m_case5", "forward_group_kernel<1,3,1>"): 410.1e6 + 224.8e6,
-    ("1d_n16m_case6", "forward_group_kernel<1,2,1>"): 271.8e6 + 217.0e6,
-    # 3D: captured at 256^3 (the same 64^3 PEs; a 512^3 ring is 5-6 GB), scaled to 512^3 by the 8x points
-    ("3d_512_o2", "brick_kernel<1,0,0>"): 8 * (253.0e6 + 107.4e6),
-    ("3d_512_o4", "brick_kernel<2,0,0>"): 8 * (339.9e6 + 115.0e6),
+    ("1d_n16m", "blocks of 4"): (140.9e6 + 93.5e6) / 4,  # per step
+    ("1d_n16m_case3", "forward_group_kernel<1,1,0>"): 135.3e6 + 89.2e6,
+    ("1d_n16m_case4", "forward_group_kernel<1,2,2>"): 271.7e6 + 216.6e6,
+    ("1d_n16m_case5", "forward_group_kernel<1,3,1>"): 407.5e6 + 228.1e6,
+    ("1d_n16m_case6", "forward_group_kernel<1,2,1>"): 271.7e6 + 219.7e6,
+    # 3D: captured at 256^3 (the same 64^3 PEs; a 512^3 ring is 5-6 GB), scaled to 512^3 by the 8x points; the march and the
+    # launch for the groups it lists
+    ("3d_512_o2", "brick_kernel<1,0,0>"): 8 * (240.7e6 + 104.8e6 + 5.9e6),
+    ("3d_512_o4", "brick_kernel<2,0,0>"): 8 * (314.9e6 + 111.5e6 + 11.5e6),
 }
 TRAFFIC_NOTES = {
     "3d_512_o2": "DRAM read + write per launch from ncu at 256^3 in 4^3 PEs of 64^3, scaled by points to 512^3",
@@ -196,6 +197,8 @@ def launches_per_run(spec, T: int, K: int = 1) -> int:
     G = 50 // K * K if K > 1 else 50
 
     def launches(steps):
+        if dim == 3:  # a step in tiles: the march and the groups it lists
+            return 2 * steps
         return steps // K + steps % K if K > 1 else steps
 
     chunks = T // G
@@ -340,7 +343,7 @@ def measure_dgemm(local: int, n: int = 8192, reps: int = 3):
 
 
 def roofline(flop_per_launch, bytes_per_launch, launch_ms, ops_per_launch, kernel, local, clocks, traffic=None,
-             dgemm=None):
+             dgemm=None, limit=None):
     """Roofline of one kernel.  The step kernels sum their stencils on the integer pipes (block fixed point), so the FP64
     pipe is no ceiling any more: `achieved` is the HBM rate of the algorithmic bytes against the measured copy rate, and
     beside it stands the rate of the algorithmic FP64 operations, as a multiple of what the FP64 pipe could do."""
@@ -352,12 +355,25 @@ def roofline(flop_per_launch, bytes_per_launch, launch_ms, ops_per_launch, kerne
     out = {"bound": "memory", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "traffic": traffic,
            "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
            "algorithmic_bytes_per_launch": bytes_per_launch, "kernel": kernel, "launch_ms": launch_ms,
-           "peak_source": "measured copy bandwidth", "limit_now": "issue of the integer and FP32 pipes",
+           "peak_source": "measured copy bandwidth", "limit_now": limit,
            "algorithmic_tflops": flops / 1e12, "fp64_pipe_tflops": peak / 1e12, "multiple_of_fp64_pipe": flops / peak,
            "fp64_operations_per_clk_sm": ops_per_launch / (launch_ms / 1e3) / sms / (mhz_run * 1e6)}
     if dgemm:
         out["dgemm_fp64_tflops"] = dgemm
     return out
+
+
+def step_limit(spec, kernel):
+    """What bounds a step kernel (profiles/fixed_point_kernels.md)."""
+    if kernel.startswith("brick"):
+        return "latency: a plane's chain of loads, barrier and shared-memory round trips at 16 warps per SM"
+    if kernel.startswith("small"):
+        return "latency: the step's dependent chain and barrier in one block"
+    if kernel.startswith("forward_block"):
+        return "issue of the integer and FP32 pipes"
+    if time_levels(spec) > 1 and not spec.get("burgers"):
+        return "HBM and the issue of the integer and FP64 pipes together"
+    return "issue of the integer pipes"
 
 
 def _free():
@@ -491,7 +507,7 @@ def measure_forward(spec, T, args, local, warmup, steps, world=1, e2e=False, flu
         ops = (spec["order"] * kblock + 1) / kblock
         bytes_update = 16 / kblock
     out["roofline"] = roofline(flops_per_update(spec) * ntot, bytes_update * ntot, kern_ms,
-                                   ops * ntot, kname, local, clocks, traffic, dgemm)
+                                   ops * ntot, kname, local, clocks, traffic, dgemm, step_limit(spec, kname))
     if kblock > 1:
         out["roofline"]["traffic_note"] = "DRAM read + write per step (one launch per K steps, ncu)"
         out["roofline"]["note"] = ("algorithmic_tflops counts the single step's flop per update (1 multiply and 2 h FMAs); "
@@ -596,7 +612,7 @@ def measure_ensemble(args, local, specs, steps_list, T, groups_in, twins, warmup
            "one_at_a_time_clocks": one_clocks, "groups": groups, "clocks": clocks, "gpu_launches": steps * 4}
     if T is not None:
         rec["roofline"] = roofline(flop, 16 * updates, ms, 5 * updates, "ensemble_kernel (whole graph launch)", local,
-                                   clocks)
+                                   clocks, limit="latency: one barrier per step, 32 warps per SM with spills")
     return rec
 
 
@@ -782,7 +798,8 @@ def adjoint_record(args, local, T, warmup, steps) -> dict:
                            "u0_only_forward_ratio": rs["adjoint_u0_only_ms"] / f_ms, "clocks": rs["clocks"]}
         rec["roofline"] = roofline(ADJ_FLOP_PER_CELL * ntot, 8 * 8 * ntot, rs["backward_ms"] / T, 27 * ntot,
                                        "brick_kernel<2,0,2> + brick_kernel<2,0,1> + brick_faces_kernel<2> (a backward step with "
-                                       "the alpha term, every level resident)", local, rs["clocks"])
+                                       "the alpha term, every level resident)", local, rs["clocks"],
+                                       limit="latency: a plane's chain of loads, barrier and shared-memory round trips")
     else:
         rec["resident"] = {"skipped": f"needs {need / 1e9:.0f} GB free, {free / 1e9:.0f} GB free"}
         rec["roofline"] = None

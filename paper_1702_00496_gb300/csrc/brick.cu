@@ -11,8 +11,8 @@
 //    levels (FP64, as everywhere) once per tile when their plane is loaded, with that side's delay.
 //  - One scale serves the planes of the ring.  A plane whose largest value exceeds it, or a ring that has fallen two
 //    bits below it, rescales the ring (a shift of every entry: rare, fields change little from plane to plane).  Planes cut
-//    at a scale that has fallen since lack the digits between: their sums must be as much larger, and from kFxLift such
-//    bits on they are not used (fixed.cuh, FxRing).
+//    at a scale that has fallen since lack the digits between: their values must be as much larger, and beyond kFxLift such
+//    bits they are not used (fixed.cuh, FxRing).
 //  - One barrier per plane: iteration i sums output plane i-2-h from planes the ring already holds (while the loads of
 //    plane i are in flight), publishes plane i's largest value, and after the barrier stores plane i.
 //  - A thread sums four x-consecutive points.  A group with a half more than kBrickGuard bits below the scale (where the
@@ -24,9 +24,10 @@
 // small kernel for what the cells at the faces send to older levels.  256^3 in 4^3 PEs, order 4: 1.01 -> 0.63 ms per
 // backward step with the alpha term, 0.52 -> 0.37 ms without.
 //
-// What bounds it: the issue of the integer pipes (at order 4 39 multiply-adds per point, 22 instructions for 1.4
-// conversions, 25 for the rounding, the rest addresses and control) and the barrier.  512^3 in 8^3 PEs, L = 3 on GB300:
-// order 4 3.51 -> 1.43 ms per step, order 2 1.83 -> 0.96 ms; 256^3 in 4^3 PEs 453 -> 247 and 236 -> 160 us.
+// What bounds it: latency.  A block's plane is a chain of loads, the largest value, a barrier, conversions and shared-memory
+// round trips, and the ring leaves 16 warps per SM to hide it: issue 42 % active, the busiest pipe 39 %, DRAM 2.2 TB/s at
+// order 4.  512^3 in 8^3 PEs, L = 3 on GB300: order 4 3.51 -> 1.53 ms per step, order 2 1.83 -> 1.0 ms; 256^3 in 4^3 PEs 438 ->
+// 248 and 235 -> 175 us, the second launch (10 us) included.
 #include <cmath>
 
 #include "stencil.cuh"
@@ -585,8 +586,8 @@ __global__ void __launch_bounds__(kBrickThreads, kBrickBlocks) brick_kernel(cons
 // blocks have next to no L1 beside the ring and no registers to spare, a few of them hold most of a field's listed groups,
 // and past what they could list they held their barriers for the chains.  256^3 in 4^3 PEs, us per step (order 4 / 2; all
 // FP64 chains 438 / 235): a Gaussian of 13 cells 830 / 465 -> 637 / 372, a ball of ones in zeros 607 / 332 -> 228 / 149, noise
-// with spikes 832 / 457 -> 542 / 297; a field that is zero in half of the box 645 / 357 -> 287 / 198; smooth fields, with 0.5 %
-// of their groups listed, pay 10 us for it (226 -> 248, 160 -> 175).
+// with spikes 832 / 457 -> 542 / 297; a field that is zero in half of the box 645 / 357 -> 287 / 198; smooth fields, with 0.7 %
+// (0.5 %) of their groups listed, pay for it (226 -> 248, 160 -> 175).
 constexpr int kListThreads = 256;
 constexpr int kListWords = 512;  // 32 KB of list
 

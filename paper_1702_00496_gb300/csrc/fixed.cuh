@@ -1,17 +1,17 @@
 // fixed.cuh -- stencil sums in block fixed point: the contractions of the step kernels on the integer pipes.
 //
-// GB300 retires 2 FP64 FMAs per SM and clock but 62 multiply-adds of 32 x 32 + 64 bits (mad.wide.s32; measured 1.99 and
-// 62.5, and 63-126 for the logic, shift and add instructions around them), so a product of 62 by 60 bits in three of
-// them takes a tenth of the time of one DFMA.  The FP64 pipe bounds every step kernel at 9-20 % of the memory
-// bandwidth, and a stencil sum is a contraction of values of similar size with constant weights, so it needs no
-// exponent per term:
+// GB300 retires 2 FP64 FMAs per SM and clock (measured 1.99) but about 30 multiply-adds of 32 x 32 + 64 bits with a 64-bit
+// addend (and 60-126 of the logic, shift and add instructions around them), so a product of 62 by 60 bits in three of them
+// takes a fifth of the time of one DFMA.  As FP64 chains the pipe bounded every step kernel at 9-20 % of the memory
+// bandwidth, and a stencil sum is a contraction of values of similar size with constant weights, so it needs no exponent
+// per term:
 //
 //   values   X = floor(v 2^(61 - e)), e the largest exponent in the window (biased: E): |X| < 2^62, 8 bits below the
 //            last bit of the window's largest value.  X = hi 2^32 + lo, hi and lo signed.
 //   weights  W = round(w 2^sw), sw so that sum |W| <= 1.9 2^60 (prepared on the host).  W = w1 2^29 + w0, w0 signed.
 //   sum      A = sum w1 hi, B = sum w1 lo, C = sum w0 hi, in 64 bits each without overflow (|w1 hi| sums to under
-//            2^62, |w1 lo| to under 2^63, |w0 hi| to under 31 2^58 for up to 31 taps); w0 lo, under 2^-60 of the
-//            window's largest value for all taps together, is left out.
+//            2^62, |w1 lo| to under 2^63, |w0 hi| to under 31 2^58 for up to 31 taps); w0 lo, up to a
+//            quarter of a unit of R per tap, is left out.
 //            R = A + B 2^-32 + C 2^-29 = sum W X 2^-61, rounded once to the nearest FP64 value R 2^(E - 1023 - sw).
 //
 // R is off by a few units: at most one for the cut values and one for the joins, a quarter per tap for w0 lo and half of

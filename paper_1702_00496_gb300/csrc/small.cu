@@ -4,10 +4,10 @@
 // step as nodes of a captured graph.  Here one thread block keeps the whole problem for a run of steps: every thread
 // updates a group of four points with the step kernels' own group_step (the same bits), spare warps draw the next step's
 // delays meanwhile, and a barrier separates the steps.  What bounds it is latency: the barrier, the reads of the ring
-// through L1 and the step's dependent chain (1.35 us per step at order 2, 2.4 us at order 4).
+// through L1 and the step's dependent chain (256 points: 1.14 us per step at order 2, 2.2 us at order 4).
 //
-// Measured against the graph, per step at order 2 / 4: 256 points 3.8 / 5.1 -> 1.35 / 2.4 us, 2048 points in 32 PEs 3.1 / 5.4
-// -> 2.1 / 3.8 us.  Beyond one group per thread, and as a cluster of up to eight blocks with a cluster barrier between
+// Measured against the graph, per step at order 2 / 4: 256 points 3.8 / 5.1 -> 1.14 / 2.2 us, 2048 points in 32 PEs 3.1 / 5.4
+// -> 2.1 / 3.4 us.  Beyond one group per thread, and as a cluster of up to eight blocks with a cluster barrier between
 // steps (4096 points in 64 PEs: 3.1 / 5.4 -> 3.5 / 5.8 us; 16384: 2.8 / 4.3 -> 3.5 / 5.8 us), the graph is faster, and
 // blocks of K steps are where the PEs are wide enough for K >= 3 (131072 points: 1.2 / 1.5 us).
 #include "stencil.cuh"
